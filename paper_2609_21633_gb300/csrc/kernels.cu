@@ -58,15 +58,6 @@ inline unsigned nblk(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); 
 #ifndef TN_MINB_F32
 #define TN_MINB_F32 2
 #endif
-// Radial chunking: the grid is split radially until it has at least this many CTAs
-// (chunks never shorter than TN_KC_MIN cells).
-#ifndef TN_CTA_TARGET
-#define TN_CTA_TARGET (32 * 152)
-#endif
-// CTA target for wide (16 x 32) tiles, which run one CTA per SM; 0 disables wide tiles.
-#ifndef TN_CTA_TARGET_WIDE
-#define TN_CTA_TARGET_WIDE (16 * 152)
-#endif
 #ifndef TN_WIDE_TILES
 #define TN_WIDE_TILES 1
 #endif
@@ -83,21 +74,34 @@ inline unsigned nblk(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); 
 #ifndef TN_WIDE_MAXREG
 #define TN_WIDE_MAXREG 96
 #endif
-#ifndef TN_KC_MIN
-#define TN_KC_MIN 8
-#endif
 // 1: load node layer k+2 while cell layer k is computed
 #ifndef TN_PREFETCH
 #define TN_PREFETCH 0
 #endif
-// FP32 A apply on paired-cell tiles (pair32.cuh) where N >= 32 (0: the square tiles), and its CTA
-// target: radial chunks halve until the grid has this many CTAs (two resident per SM)
+// FP32 A apply on paired-cell tiles (pair32.cuh) where N >= 32 (0: the square tiles)
 #ifndef TN_PAIR32
 #define TN_PAIR32 1
 #endif
-#ifndef TN_PAIR_CTA_TARGET
-#define TN_PAIR_CTA_TARGET (16 * 152)
-#endif
+
+// Cell layers per radial chunk of a streaming tile kernel with `columns` tile columns and `resident`
+// CTAs per SM.  A CTA sweeps its chunk plus the cell layer below it (recomputed for the carried
+// contributions) and a prologue worth about half a layer, and the GPU runs the CTAs in
+// ceil(CTAs / (152 resident)) waves, so a launch takes waves * (kc + 1.5) layer times; the chunk
+// count that minimises it is taken.  Small grids get short chunks that fill the SMs (level 4 / 17
+// layers FP64: 80 CTAs of 2 layers instead of 20 of 8), large ones a last wave that is nearly full
+// (level 7 / 129 layers: 16 layers, the best of a sweep as well).
+inline int radial_chunk(int64_t columns, int ncells, int resident, int kmax) {
+  int best = 1;
+  double cost = 1e30;
+  for (int c = 1; c <= ncells; ++c) {
+    const int kc = (ncells + c - 1) / c;
+    if (kc > kmax) continue;
+    const int64_t ctas = columns * ((ncells + kc - 1) / kc), slots = (int64_t)152 * resident;
+    const double t = (double)((ctas + slots - 1) / slots) * (kc + 1.5);
+    if (t < cost) cost = t, best = kc;
+  }
+  return best;
+}
 template <typename T>
 struct MinBlocks {
   static constexpr int value = sizeof(T) == 8 ? TN_MINB_F64 : TN_MINB_F32;
@@ -1991,10 +1995,8 @@ cudaError_t launch_tile(const Level& L, BC bc, Op op, const T* const* in, T* con
   const int ti_ = L.N >= TILE ? TILE : L.N, tj_ = wide ? 2 * TILE : ti_;
   const int ntiles = (L.N / ti_) * (L.N / tj_);
   const int ncells = L.n_r - 1;
-  // radial chunks: enough CTAs to fill the GPU a few times over (wide tiles: one CTA per SM)
-  const int64_t target = wide ? TN_CTA_TARGET_WIDE : TN_CTA_TARGET;
-  int kc = ncells;
-  while (kc > TN_KC_MIN && (int64_t)ntiles * 10 * ((ncells + kc - 1) / kc) < target) kc = (kc + 1) / 2;
+  // FP64 (one FP64 pipe per SM, wide tiles one CTA): one CTA's layers at a time; FP32: two overlap
+  const int kc = radial_chunk((int64_t)ntiles * 10, ncells, sizeof(T) == 8 ? 1 : 2, ncells);
   dim3 grid(ntiles, (ncells + kc - 1) / kc, 10);
   const T* i1 = Op::NIN > 1 ? in[1] : in[0];
   const T* i2 = Op::NIN > 2 ? in[2] : in[0];
@@ -2619,9 +2621,7 @@ cudaError_t launch_pair32(const Level& L, BC bc, const OpA<float, HG>& op, const
   if (epi) E = *epi;
   const Dims D = dims(L);
   const int ntiles = (L.N / kPTI) * (L.N / kPTJ), ncells = L.n_r - 1;
-  int kc = ncells;
-  while (kc > kPMaxKc || (kc > TN_KC_MIN && (int64_t)ntiles * 10 * ((ncells + kc - 1) / kc) < TN_PAIR_CTA_TARGET))
-    kc = (kc + 1) / 2;
+  const int kc = radial_chunk((int64_t)ntiles * 10, ncells, 2, kPMaxKc);
   const dim3 grid(ntiles, (ncells + kc - 1) / kc, 10);
   const EtaView<float> ev = etav<float>(L);
   float4* const ring = reinterpret_cast<float4*>(L.ring64);  // 16 floats per 12 doubles of the FP64 layout
