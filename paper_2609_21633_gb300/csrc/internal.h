@@ -189,6 +189,36 @@ struct EpiArgs {
 template <typename T>
 cudaError_t launch_apply_A_epi(const Level& L, BC bc, int div_term, int epi, const T* const* in, const EpiArgs<T>& E,
                                T* const* t, cudaStream_t st, const int* skip = nullptr);
+// A apply of a coarse multigrid level (N <= 16) through a scratch array of the cells' contributions
+// (small.cuh), with one of the fused updates or (EPI_NONE) to y; `scratch` holds small_scratch_entries(L)
+// values and belongs to the caller: calls that share it must not overlap.
+inline bool small_level(const Level& L) { return L.N <= 16 && L.n_layout < ((int64_t)1 << 26); }
+inline int64_t small_scratch_entries(const Level& L) {
+  return small_level(L) ? (int64_t)24 * 10 * L.N * L.N * (L.n_r - 1) : 0;
+}
+template <typename T>
+cudaError_t launch_small_A(const Level& L, BC bc, int div_term, int epi, const T* const* in, const EpiArgs<T>& E,
+                           T* const* y, T* scratch, cudaStream_t st);
+
+// Coarsest-level block-Jacobi CG from x = 0 in one launch (small.cuh): until (r, D^-1 r) <= tol2 (r0, D^-1 r0)
+// or maxit steps; project: rigid rotations out of b and x (ginv: inverse rotation Gram matrix).  r, z, p: work
+// vectors of the level's layout.  One cluster of eight SMs: levels whose cells those carry faster than the
+// launches of a step cost (FP64: eight FP64 pipes, 4096 cells take about 35 us).
+template <typename T>
+struct CoarseCg {
+  T *x[3], *r[3], *z[3], *p[3];
+  const T* binv[6];
+  T* scratch;
+  double ginv[9], tol2;
+  int maxit, project;
+};
+template <typename T>
+inline bool coarse_cg_fits(const Level& L) {
+  return small_level(L) && L.n_layout <= 32768 && (sizeof(T) == 4 || 10 * (int64_t)L.N * L.N * (L.n_r - 1) <= 4096);
+}
+template <typename T>
+cudaError_t launch_coarse_cg(const Level& L, BC bc, int div_term, const T* const* b, const CoarseCg<T>& C,
+                             cudaStream_t st);
 template <typename T>
 cudaError_t launch_div_fine(const Level& L, BC bc, const T* const* u, T* q, cudaStream_t st);
 template <typename T>

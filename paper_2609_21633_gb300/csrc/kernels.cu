@@ -29,16 +29,17 @@
 #include <cstdio>
 #include <type_traits>
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "dfloat.cuh"
 #include "internal.h"
 
-// The file is compiled five times: TN_PART 1 holds everything but the A-apply launchers, TN_PART 2
+// The file is compiled six times: TN_PART 1 holds everything but the A-apply launchers, TN_PART 2
 // the FP64 and TN_PART 3 the FP32 A-apply launchers, TN_PART 4 and 5 those of the A apply with
 // the second radial quadrature point (their many tile-kernel instantiations then compile in
-// parallel); 0 = all.
+// parallel), TN_PART 6 the coarse multigrid levels' kernels (small.cuh); 0 = all.
 #ifndef TN_PART
 #define TN_PART 0
 #endif
@@ -2131,6 +2132,10 @@ __global__ void k_interface_epi(Dims D, int n_groups, const int* __restrict__ gp
   for (int q = b; q < e; ++q) epilogue<T, EPI>(E, x0, x1, x2, (int)(goff[q] + lo), v);
 }
 
+#if TN_PART == 0 || TN_PART == 6
+#include "small.cuh"
+#endif
+
 // ------------------------------------------------------------------------------------ diag(A)
 // Thread per layout node; gathers the 3x3 node block of A from the (up to) 12 wedges
 // around the node: A_jj = sum_e V eta (|g|^2 I + 1/3 g g^T) (the -2/3 div term gives
@@ -3152,5 +3157,75 @@ cudaError_t prepare_tile_kernels_q2() { return set_wide_attrs<OpA2<double>>(); }
 TN_INST_Q2(float)
 #endif
 #undef TN_INST_Q2
+
+// ------------------------------------------------------------ coarse multigrid levels (small.cuh)
+#if TN_PART == 0 || TN_PART == 6
+template <typename T, typename Op>
+cudaError_t small_A(const Level& L, BC bc, const Op& op, int epi, const T* const* in, const EpiArgs<T>& E, T* const* y,
+                    T* sc, cudaStream_t st) {
+  const SmallDims S = small_dims(L);
+  const SmallTab<T> B = small_tab<T>(L, bc);
+  k_small_cell<T, Op><<<nblk(S.ncell, kSmallBlock), kSmallBlock, 0, st>>>(S, B, op, in[0], in[1], in[2], sc);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const unsigned nb = nblk((int64_t)S.n_lat * S.n_r, 128);
+#define TN_SMALL_NODE(EP) k_small_node<T, EP><<<nb, 128, 0, st>>>(S, B, in[0], in[1], in[2], sc, y[0], y[1], y[2], E)
+  switch (epi) {
+    case EPI_NONE: TN_SMALL_NODE(EPI_NONE); break;
+    case EPI_RESID: TN_SMALL_NODE(EPI_RESID); break;
+    case EPI_CHEB1: TN_SMALL_NODE(EPI_CHEB1); break;
+    case EPI_CHEB2: TN_SMALL_NODE(EPI_CHEB2); break;
+    default: return cudaErrorInvalidValue;
+  }
+#undef TN_SMALL_NODE
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_small_A(const Level& L, BC bc, int div_term, int epi, const T* const* in, const EpiArgs<T>& E,
+                           T* const* y, T* sc, cudaStream_t st) {
+  if (!small_level(L)) return cudaErrorInvalidValue;
+  const T hgk = (T)hg_coef(L, div_term);
+  if (L.quad == 2) return small_A<T>(L, bc, OpA2<T>{div_term}, epi, in, E, y, sc, st);
+  if (L.hg_kappa > 0) return small_A<T>(L, bc, OpA<T, true>{div_term, hgk}, epi, in, E, y, sc, st);
+  return small_A<T>(L, bc, OpA<T, false>{div_term, hgk}, epi, in, E, y, sc, st);
+}
+
+template <typename T, typename Op>
+cudaError_t cg_cluster(const Level& L, BC bc, const Op& op, const CgArgs<T>& A, cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(kCgCtas), cfg.blockDim = dim3(kCgThreads), cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kCgCtas, at.val.clusterDim.y = 1, at.val.clusterDim.z = 1;
+  cfg.attrs = &at, cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_cg_cluster<T, Op>, small_dims(L), small_tab<T>(L, bc), op, A);
+}
+
+template <typename T>
+cudaError_t launch_coarse_cg(const Level& L, BC bc, int div_term, const T* const* b, const CoarseCg<T>& C,
+                             cudaStream_t st) {
+  if (!coarse_cg_fits<T>(L)) return cudaErrorInvalidValue;
+  CgArgs<T> A{};
+  A.b0 = b[0], A.b1 = b[1], A.b2 = b[2];
+  for (int c = 0; c < 3; ++c) A.x[c] = C.x[c], A.r[c] = C.r[c], A.z[c] = C.z[c], A.p[c] = C.p[c];
+  for (int q = 0; q < 6; ++q) A.binv[q] = C.binv[q];
+  A.rad = sizeof(T) == 8 ? (const T*)L.rad64 : (const T*)L.rad32;
+  A.sc = C.scratch, A.tol2 = C.tol2, A.maxit = C.maxit, A.project = C.project;
+  for (int q = 0; q < 9; ++q) A.ginv[q] = C.ginv[q];
+  const T hgk = (T)hg_coef(L, div_term);
+  if (L.quad == 2) return cg_cluster<T>(L, bc, OpA2<T>{div_term}, A, st);
+  if (L.hg_kappa > 0) return cg_cluster<T>(L, bc, OpA<T, true>{div_term, hgk}, A, st);
+  return cg_cluster<T>(L, bc, OpA<T, false>{div_term, hgk}, A, st);
+}
+
+#define TN_INST_SMALL(T)                                                                                          \
+  template cudaError_t launch_small_A<T>(const Level&, BC, int, int, const T* const*, const EpiArgs<T>&, T* const*, \
+                                         T*, cudaStream_t);                                                        \
+  template cudaError_t launch_coarse_cg<T>(const Level&, BC, int, const T* const*, const CoarseCg<T>&, cudaStream_t);
+TN_INST_SMALL(double)
+TN_INST_SMALL(float)
+#undef TN_INST_SMALL
+#endif
 
 }  // namespace tn

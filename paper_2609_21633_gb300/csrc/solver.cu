@@ -326,92 +326,6 @@ __global__ void k_cg_dir(int64_t n, const double* __restrict__ S, Ptr4<T> z, MPt
   const T be = (T)S[S_BETA];
   for (int c = 0; c < 3; ++c) p.c[c][i] = z.c[c][i] + be * p.c[c][i];
 }
-// Coarse CG on a small coarsest level (n <= SMALL_CG): one block runs the whole vector part of a
-// CG step, so a step is the operator apply plus one launch.  Sums over the masked (unique)
-// entries in FP64, in a fixed order (thread-strided partial sums, then a tree over the block).
-constexpr int SMALL_CG = 32768;
-constexpr int SB = 1024;  // threads of the single-block CG kernels
-
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();  // sh may still be read from a previous sum
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  double s = 0.0;
-  for (int w = 0; w < SB / 32; ++w) s += sh[w];  // every thread, same order
-  return s;
-}
-
-// r = b, z = D^-1 r, p = z, x = 0, rz0 = (r, z); flag = 0 unless rz0 = 0
-template <typename T>
-__global__ void __launch_bounds__(SB) k_cg_start_small(int64_t n, const uint8_t* __restrict__ mask, Ptr4<T> b,
-                                                       B6<T> binv, MPtr4<T> r, MPtr4<T> z, MPtr4<T> p, MPtr4<T> x,
-                                                       double* S, int* flag) {
-  __shared__ double sh[SB / 32];
-  double acc = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += SB) {
-    T rr[3] = {b.c[0][i], b.c[1][i], b.c[2][i]}, zz[3];
-    bmul(binv, i, rr, zz);
-    T d = (T)0;
-    for (int c = 0; c < 3; ++c) {
-      r.c[c][i] = rr[c], z.c[c][i] = zz[c], p.c[c][i] = zz[c], x.c[c][i] = (T)0;
-      d += rr[c] * zz[c];
-    }
-    if (mask[i]) acc += (double)d;
-  }
-  const double rz0 = block_sum(acc, sh);
-  if (threadIdx.x == 0) {
-    S[S_RZ0] = rz0, S[S_RZ] = rz0;
-    *flag = rz0 > 0.0 ? 0 : 1;
-  }
-}
-
-// one CG step after q = K p: alpha = (r, z) / (p, q); x += alpha p; r -= alpha q; z = D^-1 r;
-// beta = (r, z)_new / (r, z); p = z + beta p; flag once (r, z) <= tol2 (r0, z0) or at the last step
-template <typename T>
-__global__ void __launch_bounds__(SB) k_cg_step_small(int64_t n, const uint8_t* __restrict__ mask, MPtr4<T> p,
-                                                      Ptr4<T> q, B6<T> binv, MPtr4<T> x, MPtr4<T> r, MPtr4<T> z,
-                                                      double* S, int* flag, double tol2, int last) {
-  if (*flag) return;
-  __shared__ double sh[SB / 32];
-  double acc = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += SB) {
-    if (!mask[i]) continue;
-    T d = (T)0;
-    for (int c = 0; c < 3; ++c) d += p.c[c][i] * q.c[c][i];
-    acc += (double)d;
-  }
-  const double pq = block_sum(acc, sh);
-  const double rz = S[S_RZ];
-  const T al = (T)(rz / pq);
-  acc = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += SB) {
-    T rr[3], zz[3];
-    for (int c = 0; c < 3; ++c) {
-      x.c[c][i] += al * p.c[c][i];
-      rr[c] = r.c[c][i] - al * q.c[c][i];
-      r.c[c][i] = rr[c];
-    }
-    bmul(binv, i, rr, zz);
-    T d = (T)0;
-    for (int c = 0; c < 3; ++c) z.c[c][i] = zz[c], d += rr[c] * zz[c];
-    if (mask[i]) acc += (double)d;
-  }
-  const double rzn = block_sum(acc, sh);
-  const bool stop = !(rzn > tol2 * S[S_RZ0]) || last;
-  if (!stop) {
-    const T be = (T)(rzn / rz);
-    for (int64_t i = threadIdx.x; i < n; i += SB)
-      for (int c = 0; c < 3; ++c) p.c[c][i] = z.c[c][i] + be * p.c[c][i];
-  }
-  __syncthreads();  // every thread has read S[S_RZ] and S[S_RZ0]
-  if (threadIdx.x == 0) {
-    S[S_RZ] = rzn;
-    if (stop) *flag = 1;
-  }
-}
-
 __global__ void k_set_int(int* f, int v) { *f = v; }
 __global__ void k_cg_start(double* S, int* flag) {
   S[S_RZ] = S[S_RZ0];
@@ -511,6 +425,7 @@ struct PrecState {
   cudaGraphExec_t vgraph = nullptr;   // the V-cycle (level-0 b -> level-0 x) captured after set-up
   cudaGraph_t vtemplate = nullptr;    // its graph, kept for composing several systems' V-cycles
   T* tu[3] = {nullptr, nullptr, nullptr};  // velocity scratch (level 0)
+  T* cells = nullptr;                 // cell contributions of the coarse levels' applies (largest one)
 };
 
 struct MGState {
@@ -708,7 +623,22 @@ void project_rotations(MGState* m, const Level& L, T* const* u, cudaStream_t st,
 template <typename T>
 void apply_K_level(const tn_mesh* mesh, int h, const T* const* x, T* const* y, cudaStream_t st,
                    const int* skip = nullptr) {
-  ck(launch_apply_A<T>(*mesh->mg->geo[h], BC{mesh->bc_in, mesh->bc_out}, mesh->div_term, x, y, st, skip));
+  const Level& L = *mesh->mg->geo[h];
+  const BC bc{mesh->bc_in, mesh->bc_out};
+  if (!skip && small_level(L))
+    ck(launch_small_A<T>(L, bc, mesh->div_term, EPI_NONE, x, EpiArgs<T>{}, y, ps<T>(mesh->mg).cells, st));
+  else
+    ck(launch_apply_A<T>(L, bc, mesh->div_term, x, y, st, skip));
+}
+
+// K x of a multigrid level with a fused update (see EpiArgs): the coarse levels through the cells' scratch.
+template <typename T>
+void apply_K_epi(MGState* m, const tn_mesh* mesh, int h, int epi, const T* const* x, const EpiArgs<T>& E, T* const* t,
+                 cudaStream_t st) {
+  const Level& L = *m->geo[h];
+  const BC bc{mesh->bc_in, mesh->bc_out};
+  if (small_level(L)) ck(launch_small_A<T>(L, bc, mesh->div_term, epi, x, E, t, ps<T>(m).cells, st));
+  else ck(launch_apply_A_epi<T>(L, bc, mesh->div_term, epi, x, E, t, st));
 }
 
 // Block-Jacobi-preconditioned CG on the coarsest level: x = K^-1 b (x0 = 0); stops when
@@ -719,24 +649,18 @@ void coarse_cg(MGState* m, const tn_mesh* mesh, int h, cudaStream_t st) {
   const Level& L = *m->geo[h];
   const int64_t n = L.n_layout;
   const bool proj = rotations_singular(mesh);
-  if (proj) project_rotations<T>(m, L, C.b.mm(), st);
-  const double tol2s = m->opts.coarse_rtol * m->opts.coarse_rtol;
-  if (n <= SMALL_CG) {  // single-block vector kernels: two launches per CG step plus the apply
-    k_cg_start_small<T><<<1, SB, 0, st>>>(n, L.wmask, P4<T>(C.b.cc(), 3), C.bi(), M4<T>(C.r.mm(), 3),
-                                          M4<T>(C.d().mm(), 3), M4<T>(C.p.mm(), 3), M4<T>(C.x().mm(), 3), m->S,
-                                          m->flag);
-    ckl();
-    const int maxit = m->opts.coarse_max_iters;
-    for (int it = 0; it < maxit; ++it) {
-      apply_K_level<T>(mesh, h, C.p.cc(), C.t.mm(), st, m->flag);
-      k_cg_step_small<T><<<1, SB, 0, st>>>(n, L.wmask, M4<T>(C.p.mm(), 3), P4<T>(C.t.cc(), 3), C.bi(),
-                                           M4<T>(C.x().mm(), 3), M4<T>(C.r.mm(), 3), M4<T>(C.d().mm(), 3), m->S,
-                                           m->flag, tol2s, it == maxit - 1);
-      ckl();
-    }
-    if (proj) project_rotations<T>(m, L, C.x().mm(), st);
+  if (coarse_cg_fits<T>(L)) {  // one launch
+    CoarseCg<T> A{};
+    for (int c = 0; c < 3; ++c) A.x[c] = C.x().c[c], A.r[c] = C.r.c[c], A.z[c] = C.d().c[c], A.p[c] = C.p.c[c];
+    for (int q = 0; q < 6; ++q) A.binv[q] = C.binv[q];
+    A.scratch = ps<T>(m).cells;
+    const M33 g = inverse33(L.inertia);
+    for (int q = 0; q < 9; ++q) A.ginv[q] = g.a[q / 3][q % 3];
+    A.tol2 = m->opts.coarse_rtol * m->opts.coarse_rtol, A.maxit = m->opts.coarse_max_iters, A.project = proj;
+    ck(launch_coarse_cg<T>(L, BC{mesh->bc_in, mesh->bc_out}, mesh->div_term, C.b.cc(), A, st));
     return;
   }
+  if (proj) project_rotations<T>(m, L, C.b.mm(), st);
   // r = b, z = D^-1 r (stored in d), p = z, x = 0
   k_axpby<T><<<nb(n), EB, 0, st>>>(n, 3, 1.0, P4<T>(C.b.cc(), 3), 0.0, M4<T>(C.r.mm(), 3));
   ckl();
@@ -787,7 +711,6 @@ template <typename T>
 void cheb_step(MGState* m, const tn_mesh* mesh, int h, bool zero_x, cudaStream_t st) {
   MGLevelT<T>& G = ps<T>(m).L[h];
   const Level& L = *m->geo[h];
-  const BC bc{mesh->bc_in, mesh->bc_out};
   const int64_t n = L.n_layout;
   const double a = m->opts.cheb_lo * G.lam, b = m->opts.cheb_hi * G.lam;
   const double theta = 0.5 * (b + a), delta = 0.5 * (b - a), sigma = theta / delta;
@@ -800,14 +723,14 @@ void cheb_step(MGState* m, const tn_mesh* mesh, int h, bool zero_x, cudaStream_t
     EpiArgs<T> E = epi_of(G);
     E.c0 = 1.0 / theta;
     for (int c = 0; c < 3; ++c) E.dout[c] = G.d().c[c], E.xout[c] = G.xb[1 - G.xi].c[c];
-    ck(launch_apply_A_epi<T>(L, bc, mesh->div_term, EPI_CHEB1, G.x().cc(), E, G.t.mm(), st));
+    apply_K_epi<T>(m, mesh, h, EPI_CHEB1, G.x().cc(), E, G.t.mm(), st);
     G.xi = 1 - G.xi;
   }
   EpiArgs<T> E = epi_of(G);
   E.c1 = rho1 * rho0;
   E.c2 = 2.0 * rho1 / delta;
   for (int c = 0; c < 3; ++c) E.xacc[c] = G.x().c[c], E.xout[c] = G.x().c[c], E.dout[c] = G.db[1 - G.di].c[c];
-  ck(launch_apply_A_epi<T>(L, bc, mesh->div_term, EPI_CHEB2, G.d().cc(), E, G.t.mm(), st));
+  apply_K_epi<T>(m, mesh, h, EPI_CHEB2, G.d().cc(), E, G.t.mm(), st);
   G.di = 1 - G.di;
 }
 
@@ -833,7 +756,7 @@ void vcycle_level(MGState* m, const tn_mesh* mesh, int h, cudaStream_t st) {
   // r = b - K x (fused into the apply)
   {
     EpiArgs<T> E = epi_of(G);
-    ck(launch_apply_A_epi<T>(F, bc, mesh->div_term, EPI_RESID, G.x().cc(), E, G.t.mm(), st));
+    apply_K_epi<T>(m, mesh, h, EPI_RESID, G.x().cc(), E, G.t.mm(), st);
   }
   ck(launch_restrict<T>(F, Lc, bc, 3, 1, G.r.cc(), C.b.mm(), st));
   vcycle_level<T>(m, mesh, h + 1, st);
@@ -902,6 +825,9 @@ tn_status mg_setup_t(tn_mesh* mesh, const void* const* v0, cudaStream_t st) {
       for (int q = 0; q < 6; ++q) G.binv[q] = alloc_zero<T>(m, n);
       if (h == m->nlev - 1) G.p = alloc3<T>(m, n);
     }
+    int64_t cells = 0;
+    for (int h = 0; h < m->nlev; ++h) cells = std::max(cells, small_scratch_entries(*m->geo[h]));
+    if (cells > 0) P.cells = alloc_zero<T>(m, cells);
     P.mdiag = alloc_zero<T>(m, mesh->lv[1].n_layout);
     P.ones_p = alloc_zero<T>(m, mesh->lv[1].n_layout);
     P.sq = alloc_zero<T>(m, mesh->lv[1].n_layout);
