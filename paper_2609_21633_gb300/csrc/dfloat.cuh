@@ -15,14 +15,15 @@
 // contracts nor reorders it.
 //
 // Conversions from and to binary64 use integer operations only (no FP64 instruction):
-//   split: hi = the double truncated to 24 significand bits, lo = the next 23 bits (exact
-//   integer-to-float trick), then FastTwoSum to restore |lo| <= ulp(hi) / 2; relative error
-//   below 2^-46 (both parts are truncated).  Magnitudes below 2^-80 keep only hi, and values outside the FP32 exponent range
+//   split: hi = the double truncated to 24 significand bits, lo = the remaining 29 bits rounded to
+//   FP32 (exact integer-to-float tricks for 23 and 6 of them, one FMA), then FastTwoSum to restore
+//   |lo| <= ulp(hi) / 2; relative error at most 2^-48.  Magnitudes below 2^-80 keep only hi, and values outside the FP32 exponent range
 //   are not representable (the wedge operator's data are far inside both limits).
 //   join: hi and lo widened exactly to binary64 (bit manipulation) and added with one FP64 add,
 //   which is exact because hi + lo has at most 48 significant bits.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -161,8 +162,11 @@ TN_DF_HD dfl split(double x) {
   if (e < 1023 - 126) return dfl(df_float_of(sign), 0.0f);  // zero or below the FP32 normal range
   const uint32_t m23 = ((bh & 0xfffffu) << 3) | (bl >> 29);  // top 23 stored significand bits
   const float hi = df_float_of(sign | ((uint32_t)(e - 1023 + 127) << 23) | m23);
-  // the next 23 bits as an exact integer t (2^23 + t - 2^23), scaled by 2^(e - 1023 - 46)
-  const float t = TN_FSUB(df_float_of(0x4b000000u | ((bl >> 6) & 0x7fffffu)), 8388608.0f);
+  // the next 23 and the last 6 bits as exact integers (2^23 + n - 2^23), joined and rounded once, scaled by
+  // 2^(e - 1023 - 46)
+  const float t23 = TN_FSUB(df_float_of(0x4b000000u | ((bl >> 6) & 0x7fffffu)), 8388608.0f);
+  const float t6 = TN_FSUB(df_float_of(0x4b000000u | (bl & 0x3fu)), 8388608.0f);
+  const float t = TN_FFMA(t6, 0.015625f, t23);
   const int se = e - 1023 - 46 + 127;
   const float lo_mag = se >= 1 ? TN_FMUL(t, df_float_of((uint32_t)se << 23)) : 0.0f;
   const float lo = df_float_of(df_ubits_of(lo_mag) | sign);
@@ -194,6 +198,7 @@ TN_DF_HD double join(dfl a) { return widen(a.hi) + widen(a.lo); }
 struct df2 {
   float2 hi, lo;
 };
+__device__ __forceinline__ float2 p2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 p2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
 // a - b lane-wise, rounded to nearest: the packed subtraction of PTX (no intrinsic exists)
 __device__ __forceinline__ float2 p2sub(float2 a, float2 b) {
@@ -205,8 +210,10 @@ __device__ __forceinline__ float2 p2sub(float2 a, float2 b) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(rd));
   return d;
 }
-__device__ __forceinline__ float2 p2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 p2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// A rounded product, as a fused multiply-add with 0: nvcc 13.0 contracts a packed multiplication and an addition
+// of its result into one fused operation, also from PTX with explicit rounding (measured: the running sums
+// below then lose 1e-7 where s cancels most of x y).  Same cost; a product of -0 becomes +0.
+__device__ __forceinline__ float2 p2mul(float2 a, float2 b) { return p2fma(a, b, make_float2(0.f, 0.f)); }
 __device__ __forceinline__ float2 p2neg(float2 a) { return make_float2(-a.x, -a.y); }
 
 __device__ __forceinline__ df2 pack(dfl a, dfl b) { return df2{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)}; }
@@ -259,6 +266,59 @@ __device__ __forceinline__ df2 fma_nc2(const df2& x, const df2& y, const df2& w)
   fast_two_sum2(sh, p2add(sl, p2add(pl, w.lo)), zh, zl);
   return df2{zh, zl};
 }
+
+// Running sums of packed double-words, not renormalised between steps (acc2: value s + l, s the rounded sum
+// of the high parts, l everything below it).  A contraction of three products costs 24 packed
+// operations this way against 39 with a renormalised multiplication and two fma_nc2.  Errors: each
+// step rounds l, which stays a few u |terms|, so a step adds about u^2 |terms|; the products drop l l.  That
+// is the level at which the operands are rounded to double-words anyway (the accurate additions they
+// replace keep no more digits of such operands).
+//   acc_fma2 is TwoSum (Knuth, Moller) of s and the rounded product p; its second error term p - (s' - s) is
+//   formed by FMA from x y itself, so it holds the product's rounding too.  (With s' = fma(x, y, s), one
+//   operation less, TwoSum loses its exactness when s cancels most of x y: 1e-7 errors at single nodes.)
+struct acc2 {
+  float2 s, l;
+};
+__device__ __forceinline__ acc2 acc_of(const df2& x) { return acc2{x.hi, x.lo}; }
+__device__ __forceinline__ df2 df_of(const acc2& a) { return df2{a.s, a.l}; }
+__device__ __forceinline__ acc2 prod2(const df2& x, const df2& y) {
+  const float2 p = p2mul(x.hi, y.hi);
+  float2 l = p2fma(x.hi, y.hi, p2neg(p));
+  l = p2fma(x.hi, y.lo, l);
+  l = p2fma(x.lo, y.hi, l);
+  return acc2{p, l};
+}
+__device__ __forceinline__ void acc_fma2(acc2& a, const df2& x, const df2& y) {
+  const float2 s = p2add(a.s, p2mul(x.hi, y.hi));
+  const float2 nb = p2sub(a.s, s);                 // -(s - a.s)
+  const float2 ea = p2sub(a.s, p2add(s, nb));      // what a.s lost
+  const float2 eb = p2fma(x.hi, y.hi, nb);         // what x y lost, the rounding of the product included
+  float2 l = p2add(a.l, p2add(ea, eb));
+  l = p2fma(x.hi, y.lo, l);
+  a.l = p2fma(x.lo, y.hi, l);
+  a.s = s;
+}
+__device__ __forceinline__ void acc_add2(acc2& a, const df2& x) {
+  float2 s, e;
+  two_sum2(a.s, x.hi, s, e);
+  a.l = p2add(a.l, p2add(e, x.lo));
+  a.s = s;
+}
+__device__ __forceinline__ acc2 sum2(const df2& x, const df2& y) {
+  acc2 a = acc_of(x);
+  acc_add2(a, y);
+  return a;
+}
+__device__ __forceinline__ df2 neg2(const df2& x) { return df2{p2neg(x.hi), p2neg(x.lo)}; }
+__device__ __forceinline__ df2 diff2(const df2& x, const df2& y) { return df_of(sum2(x, neg2(y))); }
+__device__ __forceinline__ df2 dot3(const df2& x0, const df2& y0, const df2& x1, const df2& y1, const df2& x2,
+                                    const df2& y2) {
+  acc2 a = prod2(x0, y0);
+  acc_fma2(a, x1, y1);
+  acc_fma2(a, x2, y2);
+  return df_of(a);
+}
+__device__ __forceinline__ df2 both(const dfl& a) { return pack(a, a); }
 #endif
 
 }  // namespace tn

@@ -323,80 +323,6 @@ struct OpA {
   }
 };
 
-// Double-float viscous block without hourglass control: the arithmetic of OpA with the sums
-// split by whether their terms can cancel.  The corner differences (a_xi, a_eta of nearly equal
-// nodal sums) and every node-level accumulation (corner combinations, carried and exchanged
-// partials) use the accurate double-word addition; the contractions that form the strain, the
-// stress and H = S M^-T, whose terms carry no such cancellation, use the fused multiply-add and the
-// sum without the second TwoSum (add_nc / fma_nc).  The two wedges of the cell are the two lanes of
-// packed f32x2 double-floats (x = W0, y = W1; lane pairs of corners (00, 11), (10, 01), (01, 10),
-// as in OpA<float, false>), one issue slot per pair; lanes meet only where corners 10 and 01 and
-// the top-minus-bottom parts combine.
-template <>
-struct OpA<dfl, false> {
-  static constexpr int NIN = 3, NOUT = 3;
-  static constexpr bool USES_ETA = true, LOADS = true, NEEDS_D = true;
-  struct Col {
-    df2 M[9], dM;  // M^-1 entries and |det M| of (W0, W1)
-  };
-  int div_term;
-  dfl hgk;
-  __device__ __forceinline__ Col column(const dfl (&Mi)[2][9], const dfl (&dM)[2], int) const {
-    Col c;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) c.M[q] = pack(Mi[0][q], Mi[1][q]);
-    c.dM = pack(dM[0], dM[1]);
-    return c;
-  }
-  __device__ __forceinline__ void cell(const dfl (&s)[4][3], const dfl (&dd)[4][3], const dfl (&)[2][9],
-                                       const dfl (&)[2], const dfl* lc, const dfl (&eta)[2], dfl (&accb)[4][3],
-                                       dfl (&acct)[4][3], const Col& col) const {
-    const df2 r = pack(lc[4], lc[4]), vw2 = pack(lc[5], lc[5]);
-    const df2* M = col.M;
-    const df2 mr[3] = {mul2(r, M[6]), mul2(r, M[7]), mul2(r, M[8])};
-    df2 G[3][3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const df2 s0 = pack(s[0][c], s[3][c]), s1 = pack(s[1][c], s[2][c]), s2 = pack(s[2][c], s[1][c]);
-      const df2 ax = sub2(s1, s0), ay = sub2(s2, s0);
-      const df2 az = add_nc2(add_nc2(pack(dd[0][c], dd[3][c]), pack(dd[1][c], dd[2][c])), pack(dd[2][c], dd[1][c]));
-#pragma unroll
-      for (int x = 0; x < 3; ++x) G[c][x] = fma_nc2(ax, M[x], fma_nc2(ay, M[3 + x], mul2(az, mr[x])));
-    }
-    const df2 ve = mul2(mul2(vw2, col.dM), pack(eta[0], eta[1]));
-    const df2 ve2{p2add(ve.hi, ve.hi), p2add(ve.lo, ve.lo)};  // exact doubling
-    df2 S[3][3];
-    if (div_term) {
-      const dfl m23(-2.0 / 3.0);
-      const df2 vt = mul2(mul2(ve, pack(m23, m23)), add_nc2(add_nc2(G[0][0], G[1][1]), G[2][2]));
-      S[0][0] = fma_nc2(ve2, G[0][0], vt), S[1][1] = fma_nc2(ve2, G[1][1], vt), S[2][2] = fma_nc2(ve2, G[2][2], vt);
-    } else {
-      S[0][0] = mul2(ve2, G[0][0]), S[1][1] = mul2(ve2, G[1][1]), S[2][2] = mul2(ve2, G[2][2]);
-    }
-    S[0][1] = S[1][0] = mul2(ve, add_nc2(G[0][1], G[1][0]));
-    S[0][2] = S[2][0] = mul2(ve, add_nc2(G[0][2], G[2][0]));
-    S[1][2] = S[2][1] = mul2(ve, add_nc2(G[1][2], G[2][1]));
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const df2 h0 = fma_nc2(S[c][0], M[0], fma_nc2(S[c][1], M[1], mul2(S[c][2], M[2])));
-      const df2 h1 = fma_nc2(S[c][0], M[3], fma_nc2(S[c][1], M[4], mul2(S[c][2], M[5])));
-      const df2 h2 = fma_nc2(S[c][0], mr[0], fma_nc2(S[c][1], mr[1], mul2(S[c][2], mr[2])));
-      // X at corners (00, 11) = -(h0 + h1) per lane; at (10, 01) = (h0.x + h1.y, h1.x + h0.y)
-      const df2 x03 = add2(h0, h1);
-      const df2 x12 = add2(pack(lane_x(h0), lane_x(h1)), pack(lane_y(h1), lane_y(h0)));
-      // top-minus-bottom part: h2 at (00, 11), h2.x + h2.y at (10, 01)
-      const dfl hs = lane_x(h2) + lane_y(h2);
-      const df2 h12 = pack(hs, hs);
-      const df2 b03 = add2(x03, h2), t03 = sub2(h2, x03);  // bottom -(x03 + h2), top h2 - x03
-      const df2 b12 = sub2(x12, h12), t12 = add2(x12, h12);
-      accb[0][c] = -lane_x(b03), acct[0][c] = lane_x(t03);
-      accb[3][c] = -lane_y(b03), acct[3][c] = lane_y(t03);
-      accb[1][c] = lane_x(b12), acct[1][c] = lane_x(t12);
-      accb[2][c] = lane_y(b12), acct[2][c] = lane_y(t12);
-    }
-  }
-};
-
 // Packed FP32 pairs (sm_100+ f32x2 instructions): one instruction per pair halves the issue
 // slots of the FP32 element arithmetic, which bounds the FP32 tile kernels.
 __device__ __forceinline__ float2 p2(float a, float b) { return make_float2(a, b); }
@@ -1940,6 +1866,9 @@ __global__ void k_ring_fix(Dims D, RingDims RD, const T* __restrict__ ring, cons
 }
 
 #include "pair32.cuh"
+#if TN_PART == 0 || TN_PART == 2
+#include "df_tile.cuh"
+#endif
 
 // Square tiles: MinBlocks CTAs per SM through the register cap of the launch bounds.
 template <typename T, typename Op, int TI, int TJ, int FLAGS, int EPI = EPI_NONE, int EK = TN_ETA_F32>
@@ -1959,10 +1888,6 @@ __global__ void __maxnreg__(TN_WIDE_MAXREG) k_tile_wide(TN_TILE_PARAMS) {
 template <typename Op, typename T>
 struct OpCompute {
   using type = T;
-};
-template <bool HG, typename T>
-struct OpCompute<OpA<dfl, HG>, T> {
-  using type = dfl;
 };
 template <bool RHO, typename T>
 struct OpCompute<OpDiv<dfl, RHO>, T> {
@@ -2651,15 +2576,41 @@ cudaError_t launch_pair32(const Level& L, BC bc, const OpA<float, HG>& op, const
   return cudaGetLastError();
 }
 
+// The double-float A apply with its tile-line pass (df_tile.cuh; defined with the FP64 launchers).
+template <bool HG, int EPI>
+cudaError_t launch_df_A(const Level& L, BC bc, int div_term, const double* const* in, double* const* out,
+                        cudaStream_t st, const int* skip, const EpiArgs<double>* epi);
+#if TN_PART == 0 || TN_PART == 2
+template <bool HG, int EPI>
+cudaError_t launch_df_A(const Level& L, BC bc, int div_term, const double* const* in, double* const* out,
+                        cudaStream_t st, const int* skip, const EpiArgs<double>* epi) {
+  constexpr int F = PROJ_IN | PROJ_OUT | ADD_ID;
+  EpiArgs<double> E{};
+  if (epi) E = *epi;
+  const Dims D = dims(L);
+  if (!L.laydf || !L.ring64 || L.n_layout >= (int64_t)INT32_MAX || L.n_wedges >= (int64_t)INT32_MAX ||
+      10 * L.n_tri >= (int64_t)INT32_MAX)
+    return cudaErrorInvalidValue;  // 32-bit offsets
+  const int ntiles = (L.N / kDfTI) * (L.N / kDfTJ), ncells = L.n_r - 1;
+  const int kc = radial_chunk((int64_t)ntiles * 10, ncells, 2, kDfMaxKc);
+  k_df_A<HG, F, EPI><<<dim3(ntiles, (ncells + kc - 1) / kc, 10), kDfThreads, df_smem_bytes(HG), st>>>(
+      D, div_term, dfl(hg_coef(L, div_term)), in[0], in[1], in[2], out[0], out[1], out[2], L.geo64,
+      reinterpret_cast<const dfl*>(L.laydf), L.eta64, L.s64, bc.in, bc.out, kc, skip, E, L.ring64);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const RingDims RD = ring_dims(L.N, kDfTI, kDfTJ);
+  k_ring_fix<double, 3, F, EPI><<<dim3(nblk(RD.RC, 256), L.n_r, 10), 256, 0, st>>>(
+      D, RD, L.ring64, in[0], in[1], in[2], out[0], out[1], out[2], L.s64, bc.in, bc.out, skip, E);
+  return cudaGetLastError();
+}
+#endif
+
 template <typename T, bool HG>
 cudaError_t apply_A_hg(const Level& L, BC bc, int div_term, const T* const* u, T* const* y, cudaStream_t st,
                        const int* skip) {
   constexpr int F = PROJ_IN | PROJ_OUT | ADD_ID;
   if constexpr (sizeof(T) == 8) {
-    if (use_df<T>(L)) {
-      OpA<dfl, HG> op{div_term, dfl(hg_coef(L, div_term))};
-      return launch_tile<T, OpA<dfl, HG>, F>(L, bc, op, u, y, etav<T>(L), st, skip);
-    }
+    if (use_df<T>(L)) return launch_df_A<HG, EPI_NONE>(L, bc, div_term, u, y, st, skip, nullptr);
   }
   OpA<T, HG> op{div_term, (T)hg_coef(L, div_term)};
   return launch_tile<T, OpA<T, HG>, F>(L, bc, op, u, y, etav<T>(L), st, skip);
@@ -2713,12 +2664,10 @@ cudaError_t apply_A_epi_hg(const Level& L, BC bc, int div_term, int epi, const T
   constexpr int F = PROJ_IN | PROJ_OUT | ADD_ID;
   if constexpr (sizeof(T) == 8) {
     if (use_df<T>(L)) {
-      using Od = OpA<dfl, HG>;
-      const Od od{div_term, dfl(hg_coef(L, div_term))};
       switch (epi) {
-        case EPI_RESID: return launch_tile<T, Od, F, EPI_RESID>(L, bc, od, in, t, etav<T>(L), st, skip, &E);
-        case EPI_CHEB1: return launch_tile<T, Od, F, EPI_CHEB1>(L, bc, od, in, t, etav<T>(L), st, skip, &E);
-        case EPI_CHEB2: return launch_tile<T, Od, F, EPI_CHEB2>(L, bc, od, in, t, etav<T>(L), st, skip, &E);
+        case EPI_RESID: return launch_df_A<HG, EPI_RESID>(L, bc, div_term, in, t, st, skip, &E);
+        case EPI_CHEB1: return launch_df_A<HG, EPI_CHEB1>(L, bc, div_term, in, t, st, skip, &E);
+        case EPI_CHEB2: return launch_df_A<HG, EPI_CHEB2>(L, bc, div_term, in, t, st, skip, &E);
         default: return cudaErrorInvalidValue;
       }
     }
@@ -2954,7 +2903,8 @@ __global__ void k_eta_16(Dims D, const double* __restrict__ eta, uint16_t* __res
 
 int64_t ring_buffer_entries(int N, int n_r) {
   if (!(TN_HALO_FREE && N >= 2 * TILE)) return 0;
-  const RingDims RD = ring_dims(N, TILE, 2 * TILE);
+  // the larger line set: 16 x 16 tiles (double-float A), 16 x 32 the other users
+  const RingDims RD = ring_dims(N, TILE, TILE);
   return (int64_t)4 * 3 * n_r * 10 * RD.RC;
 }
 
@@ -3029,27 +2979,23 @@ cudaError_t set_wide_attrs() {
   return cudaSuccess;
 }
 
-// The double-float A ops (halo-free tiles only).
-template <typename Op, int EPI>
+#if TN_PART == 0 || TN_PART == 2
+TN_INST_A(double)
+
+// The double-float A kernels.
+template <bool HG, int EPI>
 cudaError_t set_df_attr() {
-  constexpr int F = PROJ_IN | PROJ_OUT | ADD_ID;
-  constexpr size_t shf = TileSmemHF<dfl, Op, TILE, 2 * TILE>::bytes;
-  if (shf > 48 * 1024)
-    return cudaFuncSetAttribute(k_tile_hf<double, Op, TILE, 2 * TILE, F, EPI, TN_ETA_F32, dfl>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shf);
-  return cudaSuccess;
+  return cudaFuncSetAttribute(k_df_A<HG, PROJ_IN | PROJ_OUT | ADD_ID, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)df_smem_bytes(HG));
 }
-template <typename Op>
+template <bool HG>
 cudaError_t set_df_attrs() {
-  const cudaError_t e[4] = {set_df_attr<Op, EPI_NONE>(), set_df_attr<Op, EPI_RESID>(), set_df_attr<Op, EPI_CHEB1>(),
-                            set_df_attr<Op, EPI_CHEB2>()};
+  const cudaError_t e[4] = {set_df_attr<HG, EPI_NONE>(), set_df_attr<HG, EPI_RESID>(), set_df_attr<HG, EPI_CHEB1>(),
+                            set_df_attr<HG, EPI_CHEB2>()};
   for (cudaError_t x : e)
     if (x != cudaSuccess) return x;
   return cudaSuccess;
 }
-
-#if TN_PART == 0 || TN_PART == 2
-TN_INST_A(double)
 
 // Energy residual (Eq. energy) and lumped mass on level L, FP64: R = (K + C(u) + S(u)) T with the
 // element op OpEnergy (u NULL: diffusion only), plus the interface sum over diamond-edge copies.
@@ -3084,7 +3030,7 @@ cudaError_t prepare_energy_kernels() {
 
 cudaError_t prepare_tile_kernels() {
   const cudaError_t e[7] = {prepare_tile_kernels_f32(), set_wide_attrs<OpA<double, false>>(), set_wide_attrs<OpA<double, true>>(),
-                            set_df_attrs<OpA<dfl, false>>(), set_df_attrs<OpA<dfl, true>>(),
+                            set_df_attrs<false>(), set_df_attrs<true>(),
                             prepare_tile_kernels_q2(), prepare_energy_kernels()};
   for (cudaError_t x : e)
     if (x != cudaSuccess) return x;
