@@ -194,13 +194,14 @@ tn_status tn_apply_A(tn_mesh* mesh, int level, tn_prec prec, const void* const* 
 tn_status tn_apply_B(tn_mesh* mesh, int level, tn_prec prec, const void* const* u_dev, void* q_dev, void* stream);
 
 /* q = B P u exactly as tn_apply_B (same kernels, same result), with the one intermediate that
- * tn_apply_B keeps in mesh-owned scratch -- the fine-level divergence field between the element
- * kernel and the restriction -- in a static device array compiled into the library instead (8 MiB,
- * held by every GPU that loads the library until the process exits).  For callers that cannot
- * allocate device memory at the point of the call, e.g. code running under an allocator that
- * forbids cudaMalloc after start-up; this call makes no cudaMalloc, cudaFree or other allocating
- * call.  FP64 levels with N >= 32 still use the ring buffer that tn_mesh_create preallocated for
- * the tile-line partial sums of the halo-free tiles (no allocation, but mesh-owned memory).
+ * tn_apply_B keeps in mesh-owned scratch -- with a reference state, the fine-level divergence field between
+ * the element kernel and the restriction; without one neither call keeps any -- in a static device array
+ * compiled into the library instead (8 MiB, held by every GPU that loads the library until the process exits).
+ * For callers that cannot allocate device memory at the point of the call, e.g. code running under an
+ * allocator that forbids cudaMalloc after start-up; this call makes no cudaMalloc, cudaFree or other
+ * allocating call.  With a reference state FP64 levels with N >= 32 still use the ring buffer that
+ * tn_mesh_create preallocated for the tile-line partial sums of the halo-free tiles (no allocation, but
+ * mesh-owned memory).
  * The paper has no counterpart; it is an addition of this library.
  * Limit: level h's node layout times the element size (8 B for TN_F64, 4 B for TN_F32) must
  * fit in 8 MiB, else TN_EINVAL with the sizes in tn_last_error().  The mesh's device must be

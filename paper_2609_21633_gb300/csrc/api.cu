@@ -73,23 +73,12 @@ cudaError_t apply_B_t(tn_mesh* m, int level, const void* const* u, void* q, cuda
   const Level& F = m->lv[level];
   const Level& C = m->lv[level + 1];
   T* scr = sizeof(T) == 8 ? (T*)F.scr64 : (T*)F.scr32;
-  cudaError_t e = launch_div_fine<T>(F, bc_of(m), (const T* const*)u, scr, st);
-  if (e != cudaSuccess) return e;
-  const T* fin[1] = {scr};
-  T* cout[1] = {(T*)q};
-  return launch_restrict<T>(F, C, bc_of(m), 1, 0, fin, cout, st);
+  return launch_div<T>(F, C, bc_of(m), (const T* const*)u, (T*)q, scr, st);
 }
 
 template <typename T>
 cudaError_t apply_BT_t(tn_mesh* m, int level, const void* p, void* const* y, cudaStream_t st) {
-  const Level& F = m->lv[level];
-  const Level& C = m->lv[level + 1];
-  T* scr = sizeof(T) == 8 ? (T*)F.scr64 : (T*)F.scr32;
-  const T* cin[1] = {(const T*)p};
-  T* fout[1] = {scr};
-  cudaError_t e = launch_prolong<T>(F, C, bc_of(m), 1, 0, cin, fout, st);
-  if (e != cudaSuccess) return e;
-  return launch_grad_fine<T>(F, bc_of(m), scr, (T* const*)y, st);
+  return launch_grad<T>(m->lv[level], m->lv[level + 1], bc_of(m), (const T*)p, (T* const*)y, st);
 }
 
 

@@ -63,9 +63,10 @@ __device__ __forceinline__ void df_cell_A(const float4* sn, const float4* gc, co
     const df2 n12 = df_of(sum2(n10, n01));  // (s, d) of 10 plus 01
     const df2 s0 = pack(lane_x(n00), lane_x(n11)), s1 = pack(lane_x(n10), lane_x(n01)),
               s2 = pack(lane_x(n01), lane_x(n10));
-    const df2 ax = diff2(s1, s0), ay = diff2(s2, s0);
+    // (normalised: after a cancellation their low part is large, and the products drop low x low)
+    const df2 ax = norm2(diff2(s1, s0)), ay = norm2(diff2(s2, s0));
     const df2 d0 = pack(lane_y(n00), lane_y(n11));
-    const df2 az = df_of(sum2(d0, both(lane_y(n12))));
+    const df2 az = norm2(df_of(sum2(d0, both(lane_y(n12)))));
 #pragma unroll
     for (int x = 0; x < 3; ++x) G[c][x] = dot3(ax, M[x], ay, M[3 + x], az, mr[x]);
     if constexpr (HG) {
@@ -96,15 +97,15 @@ __device__ __forceinline__ void df_cell_A(const float4* sn, const float4* gc, co
     for (int c = 0; c < 3; ++c) {
       acc2 a = vt;
       acc_fma2(a, ve2, G[c][c]);
-      S[c][c] = df_of(a);
+      S[c][c] = norm2(df_of(a));
     }
   } else {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) S[c][c] = df_of(prod2(ve2, G[c][c]));
+    for (int c = 0; c < 3; ++c) S[c][c] = norm2(df_of(prod2(ve2, G[c][c])));
   }
-  S[0][1] = S[1][0] = df_of(prod2(ve, df_of(sum2(G[0][1], G[1][0]))));
-  S[0][2] = S[2][0] = df_of(prod2(ve, df_of(sum2(G[0][2], G[2][0]))));
-  S[1][2] = S[2][1] = df_of(prod2(ve, df_of(sum2(G[1][2], G[2][1]))));
+  S[0][1] = S[1][0] = norm2(df_of(prod2(ve, df_of(sum2(G[0][1], G[1][0])))));
+  S[0][2] = S[2][0] = norm2(df_of(prod2(ve, df_of(sum2(G[0][2], G[2][0])))));
+  S[1][2] = S[2][1] = norm2(df_of(prod2(ve, df_of(sum2(G[1][2], G[2][1])))));
   df2 nek{}, e3{};
   if constexpr (HG) {
     acc2 g = prod2(vw2, df_from4(gc[10 * kDfThreads]));

@@ -53,7 +53,7 @@ TN_DF_HD void fast_two_sum(float a, float b, float& s, float& e) {
   e = TN_FSUB(b, TN_FSUB(s, a));
 }
 
-struct dfl {
+struct alignas(8) dfl {
   float hi, lo;
   dfl() = default;
   TN_DF_HD constexpr dfl(float h, float l) : hi(h), lo(l) {}
@@ -195,7 +195,7 @@ TN_DF_HD double join(dfl a) { return widen(a.hi) + widen(a.lo); }
 // each lane to nearest, so a lane follows the scalar formula step for step.  A kernel written with
 // df2 may still group its sums differently from its scalar version: the two then agree to the
 // double-float rounding level (about 2^-46 relative), not bitwise.
-struct df2 {
+struct alignas(16) df2 {
   float2 hi, lo;
 };
 __device__ __forceinline__ float2 p2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -308,6 +308,11 @@ __device__ __forceinline__ acc2 sum2(const df2& x, const df2& y) {
   acc2 a = acc_of(x);
   acc_add2(a, y);
   return a;
+}
+__device__ __forceinline__ df2 norm2(const df2& a) {  // FastTwoSum of the two parts
+  df2 r;
+  fast_two_sum2(a.hi, a.lo, r.hi, r.lo);
+  return r;
 }
 __device__ __forceinline__ df2 neg2(const df2& x) { return df2{p2neg(x.hi), p2neg(x.lo)}; }
 __device__ __forceinline__ df2 diff2(const df2& x, const df2& y) { return df_of(sum2(x, neg2(y))); }

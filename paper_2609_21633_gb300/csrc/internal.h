@@ -219,10 +219,14 @@ inline bool coarse_cg_fits(const Level& L) {
 template <typename T>
 cudaError_t launch_coarse_cg(const Level& L, BC bc, int div_term, const T* const* b, const CoarseCg<T>& C,
                              cudaStream_t st);
+// q = B P u onto the node layout of level C (the pressure space of F), the TALA divergence when F has a reference
+// state (through `scratch`, one value per entry of F's node layout); y = P B^T p.
 template <typename T>
-cudaError_t launch_div_fine(const Level& L, BC bc, const T* const* u, T* q, cudaStream_t st);
+cudaError_t launch_div(const Level& F, const Level& C, BC bc, const T* const* u, T* q, T* scratch, cudaStream_t st);
 template <typename T>
-cudaError_t launch_grad_fine(const Level& L, BC bc, const T* p, T* const* y, cudaStream_t st);
+cudaError_t launch_div_plain(const Level& F, const Level& C, BC bc, const T* const* u, T* q, cudaStream_t st);
+template <typename T>
+cudaError_t launch_grad(const Level& F, const Level& C, BC bc, const T* p, T* const* y, cudaStream_t st);
 template <typename T>
 cudaError_t launch_diag_A(const Level& L, BC bc, int div_term, T* const* d, cudaStream_t st);
 // Inverse of the 3x3 node blocks of P A P + I - P (6 arrays: xx, yy, zz, xy, xz, yz).

@@ -39,7 +39,8 @@
 // The file is compiled six times: TN_PART 1 holds everything but the A-apply launchers, TN_PART 2
 // the FP64 and TN_PART 3 the FP32 A-apply launchers, TN_PART 4 and 5 those of the A apply with
 // the second radial quadrature point (their many tile-kernel instantiations then compile in
-// parallel), TN_PART 6 the coarse multigrid levels' kernels (small.cuh); 0 = all.
+// parallel), TN_PART 6 the coarse multigrid levels' kernels (small.cuh) and the divergence and gradient (saddle.cuh);
+// 0 = all.
 #ifndef TN_PART
 #define TN_PART 0
 #endif
@@ -568,34 +569,29 @@ struct OpA2 {
   }
 };
 
-// Fine-level divergence: each of the six nodes of a wedge gets -V tr(grad u)(q_c) / 6
-// (pressure test function psi = N_n with N_n(q_c) = 1/6); tr grad u = w0 tr G'.
-// RHO (TALA, Eq. mass): -V (rho(q_c) div u_h(q_c) + rho'(q_c) r_hat(q_c) . u_h(q_c)) / 6, the
+// Fine-level divergence with a reference state (without one: k_div, saddle.cuh): each of the six nodes of a
+// wedge gets -V div / 6 (pressure test function psi = N_n with N_n(q_c) = 1/6), tr grad u = w0 tr G'.
+// TALA, Eq. mass: -V (rho(q_c) div u_h(q_c) + rho'(q_c) r_hat(q_c) . u_h(q_c)) / 6, the
 // product rule at the quadrature point; the layer table carries rho(q_c) in slot 10 and
 // rho'(q_c) / (6 w0) in slot 11, u_h(q_c) is the sum of the wedge's three corner sums (top + bottom)
 // over 6, so the bracket is w0 (slot 10 tr G' + slot 11 r_hat . sum_a s_a); r_hat(q_c) per lateral
 // triangle comes from the level's table.
-template <typename T, bool RHO = false>
+template <typename T>
 struct OpDiv {
   static constexpr int NIN = 3, NOUT = 1;
   static constexpr bool USES_ETA = false, LOADS = true, NEEDS_D = true;
-  struct ColR {
+  struct Col {
     T rh[2][3];
   };
-  using Col = typename std::conditional<RHO, ColR, NoCol>::type;
-  const T* rhat = nullptr;  // [3][n_tri] r_hat(q_c) of every lateral triangle (RHO only)
+  const T* rhat = nullptr;  // [3][n_tri] r_hat(q_c) of every lateral triangle
   int n_tri = 0;
   __device__ __forceinline__ Col column(const T (&)[2][9], const T (&)[2], int t0) const {
-    if constexpr (RHO) {
-      ColR c;
+    Col c;
 #pragma unroll
-      for (int w = 0; w < 2; ++w)
+    for (int w = 0; w < 2; ++w)
 #pragma unroll
-        for (int x = 0; x < 3; ++x) c.rh[w][x] = rhat[x * n_tri + t0 + w];
-      return c;
-    } else {
-      return Col{};
-    }
+      for (int x = 0; x < 3; ++x) c.rh[w][x] = rhat[x * n_tri + t0 + w];
+    return c;
   }
   __device__ __forceinline__ void cell(const T (&s)[4][3], const T (&dd)[4][3], const T (&Mi)[2][9],
                                        const T (&dM)[2], const T* lc, const T (&)[2], T (&accb)[4][1],
@@ -613,147 +609,19 @@ struct OpDiv {
         lat = c == 0 ? ax * M[0] + ay * M[3] : lat + ax * M[c] + ay * M[3 + c];
         rad = c == 0 ? az * M[6] : rad + az * M[6 + c];
       }
-      T div = lat + r * rad;
-      if constexpr (RHO) {
-        T rs = 0;
+      T rs = 0;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const T sc = (s[c0][c] + s[c1][c]) + s[c2][c];
-          rs = c == 0 ? col.rh[w][0] * sc : rs + col.rh[w][c] * sc;
-        }
-        div = lc[10] * div + lc[11] * rs;
+      for (int c = 0; c < 3; ++c) {
+        const T sc = (s[c0][c] + s[c1][c]) + s[c2][c];
+        rs = c == 0 ? col.rh[w][0] * sc : rs + col.rh[w][c] * sc;
       }
-      v[w] = (vw6 * dM[w]) * div;
+      v[w] = (vw6 * dM[w]) * (lc[10] * (lat + r * rad) + lc[11] * rs);
     }
     const T v01 = v[0] + v[1];
     accb[0][0] = acct[0][0] = v[0];
     accb[3][0] = acct[3][0] = v[1];
     accb[1][0] = acct[1][0] = v01;
     accb[2][0] = acct[2][0] = v01;
-  }
-};
-
-// Double-float divergence without the TALA term: the arithmetic of OpDiv with the corner
-// differences and the corner combination of the two wedges accurate, the contraction with M^-1 by
-// fused multiply-adds (add_nc / fma_nc), the two wedges in the lanes of packed double-floats.
-template <>
-struct OpDiv<dfl, false> {
-  static constexpr int NIN = 3, NOUT = 1;
-  static constexpr bool USES_ETA = false, LOADS = true, NEEDS_D = true, PREFETCH = true;
-  struct Col {
-    df2 M[9], dM;  // M^-1 entries and |det M| of (W0, W1)
-  };
-  const dfl* rhat = nullptr;
-  int n_tri = 0;
-  __device__ __forceinline__ Col column(const dfl (&Mi)[2][9], const dfl (&dM)[2], int) const {
-    Col c;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) c.M[q] = pack(Mi[0][q], Mi[1][q]);
-    c.dM = pack(dM[0], dM[1]);
-    return c;
-  }
-  // the two wedges in the lanes of packed double-floats (x = W0, y = W1), corner pairs as in
-  // OpA<dfl, false>: a_xi = s_10 - s_00 | s_01 - s_11, a_eta = s_01 - s_00 | s_10 - s_11
-  __device__ __forceinline__ void cell(const dfl (&s)[4][3], const dfl (&dd)[4][3], const dfl (&)[2][9],
-                                       const dfl (&)[2], const dfl* lc, const dfl (&)[2], dfl (&accb)[4][1],
-                                       dfl (&acct)[4][1], const Col& col) const {
-    const df2 r = pack(lc[4], lc[4]), vw6 = pack(lc[7], lc[7]);
-    const df2* M = col.M;
-    df2 lat, rad;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const df2 s0 = pack(s[0][c], s[3][c]), s1 = pack(s[1][c], s[2][c]), s2 = pack(s[2][c], s[1][c]);
-      const df2 ax = sub2(s1, s0), ay = sub2(s2, s0);
-      const dfl d12 = add_nc(dd[1][c], dd[2][c]);
-      const df2 az = add_nc2(pack(dd[0][c], dd[3][c]), pack(d12, d12));
-      lat = c == 0 ? fma_nc2(ax, M[0], mul2(ay, M[3])) : fma_nc2(ax, M[c], fma_nc2(ay, M[3 + c], lat));
-      rad = c == 0 ? mul2(az, M[6]) : fma_nc2(az, M[6 + c], rad);
-    }
-    const df2 v = mul2(mul2(vw6, col.dM), fma_nc2(r, rad, lat));
-    const dfl v01 = lane_x(v) + lane_y(v);
-    accb[0][0] = acct[0][0] = lane_x(v);
-    accb[3][0] = acct[3][0] = lane_y(v);
-    accb[1][0] = acct[1][0] = v01;
-    accb[2][0] = acct[2][0] = v01;
-  }
-};
-
-// Fine-level gradient (transpose of OpDiv): y_j += -V p(q_c) grad N_j(q_c), p(q_c) the mean of
-// the six nodal values; H[:, m] = f M^-1[m, :] (times r for m = 2), f = -vol w0 |det M| p(q_c).
-template <typename T>
-struct OpGrad {
-  static constexpr int NIN = 1, NOUT = 3;
-  static constexpr bool USES_ETA = false, LOADS = true, NEEDS_D = false;
-  using Col = NoCol;
-  __device__ __forceinline__ Col column(const T (&)[2][9], const T (&)[2], int) const { return Col{}; }
-  __device__ __forceinline__ void cell(const T (&sn)[4][1], const T (&)[4][1], const T (&Mi)[2][9],
-                                       const T (&dM)[2], const T* lc, const T (&)[2], T (&accb)[4][3],
-                                       T (&acct)[4][3], const Col&) const {
-    const T r = lc[4], vw6 = lc[7];
-    const T s[4] = {sn[0][0], sn[1][0], sn[2][0], sn[3][0]};
-    T X[4][3], h[2][3];
-#pragma unroll
-    for (int w = 0; w < 2; ++w) {
-      const int c0 = kCorner[w][0], c1 = kCorner[w][1], c2 = kCorner[w][2];
-      const T* M = Mi[w];
-      const T f = (vw6 * dM[w]) * ((s[c0] + s[c1]) + s[c2]);
-      const T fr = f * r;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const T h0 = f * M[c], h1 = f * M[3 + c];
-        h[w][c] = fr * M[6 + c];
-        X[c0][c] = -(h0 + h1);
-        if (w == 0) {
-          X[c1][c] = h0, X[c2][c] = h1;
-        } else {
-          X[c1][c] += h0, X[c2][c] += h1;
-        }
-      }
-    }
-    combine_corners<T, 3>(X, h, accb, acct);
-  }
-};
-
-// Double-float gradient: the pressure sum at q_c (no cancellation) and the products by M^-1 with the
-// sum without the second TwoSum; the corner combination accurate; the two wedges in the lanes of
-// packed double-floats.
-template <>
-struct OpGrad<dfl> {
-  static constexpr int NIN = 1, NOUT = 3;
-  static constexpr bool USES_ETA = false, LOADS = true, NEEDS_D = false, PREFETCH = true;
-  struct Col {
-    df2 M[9], dM;  // M^-1 entries and |det M| of (W0, W1)
-  };
-  __device__ __forceinline__ Col column(const dfl (&Mi)[2][9], const dfl (&dM)[2], int) const {
-    Col c;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) c.M[q] = pack(Mi[0][q], Mi[1][q]);
-    c.dM = pack(dM[0], dM[1]);
-    return c;
-  }
-  // the two wedges in the lanes of packed double-floats (x = W0, y = W1); corners as in OpA<dfl, false>
-  __device__ __forceinline__ void cell(const dfl (&sn)[4][1], const dfl (&)[4][1], const dfl (&)[2][9],
-                                       const dfl (&)[2], const dfl* lc, const dfl (&)[2], dfl (&accb)[4][3],
-                                       dfl (&acct)[4][3], const Col& col) const {
-    const df2 r = pack(lc[4], lc[4]), vw6 = pack(lc[7], lc[7]);
-    const df2* M = col.M;
-    const dfl s12 = add_nc(sn[1][0], sn[2][0]);  // corners 10 and 01 belong to both wedges
-    const df2 f = mul2(mul2(vw6, col.dM), add_nc2(pack(sn[0][0], sn[3][0]), pack(s12, s12)));
-    const df2 fr = mul2(f, r);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const df2 h0 = mul2(f, M[c]), h1 = mul2(f, M[3 + c]), h2 = mul2(fr, M[6 + c]);
-      const df2 x03 = add2(h0, h1);
-      const df2 x12 = add2(pack(lane_x(h0), lane_x(h1)), pack(lane_y(h1), lane_y(h0)));
-      const dfl hs = lane_x(h2) + lane_y(h2);
-      const df2 h12 = pack(hs, hs);
-      const df2 b03 = add2(x03, h2), t03 = sub2(h2, x03);  // bottom -(x03 + h2), top h2 - x03
-      const df2 b12 = sub2(x12, h12), t12 = add2(x12, h12);
-      accb[0][c] = -lane_x(b03), acct[0][c] = lane_x(t03);
-      accb[3][c] = -lane_y(b03), acct[3][c] = lane_y(t03);
-      accb[1][c] = lane_x(b12), acct[1][c] = lane_x(t12);
-      accb[2][c] = lane_y(b12), acct[2][c] = lane_y(t12);
-    }
   }
 };
 
@@ -1505,10 +1373,6 @@ template <typename Op, typename = void>
 struct IsPositive : std::false_type {};
 template <typename Op>
 struct IsPositive<Op, std::void_t<decltype(Op::POSITIVE)>> : std::integral_constant<bool, Op::POSITIVE> {};
-template <typename Op, typename = void>
-struct IsPrefetch : std::false_type {};
-template <typename Op>
-struct IsPrefetch<Op, std::void_t<decltype(Op::PREFETCH)>> : std::integral_constant<bool, Op::PREFETCH> {};
 template <typename Op, typename C>
 __device__ __forceinline__ C node_add(const C& a, const C& b) {
   if constexpr (std::is_same<C, dfl>::value && IsPositive<Op>::value) return add_nc(a, b);
@@ -1689,12 +1553,6 @@ __device__ __forceinline__ void tile_body_hf(TN_TILE_PARAMS, T* __restrict__ rin
 #pragma unroll
     for (int c = 0; c < NOUT; ++c) carry[q][c] = C(0.0);
   const int kstart = kc0 > 0 ? kc0 - 1 : 0;
-  // PREFETCH ops (light element work, held by load latency): the raw input of node layer k + 2 is
-  // loaded while cell layer k is computed, and the extra node (one per thread < NX) keeps its
-  // bottom values from the previous layer instead of loading them again
-  constexpr bool PF = IsPrefetch<Op>::value && NS > 0;
-  T rawn[PF ? NIN : 1], rawx[PF ? NIN : 1];
-  C xbot[PF ? NIN : 1];
   int xoff = 0, xlat = 0, xsi = 0, xsj = 0;
   const bool hasx = (int)threadIdx.x < NX;  // blockDim.x = TI TJ > NX
   if (hasx) {
@@ -1704,32 +1562,9 @@ __device__ __forceinline__ void tile_body_hf(TN_TILE_PARAMS, T* __restrict__ rin
     xlat = d * (N + 1) * P + ni * P + nj;
   }
   if (NS > 0) load_node(c00, lat00, kstart, ub);
-  if constexpr (PF) {
-    load_raw(c00, kstart + 1, rawn);
-    if (hasx) {
-      load_node(xoff, xlat, kstart, xbot);
-      load_raw(xoff, kstart + 1, rawx);
-    }
-  }
   for (int k = kstart; k < kc1; ++k) {
     C s[4][NIN], dd[4][NIN];
-    if constexpr (PF) {
-      C ut[NIN];
-      finish_node(lat00, k + 1, rawn, ut);
-      if (k + 2 <= kc1) load_raw(c00, k + 2, rawn);
-      put_node(ti, tj, ub, ut, s[0], dd[0]);
-#pragma unroll
-      for (int c = 0; c < NIN; ++c) ub[c] = ut[c];
-      if (hasx) {
-        C xt[NIN], xs[NIN], xd[NIN];
-        finish_node(xlat, k + 1, rawx, xt);
-        if (k + 2 <= kc1) load_raw(xoff, k + 2, rawx);
-        put_node(xsi, xsj, xbot, xt, xs, xd);
-#pragma unroll
-        for (int c = 0; c < NIN; ++c) xbot[c] = xt[c];
-      }
-      __syncthreads();
-    } else if (NS > 0) {
+    if (NS > 0) {
       C ut[NIN];
       load_node(c00, lat00, k + 1, ut);
       put_node(ti, tj, ub, ut, s[0], dd[0]);
@@ -1889,12 +1724,8 @@ template <typename Op, typename T>
 struct OpCompute {
   using type = T;
 };
-template <bool RHO, typename T>
-struct OpCompute<OpDiv<dfl, RHO>, T> {
-  using type = dfl;
-};
 template <typename T>
-struct OpCompute<OpGrad<dfl>, T> {
+struct OpCompute<OpDiv<dfl>, T> {
   using type = dfl;
 };
 template <bool HG, typename T>
@@ -2059,6 +1890,7 @@ __global__ void k_interface_epi(Dims D, int n_groups, const int* __restrict__ gp
 
 #if TN_PART == 0 || TN_PART == 6
 #include "small.cuh"
+#include "saddle.cuh"
 #endif
 
 // ------------------------------------------------------------------------------------ diag(A)
@@ -2626,8 +2458,10 @@ cudaError_t apply_A_q2_epi(const Level& L, BC bc, int div_term, int epi, const T
                            T* const* t, cudaStream_t st, const int* skip);
 // Shared-memory opt-ins of the OpA2 tile kernels (see prepare_tile_kernels).
 cudaError_t prepare_tile_kernels_q2();
-// Shared-memory opt-ins of the FP32 paired-cell A kernels (defined with their launchers).
+// Shared-memory opt-ins of the FP32 paired-cell A kernels and of the divergence and gradient kernels (defined
+// with their launchers).
 cudaError_t prepare_tile_kernels_f32();
+cudaError_t prepare_saddle_kernels();
 
 // The FP32 A apply on paired-cell tiles, interface sums included (pair32.cuh).
 template <bool HG>
@@ -2711,6 +2545,7 @@ cudaError_t launch_apply_A_epi(const Level& L, BC bc, int div_term, int epi, con
 }
 
 #if TN_PART == 0 || TN_PART == 1
+// TALA divergence onto the fine node layout, copies summed.
 template <typename T>
 cudaError_t launch_div_fine(const Level& L, BC bc, const T* const* u, T* q, cudaStream_t st) {
   T* out[1] = {q};
@@ -2719,35 +2554,27 @@ cudaError_t launch_div_fine(const Level& L, BC bc, const T* const* u, T* q, cuda
   const int nt = (int)L.n_tri;
   if constexpr (sizeof(T) == 8) {
     if (use_df<T>(L)) {
-      const dfl* rh = reinterpret_cast<const dfl*>(L.rhatdf);
-      e = L.tala ? launch_tile<T, OpDiv<dfl, true>, PROJ_IN>(L, bc, OpDiv<dfl, true>{rh, nt}, u, out, EtaView<T>{}, st)
-                 : launch_tile<T, OpDiv<dfl>, PROJ_IN>(L, bc, OpDiv<dfl>{}, u, out, EtaView<T>{}, st);
+      e = launch_tile<T, OpDiv<dfl>, PROJ_IN>(L, bc, OpDiv<dfl>{reinterpret_cast<const dfl*>(L.rhatdf), nt}, u, out,
+                                              EtaView<T>{}, st);
       done = true;
     }
   }
   if (!done) {
     const T* rh = sizeof(T) == 8 ? (const T*)L.rhat64 : (const T*)L.rhat32;
-    e = L.tala ? launch_tile<T, OpDiv<T, true>, PROJ_IN>(L, bc, OpDiv<T, true>{rh, nt}, u, out, EtaView<T>{}, st)
-               : launch_tile<T, OpDiv<T>, PROJ_IN>(L, bc, OpDiv<T>{}, u, out, EtaView<T>{}, st);
+    e = launch_tile<T, OpDiv<T>, PROJ_IN>(L, bc, OpDiv<T>{rh, nt}, u, out, EtaView<T>{}, st);
   }
   if (e != cudaSuccess) return e;
   return launch_interface<T>(L, bc, 1, 0, out, nullptr, st);
 }
 
 template <typename T>
-cudaError_t launch_grad_fine(const Level& L, BC bc, const T* p, T* const* y, cudaStream_t st) {
-  const T* in[1] = {p};
-  cudaError_t e = cudaSuccess;
-  bool done = false;
-  if constexpr (sizeof(T) == 8) {
-    if (use_df<T>(L)) {
-      e = launch_tile<T, OpGrad<dfl>, PROJ_OUT>(L, bc, OpGrad<dfl>{}, in, y, EtaView<T>{}, st);
-      done = true;
-    }
-  }
-  if (!done) e = launch_tile<T, OpGrad<T>, PROJ_OUT>(L, bc, OpGrad<T>{}, in, y, EtaView<T>{}, st);
+cudaError_t launch_div(const Level& F, const Level& C, BC bc, const T* const* u, T* q, T* scratch, cudaStream_t st) {
+  if (!F.tala) return launch_div_plain<T>(F, C, bc, u, q, st);
+  cudaError_t e = launch_div_fine<T>(F, bc, u, scratch, st);
   if (e != cudaSuccess) return e;
-  return launch_interface<T>(L, bc, 3, 0, y, nullptr, st);
+  const T* fin[1] = {scratch};
+  T* cout[1] = {q};
+  return launch_restrict<T>(F, C, bc, 1, 0, fin, cout, st);
 }
 
 template <typename T>
@@ -2931,8 +2758,7 @@ cudaError_t launch_buoyancy(const Level& L, BC bc, const double* T, double Ra, d
 }
 
 #define TN_INST(T)                                                                                               \
-  template cudaError_t launch_div_fine<T>(const Level&, BC, const T* const*, T*, cudaStream_t);                 \
-  template cudaError_t launch_grad_fine<T>(const Level&, BC, const T*, T* const*, cudaStream_t);                \
+  template cudaError_t launch_div<T>(const Level&, const Level&, BC, const T* const*, T*, T*, cudaStream_t);      \
   template cudaError_t launch_diag_A<T>(const Level&, BC, int, T* const*, cudaStream_t);                        \
   template cudaError_t launch_block_inv_A<T>(const Level&, BC, int, T* const*, cudaStream_t);                   \
   template cudaError_t launch_diag_pmass<T>(const Level&, const Level&, T*, cudaStream_t);                      \
@@ -3029,9 +2855,9 @@ cudaError_t prepare_energy_kernels() {
 }
 
 cudaError_t prepare_tile_kernels() {
-  const cudaError_t e[7] = {prepare_tile_kernels_f32(), set_wide_attrs<OpA<double, false>>(), set_wide_attrs<OpA<double, true>>(),
+  const cudaError_t e[8] = {prepare_tile_kernels_f32(), set_wide_attrs<OpA<double, false>>(), set_wide_attrs<OpA<double, true>>(),
                             set_df_attrs<false>(), set_df_attrs<true>(),
-                            prepare_tile_kernels_q2(), prepare_energy_kernels()};
+                            prepare_tile_kernels_q2(), prepare_energy_kernels(), prepare_saddle_kernels()};
   for (cudaError_t x : e)
     if (x != cudaSuccess) return x;
   return cudaSuccess;
@@ -3104,8 +2930,83 @@ TN_INST_Q2(float)
 #endif
 #undef TN_INST_Q2
 
-// ------------------------------------------------------------ coarse multigrid levels (small.cuh)
+// ------------------------------- coarse multigrid levels (small.cuh), divergence and gradient (saddle.cuh)
 #if TN_PART == 0 || TN_PART == 6
+template <typename C>
+const C* lay_of(const Level& L);
+template <>
+const float* lay_of<float>(const Level& L) { return L.lay32; }
+template <>
+const double* lay_of<double>(const Level& L) { return L.lay64; }
+template <>
+const dfl* lay_of<dfl>(const Level& L) { return reinterpret_cast<const dfl*>(L.laydf); }
+
+// 32-bit offsets of the saddle kernels
+inline bool saddle_ok(const Level& F, const Level& C) {
+  return C.N * 2 == F.N && (C.n_r - 1) * 2 == F.n_r - 1 && F.n_layout < (int64_t)INT32_MAX && 10 * F.n_tri < (int64_t)INT32_MAX;
+}
+
+template <typename T, typename C>
+cudaError_t grad_c(const Level& F, const Level& Lc, BC bc, const T* p, T* const* y, cudaStream_t st) {
+  const int nt = F.N < kGrTile ? F.N : kGrTile, nK = (F.n_r - 1) / 2;
+  const int cols = (F.N / nt) * (F.N / nt) + (F.N + kGrStrip) / kGrStrip + (F.N + kGrStrip - 1) / kGrStrip;
+  const int kc = radial_chunk((int64_t)cols * 10, nK, 2, kGrMaxKc);
+  k_grad<T, C><<<dim3(cols, (nK + kc - 1) / kc, 10), kGrThreads, grad_smem_bytes<C>(), st>>>(
+      dims(F), dims(Lc), nt, p, y[0], y[1], y[2], Tab<T>::geo(F), lay_of<C>(F), Tab<T>::s(F), bc.in, bc.out, kc);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_grad(const Level& F, const Level& C, BC bc, const T* p, T* const* y, cudaStream_t st) {
+  if (!saddle_ok(F, C)) return cudaErrorInvalidValue;
+  cudaError_t e;
+  if constexpr (sizeof(T) == 8) e = use_df<T>(F) ? grad_c<T, dfl>(F, C, bc, p, y, st) : grad_c<T, T>(F, C, bc, p, y, st);
+  else e = grad_c<T, T>(F, C, bc, p, y, st);
+  if (e != cudaSuccess) return e;
+  return launch_interface<T>(F, bc, 3, 0, y, nullptr, st);
+}
+
+template <typename T, typename C>
+cudaError_t div_c(const Level& F, const Level& Lc, BC bc, const T* const* u, T* q, cudaStream_t st) {
+  const int nt = F.N < kDvTile ? F.N : kDvTile, nK = (F.n_r - 1) / 2;
+  const int cols = (F.N / nt) * (F.N / nt);
+  const int kc = radial_chunk((int64_t)cols * 10, nK, 2, kDvMaxKc);
+  k_div<T, C><<<dim3(cols, (nK + kc - 1) / kc, 10), kDvThreads, div_smem_bytes<T, C>(), st>>>(
+      dims(F), dims(Lc), nt, u[0], u[1], u[2], q, Tab<T>::geo(F), lay_of<C>(F), Tab<T>::s(F), bc.in, bc.out, kc);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_div_plain(const Level& F, const Level& C, BC bc, const T* const* u, T* q, cudaStream_t st) {
+  if (!saddle_ok(F, C)) return cudaErrorInvalidValue;
+  cudaError_t e;
+  if constexpr (sizeof(T) == 8) e = use_df<T>(F) ? div_c<T, dfl>(F, C, bc, u, q, st) : div_c<T, T>(F, C, bc, u, q, st);
+  else e = div_c<T, T>(F, C, bc, u, q, st);
+  if (e != cudaSuccess) return e;
+  T* out[1] = {q};
+  return launch_interface<T>(C, bc, 1, 0, out, nullptr, st);
+}
+
+template <typename T, typename C>
+cudaError_t set_saddle_attr() {
+  cudaError_t e = cudaFuncSetAttribute(k_grad<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem_bytes<C>());
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_div<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)div_smem_bytes<T, C>());
+}
+cudaError_t prepare_saddle_kernels() {
+  const cudaError_t e[3] = {set_saddle_attr<float, float>(), set_saddle_attr<double, double>(), set_saddle_attr<double, dfl>()};
+  for (cudaError_t x : e)
+    if (x != cudaSuccess) return x;
+  return cudaSuccess;
+}
+
+#define TN_INST_SADDLE(T)                                                                                          \
+  template cudaError_t launch_grad<T>(const Level&, const Level&, BC, const T*, T* const*, cudaStream_t);         \
+  template cudaError_t launch_div_plain<T>(const Level&, const Level&, BC, const T* const*, T*, cudaStream_t);
+TN_INST_SADDLE(double)
+TN_INST_SADDLE(float)
+#undef TN_INST_SADDLE
+
 template <typename T, typename Op>
 cudaError_t small_A(const Level& L, BC bc, const Op& op, int epi, const T* const* in, const EpiArgs<T>& E, T* const* y,
                     T* sc, cudaStream_t st) {

@@ -45,12 +45,7 @@ cudaError_t apply_B_static_t(const tn_mesh* m, int level, const void* const* u, 
   const Level& F = m->lv[level];
   const Level& C = m->lv[level + 1];
   const BC bc{m->bc_in, m->bc_out};
-  T* scr = (T*)scratch;
-  cudaError_t e = launch_div_fine<T>(F, bc, (const T* const*)u, scr, st);
-  if (e != cudaSuccess) return e;
-  const T* fin[1] = {scr};
-  T* cout[1] = {(T*)q};
-  return launch_restrict<T>(F, C, bc, 1, 0, fin, cout, st);
+  return launch_div<T>(F, C, bc, (const T* const*)u, (T*)q, (T*)scratch, st);
 }
 
 }  // namespace

@@ -901,10 +901,7 @@ tn_status mg_setup_t(tn_mesh* mesh, const void* const* v0, cudaStream_t st) {
     k_fill<T><<<nb(n1), EB, 0, st>>>(n1, (T)1, P.ones_p);
     ckl();
     T* scr = sizeof(T) == 8 ? (T*)L0.scr64 : (T*)L0.scr32;
-    const T* cin[1] = {P.ones_p};
-    T* fout[1] = {scr};
-    ck(launch_prolong<T>(L0, L1, bc, 1, 0, cin, fout, st));
-    ck(launch_grad_fine<T>(L0, bc, scr, G.r.mm(), st));  // c in G.r
+    ck(launch_grad<T>(L0, L1, bc, P.ones_p, G.r.mm(), st));  // c in G.r
     Vec3<T>& wv = P.defl_w;
     Vec3<T>& cc = P.defl_c;
     for (int q = 0; q < 3; ++q) ck(cudaMemcpyAsync(cc.c[q], G.r.c[q], sizeof(T) * n0, cudaMemcpyDeviceToDevice, st));
@@ -920,10 +917,7 @@ tn_status mg_setup_t(tn_mesh* mesh, const void* const* v0, cudaStream_t st) {
       k_axpby<T><<<nb(n0), EB, 0, st>>>(n0, 3, 1.0, P4<T>(G.x().cc(), 3), 1.0, M4<T>(wv.mm(), 3));
       ckl();
     }
-    ck(launch_div_fine<T>(L0, bc, wv.cc(), scr, st));
-    const T* fin[1] = {scr};
-    T* cout[1] = {P.sq};
-    ck(launch_restrict<T>(L0, L1, bc, 1, 0, fin, cout, st));
+    ck(launch_div<T>(L0, L1, bc, wv.cc(), P.sq, scr, st));
     k_axpby<T><<<nb(n1), EB, 0, st>>>(n1, 1, 0.0, P4<T>((const T* const*)&P.sq, 1), -1.0, M4<T>(&P.sq, 1));
     ckl();
     const T* sqa[1] = {P.sq};
@@ -990,17 +984,11 @@ void apply_K(MGState* m, tn_mesh* mesh, const KVec<T>& x, KVec<T>& y, cudaStream
   const BC bc{mesh->bc_in, mesh->bc_out};
   ck(launch_apply_A<T>(L0, bc, mesh->div_term, (const T* const*)x.u, (T* const*)y.u, st));
   T* scr = sizeof(T) == 8 ? (T*)L0.scr64 : (T*)L0.scr32;
-  const T* cin[1] = {x.p};
-  T* fout[1] = {scr};
-  ck(launch_prolong<T>(L0, L1, bc, 1, 0, cin, fout, st));
-  ck(launch_grad_fine<T>(L0, bc, scr, (T* const*)P.tu, st));
+  ck(launch_grad<T>(L0, L1, bc, x.p, (T* const*)P.tu, st));
   k_axpby<T><<<nb(L0.n_layout), EB, 0, st>>>(L0.n_layout, 3, 1.0, P4<T>((const T* const*)P.tu, 3), 1.0,
                                              M4<T>((T* const*)y.u, 3));
   ckl();
-  ck(launch_div_fine<T>(L0, bc, (const T* const*)x.u, scr, st));
-  const T* fin[1] = {scr};
-  T* cout[1] = {y.p};
-  ck(launch_restrict<T>(L0, L1, bc, 1, 0, fin, cout, st));
+  ck(launch_div<T>(L0, L1, bc, (const T* const*)x.u, y.p, scr, st));
 }
 
 // z = P^-1 r: z_p = -r_p / diag(M_1/eta), z_u = V(r_u - B^T z_p).  Split around the V-cycle for
@@ -1021,11 +1009,7 @@ void prec_pre(MGState* m, tn_mesh* mesh, const KVec<T>& r, KVec<T>& z, cudaStrea
     k_schur<T><<<nb(L1.n_layout), EB, 0, st>>>(L1.n_layout, P.mdiag, r.p, z.p);
   }
   ckl();
-  T* scr = sizeof(T) == 8 ? (T*)L0.scr64 : (T*)L0.scr32;
-  const T* cin[1] = {z.p};
-  T* fout[1] = {scr};
-  ck(launch_prolong<T>(L0, L1, bc, 1, 0, cin, fout, st));
-  ck(launch_grad_fine<T>(L0, bc, scr, (T* const*)P.tu, st));
+  ck(launch_grad<T>(L0, L1, bc, z.p, (T* const*)P.tu, st));
   MGLevelT<T>& G = P.L[0];
   k_axpby<T><<<nb(L0.n_layout), EB, 0, st>>>(L0.n_layout, 3, 1.0, P4<T>((const T* const*)r.u, 3), 0.0,
                                              M4<T>(G.b.mm(), 3));
