@@ -405,7 +405,10 @@ tn_status tn_stokes_solve_batch(tn_mesh* const* meshes, int n, const tn_solve_op
  * surface layers keep their values (prescribed temperatures).  The paper's own schemes (SUPG,
  * entropy viscosity, MMOC, Sec. 6) are named there without their discrete forms; this is the
  * library's explicit SUPG reading.  The first energy call on a mesh allocates its workspace
- * (five layout vectors), kept until tn_mesh_destroy.
+ * (five layout vectors), kept until tn_mesh_destroy; the first tn_energy_steps with a velocity another 20 layout
+ * vectors and four values per wedge for the assembled rows of its residual, if they take at most a quarter of
+ * the free device memory (element-by-element residuals otherwise, and while the stream is being captured
+ * before they exist).
  * ---------------------------------------------------------------------------------------- */
 /* R = (K + C(u) + S(u)) T (u_dev NULL: the diffusion K T only; supg 0 drops S).  T_dev, R_dev: node
  * layout of level 0, equal values on node copies; R must not alias T.  Stream-ordered. */

@@ -1,7 +1,7 @@
 // Energy equation (Eq. energy) and the coupled Stokes-energy time loop.
 //
-// Space: the one-point wedge residual R = (K + C(u) + S(u)) T of the tile kernel (OpEnergy in
-// kernels.cu) and the lumped mass m_j = sum_e V_e / 6.  Time: Heun's method (explicit trapezoid),
+// Space: the one-point wedge residual R = (K + C(u) + S(u)) T, element by element in the tile kernel (OpEnergy in
+// kernels.cu) or, for the steps of one call, as assembled rows (energy_rows.cuh), and the lumped mass m_j = sum_e V_e / 6.  Time: Heun's method (explicit trapezoid),
 //   T* = T - dt M^-1 R(T),  T_new = (T + T* - dt M^-1 R(T*)) / 2,
 // on the interior node layers; the two surface layers keep their values (prescribed temperatures).
 // The substep is bounded by the diffusion eigenvalue (power iteration on M^-1 K) and the coupled step
@@ -196,12 +196,15 @@ cudaError_t diffusion_lambda(tn_mesh* mesh, cudaStream_t st, double* lam) {
   return cudaSuccess;
 }
 
+#include "energy_rows.cuh"
+
 cudaError_t heun_steps(tn_mesh* mesh, double* T, const double* const* u, double dt, int n, int supg,
                        cudaStream_t st) {
   const Level& L = mesh->lv[0];
   const Dims D = dims(L);
   EnergyState& S = mesh->en;
   double *R = S.w[0], *T1 = S.w[1], *R1 = S.w[2];
+  if (n > 0 && u && rows_ready(S, L, st)) return heun_rows(S, L, T, T1, u, dt, n, supg, st);
   cudaError_t e = cudaSuccess;
   for (int s = 0; s < n && e == cudaSuccess; ++s) {
     e = launch_energy_residual(L, u, T, R, supg, st);
@@ -272,7 +275,8 @@ double min_spacing(const tn_mesh* mesh) {
 
 void energy_free(tn_mesh* mesh) {
   EnergyState& S = mesh->en;
-  for (void* p : {(void*)S.mass, (void*)S.w[0], (void*)S.w[1], (void*)S.w[2], (void*)S.w[3], (void*)S.part})
+  for (void* p : {(void*)S.mass, (void*)S.w[0], (void*)S.w[1], (void*)S.w[2], (void*)S.w[3], (void*)S.part,
+                  (void*)S.rows, (void*)S.wq})
     if (p) cudaFree(p);
   S = EnergyState();
 }

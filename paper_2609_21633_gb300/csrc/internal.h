@@ -113,13 +113,20 @@ void mg_free(MGState*);
 }
 
 namespace tn {
+struct alignas(32) WedgeFlow {  // per-wedge velocity terms of the energy rows (energy_rows.cuh)
+  double vt, l0, l1, mu;
+};
 // Energy-equation workspace of a mesh (level 0): lumped mass, four work vectors, a reduction
-// buffer and the cached largest eigenvalue of M^-1 K (0: not computed); freed by energy_free.
+// buffer, the cached largest eigenvalue of M^-1 K (0: not computed) and the assembled rows of the Heun steps
+// with their per-wedge values (energy_rows.cuh; rows_refused: no room for them); freed by energy_free.
 struct EnergyState {
   double* mass = nullptr;
   double* w[4] = {};
   double* part = nullptr;
   double lambda = 0;
+  double* rows = nullptr;
+  WedgeFlow* wq = nullptr;
+  bool rows_refused = false;
 };
 }  // namespace tn
 
