@@ -7,7 +7,7 @@
 // instructions.  Constants are in the null space of all three terms, so the rows hold no diagonal and act on
 // differences to the node's own value: exactly zero for constants, and no cancellation of large T.
 // Measured, level 6 / 65 layers: ten Heun steps 39.9 -> 7.7 ms (wedge values 0.73 ms, rows 2.3 ms, 0.23 ms per stage,
-// all held by the FP64 pipe); one step 4.0 -> 3.5 ms.
+// all held by the FP64 pipe); one step 4.0 -> 3.6 ms.
 // Nodes that several diamonds share keep one partial row per copy (the wedges of that diamond).
 
 struct RowDims {

@@ -61,8 +61,7 @@ struct Level {
   // Per-triangle factors of the diagonal of A ([24][n_tri], see OpDiag), for div term dcoef_div.
   double* dcoef64 = nullptr;
   float* dcoef32 = nullptr;
-  float* dcoefdf = nullptr;  // the same table as double-float pairs (hi, lo)
-  // ... and per cell (the two triangles t = 2 p, 2 p + 1 of a lateral cell): [q][n_tri / 2] float4
+  // the same table as double-float pairs per cell (the two triangles t = 2 p, 2 p + 1 of a lateral cell): [q][n_tri / 2] float4
   // (hi of t, hi of t + 1, lo of t, lo of t + 1), the lanes of the packed double-float diagonal
   float4* dcoefdf2 = nullptr;
   int dcoef_div = -1;

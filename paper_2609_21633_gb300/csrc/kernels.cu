@@ -779,63 +779,6 @@ struct OpMass {
   }
 };
 
-// Double-float diagonal (one-point, no hourglass control): sums of positive terms, so every
-// addition but the accumulation over the two wedges uses add_nc / fma_nc.
-// Double-float diagonal without hourglass control, the two wedges of the cell in the lanes of
-// packed df2 values (x = W0, y = W1) as in OpA<dfl, false>; the factor table comes per cell
-// (Level::dcoefdf2), one 16-byte load per factor for both wedges.  Every contribution is a sum of
-// squares, so the node sums of the tile kernel (POSITIVE) and the corner sums here use the
-// double-word addition without the second TwoSum, which is accurate for operands of one sign.
-template <>
-struct OpDiag<dfl, false> {
-  static constexpr int NIN = 1, NOUT = 3;
-  static constexpr bool USES_ETA = true, LOADS = false, NEEDS_D = false, POSITIVE = true;
-  struct Col {
-    int p0;  // the cell's entry of the per-cell table
-  };
-  int div_term;
-  dfl hgk;
-  const float4* coef;  // [kDiagCoef][n_tri / 2]
-  int n_pair;
-  __device__ __forceinline__ Col column(const dfl (&)[2][9], const dfl (&)[2], int t0) const { return Col{t0 >> 1}; }
-  __device__ __forceinline__ void cell(const dfl (&)[4][1], const dfl (&)[4][1], const dfl (&)[2][9], const dfl (&dM)[2],
-                                       const dfl* lc, const dfl (&eta)[2], dfl (&accb)[4][3], dfl (&acct)[4][3],
-                                       const Col& col) const {
-    const df2 r = pack(lc[4], lc[4]), vw2 = pack(lc[5], lc[5]);
-    const df2 r2 = mul2(r, r), rr{p2add(r.hi, r.hi), p2add(r.lo, r.lo)};  // exact doubling
-    const df2 A = mul2(mul2(vw2, pack(dM[0], dM[1])), pack(eta[0], eta[1]));
-    const df2 Ar2 = mul2(A, r2), A2r = mul2(A, rr);
-    const float4* const cf = coef + col.p0;
-    auto C = [&](int q) {
-      const float4 v = cf[(int64_t)q * n_pair];
-      return df2{make_float2(v.x, v.y), make_float2(v.z, v.w)};
-    };
-    df2 AQ[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) AQ[d] = mul2(Ar2, C(18 + d));
-    df2 vb[3][3], vt[3][3];  // local node a, component d; lanes (W0, W1)
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const df2 inner = fma_nc2(A, C(3 * a + d), AQ[d]);
-        const df2 cr = mul2(A2r, C(9 + 3 * a + d));
-        vb[a][d] = add_nc2(inner, df2{p2neg(cr.hi), p2neg(cr.lo)});
-        vt[a][d] = add_nc2(inner, cr);
-      }
-    // corners: 00 = W0 node 0, 11 = W1 node 0, 10 = W0 node 1 + W1 node 2, 01 = W0 node 2 + W1 node 1
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      accb[0][d] = lane_x(vb[0][d]), acct[0][d] = lane_x(vt[0][d]);
-      accb[3][d] = lane_y(vb[0][d]), acct[3][d] = lane_y(vt[0][d]);
-      const df2 b12 = add_nc2(pack(lane_x(vb[1][d]), lane_x(vb[2][d])), pack(lane_y(vb[2][d]), lane_y(vb[1][d])));
-      const df2 t12 = add_nc2(pack(lane_x(vt[1][d]), lane_x(vt[2][d])), pack(lane_y(vt[2][d]), lane_y(vt[1][d])));
-      accb[1][d] = lane_x(b12), accb[2][d] = lane_y(b12);
-      acct[1][d] = lane_x(t12), acct[2][d] = lane_y(t12);
-    }
-  }
-};
-
 // Diagonal in gradient form (the FP32 path, where the table loads cost more than the arithmetic
 // they save): node (a, side) of a wedge gets ve (|g|^2 + c g_d^2) with g = l_a w0 -/+ w1 m2
 // formed per cell, plus the hourglass term of OpDiag.
@@ -1367,18 +1310,6 @@ struct TileSmemHF {
   static constexpr size_t bytes = sizeof(C) * (size_t)(SD + SM);
 };
 
-// Ops whose contributions all have one sign (POSITIVE = true) let the tile kernel sum nodes with
-// the double-word addition without the second TwoSum; the others use the accurate one.
-template <typename Op, typename = void>
-struct IsPositive : std::false_type {};
-template <typename Op>
-struct IsPositive<Op, std::void_t<decltype(Op::POSITIVE)>> : std::integral_constant<bool, Op::POSITIVE> {};
-template <typename Op, typename C>
-__device__ __forceinline__ C node_add(const C& a, const C& b) {
-  if constexpr (std::is_same<C, dfl>::value && IsPositive<Op>::value) return add_nc(a, b);
-  else return a + b;
-}
-
 // storage <-> compute conversions: identities, or binary64 <-> double-float
 template <typename C>
 __device__ __forceinline__ C to_compute(double x) {
@@ -1520,9 +1451,9 @@ __device__ __forceinline__ void tile_body_hf(TN_TILE_PARAMS, T* __restrict__ rin
 #pragma unroll
       for (int c = 0; c < NOUT; ++c) {
         C a = acc[0][c];
-        if (ti >= 1) a = node_add<Op>(a, SM(0, c, ti - 1, tj));
-        if (tj >= 1) a = node_add<Op>(a, SM(1, c, ti, tj - 1));
-        if (ti >= 1 && tj >= 1) a = node_add<Op>(a, SM(2, c, ti - 1, tj - 1));
+        if (ti >= 1) a = a + SM(0, c, ti - 1, tj);
+        if (tj >= 1) a = a + SM(1, c, ti, tj - 1);
+        if (ti >= 1 && tj >= 1) a = a + SM(2, c, ti - 1, tj - 1);
         v[c] = a;
       }
       if (interior) store_node(k, c00 + k * LS, lat00, v);
@@ -1537,9 +1468,9 @@ __device__ __forceinline__ void tile_body_hf(TN_TILE_PARAMS, T* __restrict__ rin
 #pragma unroll
       for (int c = 0; c < NOUT; ++c) {
         C a = C(0.0);
-        if (si >= 1 && sj < TJ) a = node_add<Op>(a, SM(0, c, si - 1, sj));
-        if (sj >= 1 && si < TI) a = node_add<Op>(a, SM(1, c, si, sj - 1));
-        if (si >= 1 && sj >= 1) a = node_add<Op>(a, SM(2, c, si - 1, sj - 1));
+        if (si >= 1 && sj < TJ) a = a + SM(0, c, si - 1, sj);
+        if (sj >= 1 && si < TI) a = a + SM(1, c, si, sj - 1);
+        if (si >= 1 && sj >= 1) a = a + SM(2, c, si - 1, sj - 1);
         v[c] = a;
       }
       ring_store(k, i0 + si, j0 + sj, 2 * (si == 0) + (sj == 0), v);
@@ -1618,7 +1549,7 @@ __device__ __forceinline__ void tile_body_hf(TN_TILE_PARAMS, T* __restrict__ rin
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int c = 0; c < NOUT; ++c) accb[q][c] = node_add<Op>(accb[q][c], carry[q][c]);
+        for (int c = 0; c < NOUT; ++c) accb[q][c] = accb[q][c] + carry[q][c];
       exchange_write(k, accb);
     }
     if (NS == 0 || k < kc0) __syncthreads();
@@ -1647,10 +1578,11 @@ template <typename T, int NOUT, int FLAGS, int EPI>
 __global__ void k_ring_fix(Dims D, RingDims RD, const T* __restrict__ ring, const T* __restrict__ in0,
                            const T* __restrict__ in1, const T* __restrict__ in2, T* __restrict__ out0,
                            T* __restrict__ out1, T* __restrict__ out2, const T* __restrict__ svec, int bc_in,
-                           int bc_out, const int* __restrict__ skip, EpiArgs<T> E) {
+                           int bc_out, const int* __restrict__ skip, EpiArgs<T> E, int k_first = 0) {
   if (skip && *skip) return;
   const int N = D.N, n_r = D.n_r;
-  const int rid = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y, d = blockIdx.z;  // grid: RC x n_r x 10
+  // grid: RC x node layers (k_first ...) x 10
+  const int rid = blockIdx.x * blockDim.x + threadIdx.x, k = k_first + blockIdx.y, d = blockIdx.z;
   if (rid >= RD.RC) return;
   const int64_t per_k = (int64_t)10 * RD.RC;
   int i, j;
@@ -1728,10 +1660,6 @@ template <typename T>
 struct OpCompute<OpDiv<dfl>, T> {
   using type = dfl;
 };
-template <bool HG, typename T>
-struct OpCompute<OpDiag<dfl, HG>, T> {
-  using type = dfl;
-};
 
 template <typename T, typename Op, int FLAGS, int EPI = EPI_NONE>
 cudaError_t launch_tile(const Level& L, BC bc, Op op, const T* const* in, T* const* out, const EtaView<T>& eta,
@@ -1793,7 +1721,7 @@ cudaError_t launch_tile(const Level& L, BC bc, Op op, const T* const* in, T* con
       if (e != cudaSuccess) return e;
       const RingDims RD = ring_dims(L.N, TI, TJ);
       k_ring_fix<T, Op::NOUT, FLAGS, EPI><<<dim3(nblk(RD.RC, 256), L.n_r, 10), 256, 0, st>>>(D, RD, (const T*)L.ring64, in[0], i1, i2,
-                                                                        out[0], o1, o2, sv, bc.in, bc.out, skip, E);
+                                                                        out[0], o1, o2, sv, bc.in, bc.out, skip, E, 0);
       return cudaGetLastError();
     }
     if constexpr (!kDF) {
@@ -1928,13 +1856,23 @@ __device__ __forceinline__ void add_second_point(const T (&Mi)[9], T cxi, T ceta
 }
 
 template <typename T>
-__global__ void k_diag_A(Dims D, const T* __restrict__ geo, const T* __restrict__ lay, EtaView<T> eta,
-                         const T* __restrict__ svec, int bc_in, int bc_out, int div_term, T hgk, int nq, T* d0,
-                         T* d1, T* d2) {
+struct DiagBoundary {
+  const T *geo, *lay;
+  EtaView<T> eta;
+  const T* svec;
+  int bc_in, bc_out, div_term;
+  T hgk;
+  int nq;
+};
+template <typename T>
+__device__ __forceinline__ void diag_boundary_node(const Dims& D, const DiagBoundary<T>& Q, int t, int side_, int d,
+                                                   T* d0, T* d1, T* d2) {
+  const T *geo = Q.geo, *lay = Q.lay, *svec = Q.svec;
+  const EtaView<T>& eta = Q.eta;
+  const int bc_in = Q.bc_in, bc_out = Q.bc_out, div_term = Q.div_term, nq = Q.nq;
+  const T hgk = Q.hgk;
   const int N = D.N, M = N + 1;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;  // grid: lattice points x 2 layers x 10 diamonds
-  if (t >= M * M) return;
-  const int i = t / M, j = t - i * M, side_ = blockIdx.y, d = blockIdx.z;
+  const int i = t / M, j = t - i * M;
   const int k = side_ == 0 ? 0 : D.n_r - 1;
   // (cell di, cell dj, wedge, local lateral node) of the six triangles around lattice node (i, j)
   const int tri[6][4] = {{0, 0, 0, 0}, {-1, 0, 0, 1}, {-1, 0, 1, 2}, {0, -1, 0, 2}, {0, -1, 1, 1}, {-1, -1, 1, 0}};
@@ -1998,6 +1936,16 @@ __global__ void k_diag_A(Dims D, const T* __restrict__ geo, const T* __restrict_
   const int64_t idx = (int64_t)d * D.diamond_stride + (int64_t)k * D.layer_stride + (int64_t)i * D.P + j;
   d0[idx] = out[0], d1[idx] = out[1], d2[idx] = out[2];
 }
+
+template <typename T>
+__global__ void k_diag_A(Dims D, DiagBoundary<T> Q, T* d0, T* d1, T* d2) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;  // grid: lattice points x 2 layers x 10 diamonds
+  if (t < (D.N + 1) * (D.N + 1)) diag_boundary_node<T>(D, Q, t, (int)blockIdx.y, (int)blockIdx.z, d0, d1, d2);
+}
+
+#if TN_PART == 0 || TN_PART == 2
+#include "df_diag.cuh"
+#endif
 
 // ------------------------------------------------------------------------------------ node blocks
 // Thread per layout node: the 3x3 node block of the constrained operator, P_j A_jj P_j + I - P_j,
@@ -2432,8 +2380,36 @@ cudaError_t launch_df_A(const Level& L, BC bc, int div_term, const double* const
   if (e != cudaSuccess) return e;
   const RingDims RD = ring_dims(L.N, kDfTI, kDfTJ);
   k_ring_fix<double, 3, F, EPI><<<dim3(nblk(RD.RC, 256), L.n_r, 10), 256, 0, st>>>(
-      D, RD, L.ring64, in[0], in[1], in[2], out[0], out[1], out[2], L.s64, bc.in, bc.out, skip, E);
+      D, RD, L.ring64, in[0], in[1], in[2], out[0], out[1], out[2], L.s64, bc.in, bc.out, skip, E, 0);
   return cudaGetLastError();
+}
+#endif
+
+// The double-float diag(A), boundary layers included, without the interface sum (df_diag.cuh).
+cudaError_t launch_df_diag(const Level& L, BC bc, int div_term, double* const* d, cudaStream_t st);
+#if TN_PART == 0 || TN_PART == 2
+template <bool HG>
+cudaError_t df_diag(const Level& L, BC bc, int div_term, double* const* d, cudaStream_t st) {
+  const Dims D = dims(L);
+  if (!L.laydf || !L.dcoefdf2 || !L.ring64 || L.n_layout >= (int64_t)INT32_MAX || L.n_wedges >= (int64_t)INT32_MAX ||
+      10 * L.n_tri >= (int64_t)INT32_MAX)
+    return cudaErrorInvalidValue;
+  const int ntiles = (L.N / kDfTI) * (L.N / kDfTJ), layers = L.n_r - 2;
+  const int kc = radial_chunk((int64_t)ntiles * 10, layers, 2, kDgMaxKc);
+  const DiagBoundary<double> B{L.geo64, L.lay64, etav<double>(L), L.s64, bc.in, bc.out, div_term, hg_coef(L, div_term), L.quad};
+  k_df_diag<HG><<<dim3(ntiles, 2 + (layers + kc - 1) / kc, 10), kDfThreads, df_diag_smem(HG), st>>>(
+      D, dfl(hg_coef(L, div_term)), B, d[0], d[1], d[2], L.dcoefdf2, (int)(L.n_tri / 2),
+      reinterpret_cast<const dfl*>(L.laydf), L.eta64, kc, L.ring64);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const RingDims RD = ring_dims(L.N, kDfTI, kDfTJ);
+  k_ring_fix<double, 3, 0, EPI_NONE><<<dim3(nblk(RD.RC, 256), layers, 10), 256, 0, st>>>(
+      D, RD, L.ring64, d[0], d[0], d[0], d[0], d[1], d[2], L.s64, bc.in, bc.out, nullptr, EpiArgs<double>{}, 1);
+  return cudaGetLastError();
+}
+cudaError_t launch_df_diag(const Level& L, BC bc, int div_term, double* const* d, cudaStream_t st) {
+  if (L.dcoef_div != div_term) return cudaErrorInvalidValue;
+  return L.hg_kappa > 0 ? df_diag<true>(L, bc, div_term, d, st) : df_diag<false>(L, bc, div_term, d, st);
 }
 #endif
 
@@ -2590,15 +2566,9 @@ cudaError_t launch_diag_A(const Level& L, BC bc, int div_term, T* const* d, cuda
   } else if constexpr (sizeof(T) == 8) {  // FP64: per-triangle factor table
     if (!L.dcoef64 || L.dcoef_div != div_term) return cudaErrorInvalidValue;  // built with the level
     const int nt = (int)L.n_tri;
-    if (use_df<T>(L)) {  // the table's double-float copy
-      if (!L.dcoefdf) return cudaErrorInvalidValue;
-      const dfl* cdf = reinterpret_cast<const dfl*>(L.dcoefdf);
-      const dfl hk(hg_coef(L, div_term));
-      if (!hg && !L.dcoefdf2) return cudaErrorInvalidValue;
-      e = hg ? launch_tile<T, OpDiag<dfl, true>, 0>(L, bc, OpDiag<dfl, true>{div_term, hk, cdf, nt}, none, d,
-                                                    etav<T>(L), st)
-             : launch_tile<T, OpDiag<dfl, false>, 0>(L, bc, OpDiag<dfl, false>{div_term, hk, L.dcoefdf2, nt / 2},
-                                                     none, d, etav<T>(L), st);
+    if (use_df<T>(L)) {
+      e = launch_df_diag(L, bc, div_term, d, st);
+      return e != cudaSuccess ? e : launch_interface<T>(L, bc, 3, 2, d, nullptr, st);
     } else {
       const T* coef = Tab<T>::dcoef(L);
       e = hg ? launch_tile<T, OpDiag<T, true>, 0>(L, bc, OpDiag<T, true>{div_term, hgk, coef, nt}, none, d,
@@ -2611,8 +2581,9 @@ cudaError_t launch_diag_A(const Level& L, BC bc, int div_term, T* const* d, cuda
            : launch_tile<T, OpDiagG<T, false>, 0>(L, bc, OpDiagG<T, false>{div_term, hgk}, none, d, etav<T>(L), st);
   }
   if (e != cudaSuccess) return e;
-  k_diag_A<T><<<dim3(nblk((int64_t)(L.N + 1) * (L.N + 1), 256), 2, 10), 256, 0, st>>>(D, Tab<T>::geo(L), Tab<T>::lay(L), etav<T>(L), Tab<T>::s(L), bc.in,
-                                            bc.out, div_term, hgk, L.quad, d[0], d[1], d[2]);
+  k_diag_A<T><<<dim3(nblk((int64_t)(L.N + 1) * (L.N + 1), 256), 2, 10), 256, 0, st>>>(
+      D, DiagBoundary<T>{Tab<T>::geo(L), Tab<T>::lay(L), etav<T>(L), Tab<T>::s(L), bc.in, bc.out, div_term, hgk, L.quad},
+      d[0], d[1], d[2]);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_interface<T>(L, bc, 3, 2, d, nullptr, st);
@@ -2816,8 +2787,10 @@ cudaError_t set_df_attr() {
 }
 template <bool HG>
 cudaError_t set_df_attrs() {
-  const cudaError_t e[4] = {set_df_attr<HG, EPI_NONE>(), set_df_attr<HG, EPI_RESID>(), set_df_attr<HG, EPI_CHEB1>(),
-                            set_df_attr<HG, EPI_CHEB2>()};
+  const cudaError_t e[5] = {set_df_attr<HG, EPI_NONE>(), set_df_attr<HG, EPI_RESID>(), set_df_attr<HG, EPI_CHEB1>(),
+                            set_df_attr<HG, EPI_CHEB2>(),
+                            cudaFuncSetAttribute(k_df_diag<HG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)df_diag_smem(HG))};
   for (cudaError_t x : e)
     if (x != cudaSuccess) return x;
   return cudaSuccess;
