@@ -56,7 +56,7 @@ std::vector<float> to_f32(const std::vector<T>& v) {
 void free_level(Level& L) {
   void* ptrs[] = {L.geo64, L.geo32, L.lay64, L.lay32, L.laydf, L.s64,   L.s32,   L.grp_ptr, L.grp_off, L.grp_s64,
                   L.grp_s32, L.owned, L.eta64, L.eta32, L.eta16, L.eta_cs, L.scr64, L.scr32, L.wmask, L.rad64,
-                  L.rad32, L.dcoef64, L.dcoef32,  L.dcoefdf2, L.ring64, L.grp_dij, L.bw64, L.rhat64, L.rhat32, L.rhatdf};
+                  L.rad32, L.dcoef64, L.dcoef32,  L.dcoefdf2, L.ring64, L.edge, L.bw64, L.rhat64, L.rhat32, L.rhatdf};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   L = Level();
@@ -191,15 +191,24 @@ tn_status create_level(Level& L, int l, int nr, double r_in, double r_out, int e
     chk(cudaMalloc((void**)&L.eta_cs, sizeof(float) * L.n_tri));
   }
   {
+    std::vector<int4> items;
+    for (int pass = 0; pass < 2; ++pass)  // vertices (3 or 5 copies), then edge points (2)
+      for (int g = 0; g < L.n_groups; ++g) {
+        const int b = gptr[g], cnt = gptr[g + 1] - b, lanes = pass == 0 ? 8 : 2;
+        if ((cnt > 2) != (pass == 0)) continue;
+        for (int q = 0; q < lanes; ++q) {
+          const int64_t o = goff[b + std::min(q, cnt - 1)], d = o / L.diamond_stride, r = o % L.diamond_stride;
+          items.push_back(make_int4((int)r, (int)d | (q < cnt ? cnt : 0) << 8 | q << 16,
+                                    (int)(r / L.P) | (int)(r % L.P) << 16, g));
+        }
+      }
+    L.n_edge = (int)items.size();
+    chk(upload(L.edge, items));
+  }
+  {
     const int64_t nring = ring_buffer_entries(L.N, L.n_r);
     if (nring > 0) {
       chk(cudaMalloc((void**)&L.ring64, sizeof(double) * nring));
-      std::vector<int4> dij(goff.size());
-      for (size_t q = 0; q < goff.size(); ++q) {
-        const int64_t d = goff[q] / L.diamond_stride, r = goff[q] % L.diamond_stride;
-        dij[q] = make_int4((int)d, (int)(r / L.P), (int)(r % L.P), 0);
-      }
-      chk(upload(L.grp_dij, dij));
     }
   }
   chk(cudaMalloc((void**)&L.scr64, sizeof(double) * L.n_layout));

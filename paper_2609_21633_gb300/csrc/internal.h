@@ -69,8 +69,12 @@ struct Level {
   // [4 slots][3 components][n_r][10][tile-line nodes of a diamond layer]; the FP32 paired-cell
   // tiles use the same allocation as float4 entries [4 slots][n_r][10][tile-line nodes].
   double* ring64 = nullptr;
-  // (diamond, i, j, 0) of every interface copy (grp_off order), levels with a ring buffer.
-  int4* grp_dij = nullptr;
+  // One entry per copy of every interface point, laid out for warps: the copies of a group are neighbouring lanes
+  // (the twelve icosahedron vertices first, eight lanes each, then the edge points, two lanes each), so a group is
+  // summed by shuffles.  x: i P + j, y: diamond | copies << 8 | lane in the group << 16 (0 copies: an unused lane),
+  // z: i | j << 16, w: group.
+  int4* edge = nullptr;
+  int n_edge = 0;
   uint16_t* eta16 = nullptr;
   float* eta_cs = nullptr;
   // Scratch scalar field in this level's node layout (B / B^T intermediate).
@@ -247,7 +251,7 @@ cudaError_t launch_interface(const Level& L, BC bc, int ncomp, int mode, T* cons
                              cudaStream_t st, const int* skip = nullptr);
 template <typename T>
 cudaError_t launch_prolong(const Level& F, const Level& C, BC bc, int ncomp, int apply_bc, const T* const* c,
-                           T* const* f, cudaStream_t st);
+                           T* const* f, cudaStream_t st, bool add = false);
 template <typename T>
 cudaError_t launch_restrict(const Level& F, const Level& C, BC bc, int ncomp, int apply_bc, const T* const* f,
                             T* const* c, cudaStream_t st);

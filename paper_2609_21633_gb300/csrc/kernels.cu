@@ -920,6 +920,20 @@ __device__ __forceinline__ void prefetch_l1(const T* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
+// L1 prefetch of the operands that the fused update of node idx will read.
+template <typename T, int EPI>
+__device__ __forceinline__ void epi_prefetch(const EpiArgs<T>& E, int idx) {
+  if (EPI == EPI_NONE) return;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    if (EPI == EPI_CHEB2) prefetch_l1(E.r[c] + idx), prefetch_l1(E.xacc[c] + idx);
+    else prefetch_l1(E.b[c] + idx);
+  }
+  if (EPI != EPI_RESID)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) prefetch_l1(E.binv[q] + idx);
+}
+
 // Fused vector update at node idx from y = (K x)(idx) (see EpiArgs); `in` is the apply input.
 template <typename T, int EPI>
 __device__ __forceinline__ void epilogue(const EpiArgs<T>& E, const T* in0, const T* in1, const T* in2, int idx,
@@ -1632,6 +1646,56 @@ __global__ void k_ring_fix(Dims D, RingDims RD, const T* __restrict__ ring, cons
   if (NOUT > 2) out2[idx] = v[NOUT > 2 ? 2 : 0];
 }
 
+// ------------------------------------------------------------------------------------ lattice points
+// A copy of a lateral point: diamond, lattice position, copies of the point (0: an unused lane), this copy's rank, its
+// interface group (-1: inside a diamond).
+struct Point {
+  int d, i, j, cnt, lane, g;
+};
+struct Points {
+  int N, P, n_edge, n;  // n: edge entries and the points inside the diamonds
+  const int4* edge;
+};
+inline Points points_of(const Level& L) {
+  return Points{L.N, L.P, L.n_edge, L.n_edge + 10 * (L.N - 1) * (L.N - 1), L.edge};
+}
+__device__ __forceinline__ Point edge_point(const int4& v) {
+  return Point{v.y & 0xff, v.z & 0xffff, v.z >> 16, (v.y >> 8) & 0xff, v.y >> 16, v.w};
+}
+// entry u: the edge table, then the points inside the diamonds
+__device__ __forceinline__ Point point_at(const Points& S, int u) {
+  if (u < S.n_edge) return edge_point(S.edge[u]);
+  if (u >= S.n) return Point{0, 0, 0, 0, 0, -1};
+  const int w = u - S.n_edge, n1 = S.N - 1, per = n1 * n1, d = w / per, r = w - d * per, i = r / n1;
+  return Point{d, i + 1, r - i * n1 + 1, 1, 0, -1};
+}
+// Sum over the copies of every point of the warp, in ascending copy order, the same bits in every copy.  All lanes
+// call it; u: the warp's first table entry (the vertices' warps sum up to five copies, the others two).
+template <typename T, int NC>
+__device__ __forceinline__ void copies_sum(const Point& p, int u, T (&v)[NC]) {
+  const int base = ((int)threadIdx.x & 31) - p.lane, most = u < 96 ? 5 : 2;
+  T s[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) s[c] = __shfl_sync(0xffffffffu, v[c], base);
+  for (int q = 1; q < most; ++q) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const T t = __shfl_sync(0xffffffffu, v[c], base + q);
+      if (q < p.cnt) s[c] += t;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) v[c] = s[c];
+}
+// Unit vector of a point, the same for every copy.
+template <typename T>
+__device__ __forceinline__ void point_dir(const Point& p, const T* gs, int n_groups, const T* svec, int ls, int P, int nll,
+                                          T (&s)[3]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    s[c] = p.g >= 0 ? gs[c * n_groups + p.g] : svec[c * nll + p.d * ls + p.i * P + p.j];
+}
+
 #include "pair32.cuh"
 #if TN_PART == 0 || TN_PART == 2
 #include "df_tile.cuh"
@@ -1747,73 +1811,71 @@ cudaError_t launch_tile(const Level& L, BC bc, Op op, const T* const* in, T* con
 }
 
 // ------------------------------------------------------------------------------------ interface
+// Thread per copy and node layer: the copies' partial sums added, written to every copy (mode 1: + (I - P) u at the
+// boundary layers, 2: + diag(I - P)).  One copy per thread: a thread per group walked its copies one after the
+// other, each a chain of dependent loads (29 us for the FP32 smoother's edges at level 6 / 65 layers).
 template <typename T>
-__global__ void k_interface(Dims D, int n_groups, const int* __restrict__ gptr, const int64_t* __restrict__ goff,
-                            const T* __restrict__ gs, int ncomp, int mode, T* y0, T* y1, T* y2,
-                            const T* __restrict__ u0, const T* __restrict__ u1, const T* __restrict__ u2,
-                            int bc_in, int bc_out, const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  const int g = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;  // grid: groups x layers
-  if (g >= n_groups) return;
-  T* y[3] = {y0, y1, y2};
-  const T* u[3] = {u0, u1, u2};
-  const int b = gptr[g], e = gptr[g + 1];
-  const int64_t lo = (int64_t)k * D.layer_stride;
-  T v[3] = {0, 0, 0};
-  for (int q = b; q < e; ++q)
-    for (int c = 0; c < ncomp; ++c) v[c] += y[c][goff[q] + lo];
-  if (mode != 0 && (k == 0 || k == D.n_r - 1)) {
-    const int bc = k == 0 ? bc_in : bc_out;
-    T w[3];
-    if (mode == 1)
-      for (int c = 0; c < 3; ++c) w[c] = u[c][goff[b] + lo];
-    if (bc == TN_BC_NOSLIP) {
-      for (int c = 0; c < 3; ++c) v[c] += mode == 1 ? w[c] : (T)1;
-    } else {
-      T s[3] = {gs[g], gs[n_groups + g], gs[2 * n_groups + g]};
-      if (mode == 1) {
-        T dot = w[0] * s[0] + w[1] * s[1] + w[2] * s[2];
-        for (int c = 0; c < 3; ++c) v[c] += dot * s[c];
-      } else {
-        for (int c = 0; c < 3; ++c) v[c] += s[c] * s[c];
-      }
-    }
+__device__ __forceinline__ void interface_bc(const Dims& D, const Point& p, const T* gs, int n_groups, int k, int mode,
+                                             const T (&w)[3], int bc_in, int bc_out, T (&v)[3]) {
+  if (mode == 0 || (k != 0 && k != D.n_r - 1)) return;
+  const int bc = k == 0 ? bc_in : bc_out;
+  if (bc == TN_BC_NOSLIP) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) v[c] += mode == 1 ? w[c] : (T)1;
+  } else {
+    const T s[3] = {gs[p.g], gs[n_groups + p.g], gs[2 * n_groups + p.g]};
+    const T dot = w[0] * s[0] + w[1] * s[1] + w[2] * s[2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) v[c] += mode == 1 ? dot * s[c] : s[c] * s[c];
   }
-  for (int q = b; q < e; ++q)
-    for (int c = 0; c < ncomp; ++c) y[c][goff[q] + lo] = v[c];
 }
 
-// Interface sum of K x partials (mode 1: + (I - P) x at boundary layers) followed by the fused
-// vector update of the group's node, written to every copy.
-template <typename T, int EPI>
-__global__ void k_interface_epi(Dims D, int n_groups, const int* __restrict__ gptr, const int64_t* __restrict__ goff,
-                                const T* __restrict__ gs, const T* __restrict__ t0, const T* __restrict__ t1,
-                                const T* __restrict__ t2, const T* __restrict__ x0, const T* __restrict__ x1,
-                                const T* __restrict__ x2, int bc_in, int bc_out, const int* __restrict__ skip,
-                                EpiArgs<T> E) {
+template <typename T, int NC>
+__global__ void __launch_bounds__(128) k_interface(Dims D, int n_edge, const int4* __restrict__ edge, int n_groups,
+                                                   const T* __restrict__ gs, int mode, T* y0, T* y1, T* y2,
+                                                   const T* __restrict__ u0, const T* __restrict__ u1,
+                                                   const T* __restrict__ u2, int bc_in, int bc_out,
+                                                   const int* __restrict__ skip) {
   if (skip && *skip) return;
-  const int g = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;  // grid: groups x layers
-  if (g >= n_groups) return;
-  const T* y[3] = {t0, t1, t2};
-  const T* u[3] = {x0, x1, x2};
-  const int b = gptr[g], e = gptr[g + 1];
-  const int64_t lo = (int64_t)k * D.layer_stride;
-  T v[3] = {0, 0, 0};
-  for (int q = b; q < e; ++q)
-    for (int c = 0; c < 3; ++c) v[c] += y[c][goff[q] + lo];
-  if (k == 0 || k == D.n_r - 1) {
-    const int bc = k == 0 ? bc_in : bc_out;
-    T w[3];
-    for (int c = 0; c < 3; ++c) w[c] = u[c][goff[b] + lo];
-    if (bc == TN_BC_NOSLIP) {
-      for (int c = 0; c < 3; ++c) v[c] += w[c];
-    } else {
-      T s[3] = {gs[g], gs[n_groups + g], gs[2 * n_groups + g]};
-      T dot = w[0] * s[0] + w[1] * s[1] + w[2] * s[2];
-      for (int c = 0; c < 3; ++c) v[c] += dot * s[c];
-    }
+  const int t = blockIdx.x * 128 + threadIdx.x, k = blockIdx.y;  // grid: edge entries x layers
+  const Point p = t < n_edge ? edge_point(edge[t]) : Point{0, 0, 0, 0, 0, 0};
+  const int64_t o = (int64_t)p.d * D.diamond_stride + (int64_t)k * D.layer_stride + p.i * D.P + p.j;
+  T* const y[3] = {y0, y1, y2};
+  T v[3] = {0, 0, 0}, w[3] = {0, 0, 0};
+  if (p.cnt) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) v[c] = y[c][o];
+    if (mode == 1 && (k == 0 || k == D.n_r - 1)) w[0] = u0[o], w[1] = u1[o], w[2] = u2[o];
   }
-  for (int q = b; q < e; ++q) epilogue<T, EPI>(E, x0, x1, x2, (int)(goff[q] + lo), v);
+  copies_sum<T, 3>(p, t & ~31, v);
+  if (!p.cnt) return;
+  interface_bc(D, p, gs, n_groups, k, mode, w, bc_in, bc_out, v);
+#pragma unroll
+  for (int c = 0; c < NC; ++c) y[c][o] = v[c];
+}
+
+// Interface sum of K x partials (+ (I - P) x at the boundary layers) followed by the fused vector update at every copy.
+template <typename T, int EPI>
+__global__ void __launch_bounds__(128) k_interface_epi(Dims D, int n_edge, const int4* __restrict__ edge, int n_groups,
+                                                       const T* __restrict__ gs, const T* __restrict__ t0,
+                                                       const T* __restrict__ t1, const T* __restrict__ t2,
+                                                       const T* __restrict__ x0, const T* __restrict__ x1,
+                                                       const T* __restrict__ x2, int bc_in, int bc_out,
+                                                       const int* __restrict__ skip, EpiArgs<T> E) {
+  if (skip && *skip) return;
+  const int t = blockIdx.x * 128 + threadIdx.x, k = blockIdx.y;  // grid: edge entries x layers
+  const Point p = t < n_edge ? edge_point(edge[t]) : Point{0, 0, 0, 0, 0, 0};
+  const int o = (int)(p.d * D.diamond_stride) + k * (int)D.layer_stride + p.i * D.P + p.j;
+  T v[3] = {0, 0, 0}, w[3] = {0, 0, 0};
+  if (p.cnt) {
+    epi_prefetch<T, EPI>(E, o);
+    v[0] = t0[o], v[1] = t1[o], v[2] = t2[o];
+    if (k == 0 || k == D.n_r - 1) w[0] = x0[o], w[1] = x1[o], w[2] = x2[o];
+  }
+  copies_sum<T, 3>(p, t & ~31, v);
+  if (!p.cnt) return;
+  interface_bc(D, p, gs, n_groups, k, 1, w, bc_in, bc_out, v);
+  epilogue<T, EPI>(E, x0, x1, x2, o, v);
 }
 
 #if TN_PART == 0 || TN_PART == 6
@@ -2072,95 +2134,106 @@ __global__ void k_block_inv(int64_t n, T* b0, T* b1, T* b2, T* b3, T* b4, T* b5)
 // (i/2, (j+1)/2); odd/odd -> midpoint of the coarse anti-diagonal ((i+1)/2, (j-1)/2), ((i-1)/2, (j+1)/2).
 // Semi-coarsened level pairs (lateral factor lf or radial factor rf equal to 1) keep the
 // index in that direction (weight 1).
-template <typename T>
-__global__ void k_prolong(Dims F, Dims C, int lf, int rf, int ncomp, int apply_bc, const T* __restrict__ c0,
+// Every value is the mean of two lateral parents (one twice where the position is a coarse one), then of two radial
+// ones.  ADD: f += P c (the coarse-grid correction).
+template <typename T, int NC, bool ADD>
+__global__ void k_prolong(Dims F, Dims C, int lf, int rf, int apply_bc, const T* __restrict__ c0,
                           const T* __restrict__ c1, const T* __restrict__ c2, T* f0, T* f1, T* f2,
                           const T* __restrict__ svec, int bc_in, int bc_out) {
   const int N = F.N, M = N + 1;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;  // grid: fine lattice points x F.n_r x 10
   if (t >= M * M) return;
   const int i = t / M, j = t - i * M, k = blockIdx.y, d = blockIdx.z;
-  int li[2], lj[2], nl;
-  if (lf == 1 || (!(i & 1) && !(j & 1))) {
-    li[0] = lf == 1 ? i : i / 2, lj[0] = lf == 1 ? j : j / 2, nl = 1;
-  } else if ((i & 1) && !(j & 1)) {
-    li[0] = (i - 1) / 2, lj[0] = j / 2, li[1] = (i + 1) / 2, lj[1] = j / 2, nl = 2;
-  } else if (!(i & 1) && (j & 1)) {
-    li[0] = i / 2, lj[0] = (j - 1) / 2, li[1] = i / 2, lj[1] = (j + 1) / 2, nl = 2;
-  } else {
-    li[0] = (i + 1) / 2, lj[0] = (j - 1) / 2, li[1] = (i - 1) / 2, lj[1] = (j + 1) / 2, nl = 2;
+  int I0 = i, J0 = j, I1 = i, J1 = j, K0 = k, K1 = k;
+  if (lf == 2) {
+    const int oi = i & 1, oj = j & 1;  // odd / odd: the coarse anti-diagonal's midpoint
+    I0 = (i + oi * (2 * oj - 1)) >> 1, J0 = (j - oj) >> 1, I1 = (i + oi * (1 - 2 * oj)) >> 1, J1 = (j + oj) >> 1;
   }
-  int rk[2], nrk;
-  if (rf == 1) rk[0] = k, nrk = 1;
-  else if (!(k & 1)) rk[0] = k / 2, nrk = 1;
-  else rk[0] = (k - 1) / 2, rk[1] = (k + 1) / 2, nrk = 2;
+  if (rf == 2) K0 = k >> 1, K1 = (k + 1) >> 1;
+  const int64_t b0 = (int64_t)d * C.diamond_stride + (int64_t)K0 * C.layer_stride,
+                b1 = (int64_t)d * C.diamond_stride + (int64_t)K1 * C.layer_stride;
+  const int o0 = I0 * C.P + J0, o1 = I1 * C.P + J1;
+  const int64_t idx = (int64_t)d * F.diamond_stride + (int64_t)k * F.layer_stride + (int64_t)i * F.P + j;
   const T* cs[3] = {c0, c1, c2};
   T* fs[3] = {f0, f1, f2};
-  T v[3];
-  for (int c = 0; c < ncomp; ++c) {
-    T rad[2];
-    for (int r = 0; r < nrk; ++r) {
-      const int64_t b = (int64_t)d * C.diamond_stride + (int64_t)rk[r] * C.layer_stride;
-      rad[r] = nl == 1 ? cs[c][b + (int64_t)li[0] * C.P + lj[0]]
-                       : (T)0.5 * (cs[c][b + (int64_t)li[0] * C.P + lj[0]] + cs[c][b + (int64_t)li[1] * C.P + lj[1]]);
-    }
-    v[c] = nrk == 1 ? rad[0] : (T)0.5 * (rad[0] + rad[1]);
+  T v[NC], x[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const T p0 = cs[c][b0 + o0], p1 = cs[c][b0 + o1], q0 = cs[c][b1 + o0], q1 = cs[c][b1 + o1];
+    if (ADD) x[c] = fs[c][idx];
+    v[c] = (T)0.5 * ((T)0.5 * (p0 + p1) + (T)0.5 * (q0 + q1));
   }
-  if (apply_bc && ncomp == 3 && (k == 0 || k == F.n_r - 1))
-    project_vec(v, svec, ((int64_t)d * M + i) * F.P + j, F.n_lat_layout, k == 0 ? bc_in : bc_out);
-  const int64_t idx = (int64_t)d * F.diamond_stride + (int64_t)k * F.layer_stride + (int64_t)i * F.P + j;
-  for (int c = 0; c < ncomp; ++c) fs[c][idx] = v[c];
+  if constexpr (NC == 3) {
+    if (apply_bc && (k == 0 || k == F.n_r - 1))
+      project_vec(v, svec, ((int64_t)d * M + i) * F.P + j, F.n_lat_layout, k == 0 ? bc_in : bc_out);
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) fs[c][idx] = ADD ? x[c] + v[c] : v[c];
 }
 
 // Restriction P^T: coarse node (I, J, K) gathers the fine nodes it interpolates to (semi-coarsened
 // pairs keep the index in the direction with factor 1): lateral
 // (2I, 2J) with weight 1 and its six lattice neighbours with weight 1/2, radial 2K (1) and
 // 2K +- 1 (1/2).  Fine nodes shared by several diamonds are counted by their canonical copy
-// only; the coarse copies are then summed by launch_interface.
-template <typename T>
-__global__ void k_restrict(Dims F, Dims C, int lf, int rf, int ncomp, const uint8_t* __restrict__ owned,
-                           const T* __restrict__ f0, const T* __restrict__ f1, const T* __restrict__ f2, T* c0, T* c1,
-                           T* c2) {
-  const int NC = C.N, MC = NC + 1, NF = F.N, MF = NF + 1;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;  // grid: coarse lattice points x C.n_r x 10
-  if (t >= MC * MC) return;
-  const int I = t / MC, J = t - I * MC, K = blockIdx.y, d = blockIdx.z;
-  const int nb[7][2] = {{0, 0}, {1, 0}, {-1, 0}, {0, 1}, {0, -1}, {1, -1}, {-1, 1}};
+// only; the coarse copies are summed by shuffles (one thread per copy and layer), projected and written.
+template <typename T, int NC>
+__global__ void __launch_bounds__(128)
+    k_restrict(Dims F, Dims C, Points S, int lf, int rf, int apply_bc, const uint8_t* __restrict__ owned,
+               const T* __restrict__ f0, const T* __restrict__ f1, const T* __restrict__ f2, T* c0, T* c1, T* c2,
+               const T* __restrict__ svec, const T* __restrict__ gs, int n_groups, int bc_in, int bc_out) {
+  const int u = blockIdx.x * 128 + threadIdx.x, K = blockIdx.y;  // grid: coarse points (every copy) x C.n_r
+  const Point p = point_at(S, u);
+  const int NF = F.N, MF = NF + 1;
   const T* fs[3] = {f0, f1, f2};
   T* cs[3] = {c0, c1, c2};
-  T v[3] = {0, 0, 0};
-  for (int r = -1; r <= 1; ++r) {
-    if (rf == 1 && r != 0) continue;
-    const int kf = rf * K + r;
-    if (kf < 0 || kf >= F.n_r) continue;
-    const T wr = r == 0 ? (T)1 : (T)0.5;
-    T lat[3] = {0, 0, 0};
-    for (int q = 0; q < (lf == 1 ? 1 : 7); ++q) {
-      const int fi = lf * I + nb[q][0], fj = lf * J + nb[q][1];
-      if (fi < 0 || fj < 0 || fi > NF || fj > NF) continue;
-      if (!owned[((int64_t)d * MF + fi) * F.P + fj]) continue;
-      const T wl = q == 0 ? (T)1 : (T)0.5;
-      const int64_t idx = (int64_t)d * F.diamond_stride + (int64_t)kf * F.layer_stride + (int64_t)fi * F.P + fj;
-      for (int c = 0; c < ncomp; ++c) lat[c] += wl * fs[c][idx];
+  T v[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) v[c] = (T)0;
+  if (p.cnt) {
+    const int fi = lf * p.i, fj = lf * p.j;
+    const int di[7] = {0, 1, -1, 0, 0, 1, -1}, dj[7] = {0, 0, 0, 1, -1, -1, 1};
+    T wl[7];  // lateral weights; 0 where the diamond has no such node or another copy counts
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      const int a = fi + di[q], b = fj + dj[q];
+      bool ok = (q == 0 || lf == 2) && a >= 0 && b >= 0 && a <= NF && b <= NF;
+      if (ok && p.g >= 0) ok = owned[(p.d * MF + a) * F.P + b] != 0;
+      wl[q] = ok ? (q == 0 ? (T)1 : (T)0.5) : (T)0;
     }
-    for (int c = 0; c < ncomp; ++c) v[c] += wr * lat[c];
+#pragma unroll
+    for (int r = -1; r <= 1; ++r) {
+      const int kf = rf * K + r;
+      if ((rf == 1 && r != 0) || kf < 0 || kf >= F.n_r) continue;
+      const int64_t o = (int64_t)p.d * F.diamond_stride + (int64_t)kf * F.layer_stride + fi * F.P + fj;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        T x[7], s = (T)0;
+#pragma unroll
+        for (int q = 0; q < 7; ++q) x[q] = wl[q] != (T)0 ? fs[c][o + di[q] * F.P + dj[q]] : (T)0;
+#pragma unroll
+        for (int q = 0; q < 7; ++q) s += wl[q] * x[q];
+        v[c] += (r == 0 ? (T)1 : (T)0.5) * s;
+      }
+    }
   }
-  const int64_t idx = (int64_t)d * C.diamond_stride + (int64_t)K * C.layer_stride + (int64_t)I * C.P + J;
-  for (int c = 0; c < ncomp; ++c) cs[c][idx] = v[c];
-}
-
-// In-place projection of the boundary layers (after a restriction's interface sum).
-template <typename T>
-__global__ void k_project_bdry(Dims D, T* y0, T* y1, T* y2, const T* __restrict__ svec, int bc_in, int bc_out) {
-  const int M = D.N + 1;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;  // grid: lattice points x 2 layers x 10 diamonds
-  if (t >= M * M) return;
-  const int i = t / M, j = t - i * M, side = blockIdx.y, d = blockIdx.z;
-  const int k = side == 0 ? 0 : D.n_r - 1;
-  const int64_t idx = (int64_t)d * D.diamond_stride + (int64_t)k * D.layer_stride + (int64_t)i * D.P + j;
-  T v[3] = {y0[idx], y1[idx], y2[idx]};
-  project_vec(v, svec, ((int64_t)d * M + i) * D.P + j, D.n_lat_layout, side == 0 ? bc_in : bc_out);
-  y0[idx] = v[0], y1[idx] = v[1], y2[idx] = v[2];
+  copies_sum<T, NC>(p, u & ~31, v);
+  if (!p.cnt) return;
+  if constexpr (NC == 3) {
+    if (apply_bc && (K == 0 || K == C.n_r - 1)) {
+      if ((K == 0 ? bc_in : bc_out) == TN_BC_NOSLIP) {
+        v[0] = v[1] = v[2] = (T)0;
+      } else {
+        T s[3];
+        point_dir(p, gs, n_groups, svec, (int)C.layer_stride, C.P, (int)C.n_lat_layout, s);
+        const T dot = v[0] * s[0] + v[1] * s[1] + v[2] * s[2];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[c] -= dot * s[c];
+      }
+    }
+  }
+  const int64_t idx = (int64_t)p.d * C.diamond_stride + (int64_t)K * C.layer_stride + p.i * C.P + p.j;
+#pragma unroll
+  for (int c = 0; c < NC; ++c) cs[c][idx] = v[c];
 }
 
 // ------------------------------------------------------------------------------------ diag(M_1/eta)
@@ -2319,7 +2392,7 @@ inline bool use_df(const Level& L) {
 // arrays start on 16-byte boundaries; the others take the square tiles.
 inline bool pair32_ok(const Level& L, const float* const* in) {
   auto al = [](const float* p) { return ((uintptr_t)p & 15) == 0; };
-  return TN_PAIR32 && L.quad == 1 && L.N >= 2 * TILE && L.ring64 && L.grp_dij && L.n_layout < (int64_t)INT32_MAX &&
+  return TN_PAIR32 && L.quad == 1 && L.N >= 2 * TILE && L.ring64 && L.n_layout < (int64_t)INT32_MAX &&
          L.n_wedges < (int64_t)INT32_MAX && al(in[0]) && al(in[1]) && al(in[2]);
 }
 
@@ -2349,9 +2422,9 @@ cudaError_t launch_pair32(const Level& L, BC bc, const OpA<float, HG>& op, const
   k_ring4_fix<F, EPI><<<dim3(nblk(RD.RC, 256), L.n_r, 10), 256, 0, st>>>(D, RD, ring, in[0], in[1], in[2], out[0],
                                                                         out[1], out[2], L.s32, bc.in, bc.out, skip, E);
   e = cudaGetLastError();
-  if (e != cudaSuccess || L.n_groups == 0) return e;
-  k_ring4_edges<EPI><<<dim3(nblk(L.n_groups, 128), L.n_r), 128, 0, st>>>(
-      D, RD, L.n_groups, L.grp_ptr, L.grp_off, L.grp_dij, L.grp_s32, ring, in[0], in[1], in[2], out[0], out[1], out[2],
+  if (e != cudaSuccess) return e;
+  k_ring4_edges<EPI><<<dim3(nblk(L.n_edge, 128), L.n_r), 128, 0, st>>>(
+      D, RD, L.n_edge, L.edge, L.n_groups, L.grp_s32, ring, in[0], in[1], in[2], out[0], out[1], out[2],
       bc.in, bc.out, skip, E);
   return cudaGetLastError();
 }
@@ -2506,12 +2579,11 @@ cudaError_t launch_apply_A_epi(const Level& L, BC bc, int div_term, int epi, con
                   : L.hg_kappa > 0 ? apply_A_epi_hg<T, true>(L, bc, div_term, epi, in, E, t, st, skip)
                                    : apply_A_epi_hg<T, false>(L, bc, div_term, epi, in, E, t, st, skip);
   if (e != cudaSuccess) return e;
-  const int64_t n = (int64_t)L.n_groups * L.n_r;
-  if (n == 0) return cudaSuccess;
-  const dim3 nb(nblk(L.n_groups, 128), L.n_r);
+  if (L.n_edge == 0) return cudaSuccess;
+  const dim3 nb(nblk(L.n_edge, 128), L.n_r);
   const Dims D = dims(L);
 #define TN_IEPI(EP)                                                                                             \
-  k_interface_epi<T, EP><<<nb, 128, 0, st>>>(D, L.n_groups, L.grp_ptr, L.grp_off, Tab<T>::gs(L), t[0], t[1], t[2], \
+  k_interface_epi<T, EP><<<nb, 128, 0, st>>>(D, L.n_edge, L.edge, L.n_groups, Tab<T>::gs(L), t[0], t[1], t[2],     \
                                              in[0], in[1], in[2], bc.in, bc.out, skip, E)
   if (epi == EPI_RESID) TN_IEPI(EPI_RESID);
   else if (epi == EPI_CHEB1) TN_IEPI(EPI_CHEB1);
@@ -2621,46 +2693,55 @@ cudaError_t launch_diag_pmass(const Level& F, const Level& C, T* m, cudaStream_t
 template <typename T>
 cudaError_t launch_interface(const Level& L, BC bc, int ncomp, int mode, T* const* y, const T* const* u,
                              cudaStream_t st, const int* skip) {
-  const int64_t n = (int64_t)L.n_groups * L.n_r;
-  if (n == 0) return cudaSuccess;
+  if (L.n_edge == 0) return cudaSuccess;
   T* y1 = ncomp > 1 ? y[1] : y[0];
   T* y2 = ncomp > 2 ? y[2] : y[0];
   const T* u0 = u ? u[0] : nullptr;
   const T* u1 = u ? u[1] : nullptr;
   const T* u2 = u ? u[2] : nullptr;
-  k_interface<T><<<dim3(nblk(L.n_groups, 128), L.n_r), 128, 0, st>>>(dims(L), L.n_groups, L.grp_ptr, L.grp_off,
-                                                                   Tab<T>::gs(L), ncomp, mode,
-                                               y[0], y1, y2, u0, u1, u2, bc.in, bc.out, skip);
+  const dim3 grid(nblk(L.n_edge, 128), L.n_r);
+  if (ncomp == 3)
+    k_interface<T, 3><<<grid, 128, 0, st>>>(dims(L), L.n_edge, L.edge, L.n_groups, Tab<T>::gs(L), mode, y[0], y1, y2, u0,
+                                            u1, u2, bc.in, bc.out, skip);
+  else if (ncomp == 1)
+    k_interface<T, 1><<<grid, 128, 0, st>>>(dims(L), L.n_edge, L.edge, L.n_groups, Tab<T>::gs(L), mode, y[0], y1, y2, u0,
+                                            u1, u2, bc.in, bc.out, skip);
+  else
+    return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_prolong(const Level& F, const Level& C, BC bc, int ncomp, int apply_bc, const T* const* c,
-                           T* const* f, cudaStream_t st) {
-  const T* c1 = ncomp > 1 ? c[1] : c[0];
-  const T* c2 = ncomp > 2 ? c[2] : c[0];
-  T* f1 = ncomp > 1 ? f[1] : f[0];
-  T* f2 = ncomp > 2 ? f[2] : f[0];
+                           T* const* f, cudaStream_t st, bool add) {
   const int lf = F.N / C.N, rf = (F.n_r - 1) / (C.n_r - 1);
-  k_prolong<T><<<dim3(nblk((int64_t)(F.N + 1) * (F.N + 1), 256), F.n_r, 10), 256, 0, st>>>(dims(F), dims(C), lf, rf, ncomp, apply_bc, c[0], c1, c2, f[0], f1, f2,
-                                             Tab<T>::s(F), bc.in, bc.out);
+  const dim3 grid(nblk((int64_t)(F.N + 1) * (F.N + 1), 256), F.n_r, 10);
+#define TN_PROLONG(NC, ADD)                                                                                     \
+  k_prolong<T, NC, ADD><<<grid, 256, 0, st>>>(dims(F), dims(C), lf, rf, apply_bc, c[0], c[NC - 1 < 1 ? 0 : 1],   \
+                                              c[NC - 1], f[0], f[NC - 1 < 1 ? 0 : 1], f[NC - 1], Tab<T>::s(F),   \
+                                              bc.in, bc.out)
+  if (ncomp == 3 && add) TN_PROLONG(3, true);
+  else if (ncomp == 3) TN_PROLONG(3, false);
+  else if (ncomp == 1 && !add) TN_PROLONG(1, false);
+  else return cudaErrorInvalidValue;
+#undef TN_PROLONG
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_restrict(const Level& F, const Level& C, BC bc, int ncomp, int apply_bc, const T* const* f,
                             T* const* c, cudaStream_t st) {
-  const T* f1 = ncomp > 1 ? f[1] : f[0];
-  const T* f2 = ncomp > 2 ? f[2] : f[0];
-  T* c1 = ncomp > 1 ? c[1] : c[0];
-  T* c2 = ncomp > 2 ? c[2] : c[0];
   const int lf = F.N / C.N, rf = (F.n_r - 1) / (C.n_r - 1);
-  k_restrict<T><<<dim3(nblk((int64_t)(C.N + 1) * (C.N + 1), 256), C.n_r, 10), 256, 0, st>>>(dims(F), dims(C), lf, rf, ncomp, F.owned, f[0], f1, f2, c[0], c1, c2);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  e = launch_interface<T>(C, bc, ncomp, 0, c, nullptr, st);
-  if (e != cudaSuccess || !(apply_bc && ncomp == 3)) return e;
-  k_project_bdry<T><<<dim3(nblk((int64_t)(C.N + 1) * (C.N + 1), 256), 2, 10), 256, 0, st>>>(dims(C), c[0], c[1], c[2], Tab<T>::s(C), bc.in, bc.out);
+  const Points S = points_of(C);
+  const dim3 grid(nblk(S.n, 128), C.n_r);
+#define TN_RESTRICT(NC)                                                                                          \
+  k_restrict<T, NC><<<grid, 128, 0, st>>>(dims(F), dims(C), S, lf, rf, apply_bc, F.owned, f[0], f[NC - 1 < 1 ? 0 : 1], \
+                                          f[NC - 1], c[0], c[NC - 1 < 1 ? 0 : 1], c[NC - 1], Tab<T>::s(C),       \
+                                          Tab<T>::gs(C), C.n_groups, bc.in, bc.out)
+  if (ncomp == 3) TN_RESTRICT(3);
+  else if (ncomp == 1) TN_RESTRICT(1);
+  else return cudaErrorInvalidValue;
+#undef TN_RESTRICT
   return cudaGetLastError();
 }
 
@@ -2736,7 +2817,7 @@ cudaError_t launch_buoyancy(const Level& L, BC bc, const double* T, double Ra, d
   template cudaError_t launch_interface<T>(const Level&, BC, int, int, T* const*, const T* const*, cudaStream_t,  \
                                            const int*);                                                          \
   template cudaError_t launch_prolong<T>(const Level&, const Level&, BC, int, int, const T* const*, T* const*,   \
-                                         cudaStream_t);                                                         \
+                                         cudaStream_t, bool);                                                         \
   template cudaError_t launch_restrict<T>(const Level&, const Level&, BC, int, int, const T* const*, T* const*,  \
                                           cudaStream_t);
 TN_INST(double)
@@ -2988,7 +3069,7 @@ cudaError_t small_A(const Level& L, BC bc, const Op& op, int epi, const T* const
   k_small_cell<T, Op><<<nblk(S.ncell, kSmallBlock), kSmallBlock, 0, st>>>(S, B, op, in[0], in[1], in[2], sc);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const unsigned nb = nblk((int64_t)S.n_lat * S.n_r, 128);
+  const dim3 nb(nblk(S.npad, 128), S.n_r);
 #define TN_SMALL_NODE(EP) k_small_node<T, EP><<<nb, 128, 0, st>>>(S, B, in[0], in[1], in[2], sc, y[0], y[1], y[2], E)
   switch (epi) {
     case EPI_NONE: TN_SMALL_NODE(EPI_NONE); break;
@@ -3019,7 +3100,10 @@ cudaError_t cg_cluster(const Level& L, BC bc, const Op& op, const CgArgs<T>& A, 
   at.id = cudaLaunchAttributeClusterDimension;
   at.val.clusterDim.x = kCgCtas, at.val.clusterDim.y = 1, at.val.clusterDim.z = 1;
   cfg.attrs = &at, cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_cg_cluster<T, Op>, small_dims(L), small_tab<T>(L, bc), op, A);
+  const SmallDims S = small_dims(L);
+  if (S.npad * S.n_r <= kCgCtas * kCgThreads)
+    return cudaLaunchKernelEx(&cfg, k_cg_cluster<T, Op, true>, S, small_tab<T>(L, bc), op, A);
+  return cudaLaunchKernelEx(&cfg, k_cg_cluster<T, Op, false>, S, small_tab<T>(L, bc), op, A);
 }
 
 template <typename T>

@@ -453,48 +453,45 @@ __device__ __forceinline__ void ring4_sum(const RingDims& RD, int N, int n_r, co
   }
 }
 
-// Diamond-edge nodes of the paired-cell tiles, one thread per interface group g (the copies of one
-// lattice point) and node layer k: the ring partials of every copy summed, the boundary rows
-// projected and (I - P) u added once, then the value -- or the fused vector update -- at every
-// copy (what k_ring_fix and k_interface do in two passes for the other tiles).
+// Diamond-edge nodes of the paired-cell tiles, one thread per copy and node layer k: the ring partials of the copy's
+// diamond, summed over the copies by shuffles, the boundary rows projected and (I - P) u added once, then the
+// value -- or the fused vector update -- at the copy (what k_ring_fix and k_interface do in two passes for the
+// other tiles).
 template <int EPI>
-__global__ void k_ring4_edges(Dims D, RingDims RD, int n_groups, const int* __restrict__ gptr,
-                              const int64_t* __restrict__ goff, const int4* __restrict__ gdij,
-                              const float* __restrict__ gs, const float4* __restrict__ ring,
-                              const float* __restrict__ in0, const float* __restrict__ in1,
-                              const float* __restrict__ in2, float* __restrict__ out0, float* __restrict__ out1,
-                              float* __restrict__ out2, int bc_in, int bc_out, const int* __restrict__ skip,
-                              EpiArgs<float> E) {
+__global__ void __launch_bounds__(128)
+    k_ring4_edges(Dims D, RingDims RD, int n_edge, const int4* __restrict__ edge, int n_groups,
+                  const float* __restrict__ gs, const float4* __restrict__ ring, const float* __restrict__ in0,
+                  const float* __restrict__ in1, const float* __restrict__ in2, float* __restrict__ out0,
+                  float* __restrict__ out1, float* __restrict__ out2, int bc_in, int bc_out,
+                  const int* __restrict__ skip, EpiArgs<float> E) {
   if (skip && *skip) return;
-  const int g = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;  // grid: groups x layers
-  if (g >= n_groups) return;
+  const int t = blockIdx.x * 128 + threadIdx.x, k = blockIdx.y;  // grid: edge entries x layers
+  const Point p = t < n_edge ? edge_point(edge[t]) : Point{0, 0, 0, 0, 0, 0};
   const int N = D.N, n_r = D.n_r;
-  const int b = gptr[g], e = gptr[g + 1];
-  float v[3] = {0.f, 0.f, 0.f};
-  for (int q = b; q < e; ++q) {
-    const int4 c = gdij[q];
-    ring4_sum(RD, N, n_r, ring, k, c.x, c.y, c.z, v);
+  const int o = (int)(p.d * D.diamond_stride) + k * (int)D.layer_stride + p.i * D.P + p.j;
+  const bool surface = k == 0 || k == n_r - 1;
+  float v[3] = {0.f, 0.f, 0.f}, w[3] = {0.f, 0.f, 0.f};
+  if (p.cnt) {
+    epi_prefetch<float, EPI>(E, o);
+    ring4_sum(RD, N, n_r, ring, k, p.d, p.i, p.j, v);
+    if (surface) w[0] = in0[o], w[1] = in1[o], w[2] = in2[o];
   }
-  const int lo = k * (int)D.layer_stride;
-  if (k == 0 || k == n_r - 1) {
+  copies_sum<float, 3>(p, t & ~31, v);
+  if (!p.cnt) return;
+  if (surface) {
     const int bc = k == 0 ? bc_in : bc_out;
-    const int o = (int)goff[b] + lo;
-    const float w[3] = {in0[o], in1[o], in2[o]};
     if (bc == TN_BC_NOSLIP) {
       for (int c = 0; c < 3; ++c) v[c] = w[c];
     } else {
-      const float s[3] = {gs[g], gs[n_groups + g], gs[2 * n_groups + g]};
+      const float s[3] = {gs[p.g], gs[n_groups + p.g], gs[2 * n_groups + p.g]};
       const float dv = v[0] * s[0] + v[1] * s[1] + v[2] * s[2], dw = w[0] * s[0] + w[1] * s[1] + w[2] * s[2];
       for (int c = 0; c < 3; ++c) v[c] += (dw - dv) * s[c];
     }
   }
-  for (int q = b; q < e; ++q) {
-    const int o = (int)goff[q] + lo;
-    if (EPI != EPI_NONE) {
-      epilogue<float, EPI>(E, in0, in1, in2, o, v);
-    } else {
-      out0[o] = v[0], out1[o] = v[1], out2[o] = v[2];
-    }
+  if (EPI != EPI_NONE) {
+    epilogue<float, EPI>(E, in0, in1, in2, o, v);
+  } else {
+    out0[o] = v[0], out1[o] = v[1], out2[o] = v[2];
   }
 }
 
@@ -520,9 +517,10 @@ __global__ void k_ring4_fix(Dims D, RingDims RD, const float4* __restrict__ ring
   }
   if (i == 0 || i == N || j == 0 || j == N) return;  // diamond edge
   float v[3] = {0.f, 0.f, 0.f};
+  const int idx = (int)(d * D.diamond_stride) + k * (int)D.layer_stride + i * D.P + j;
+  epi_prefetch<float, EPI>(E, idx);
   ring4_sum(RD, N, n_r, ring, k, d, i, j, v);
   const int M = N + 1;
-  const int idx = (int)(d * D.diamond_stride) + k * (int)D.layer_stride + i * D.P + j;
   const int64_t so = ((int64_t)d * M + i) * D.P + j;
   if ((FLAGS & PROJ_OUT) && (k == 0 || k == n_r - 1)) {
     const int bc = k == 0 ? bc_in : bc_out;

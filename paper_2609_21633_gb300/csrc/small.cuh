@@ -4,42 +4,40 @@
 // A streaming tile kernel gives such a level 10 tile columns, each a serial radial sweep: on level 4 / 17
 // layers the FP64 apply ran 20 CTAs on 152 SMs (229 us; 25 us per layer of one SM's FP64 pipe).  Here every
 // cell is its own thread, computed once, and leaves its 24 corner contributions in a scratch array (about
-// 200 bytes per cell, in L2); a second kernel gathers every unique node from the cells around it -- over all
-// diamonds that share it, so there is no interface pass -- and runs the fused vector update at every copy.
+// 200 bytes per cell, in L2); a second kernel gathers every copy of a node from the cells of its diamond, sums the
+// copies by shuffles -- no interface pass -- and runs the fused vector update at every copy.
 // The same two device functions carry the coarsest-level conjugate gradients (k_cg_cluster below).
-// Bound by latency (two dependent launches of a few microseconds), in FP64 by the FP64 pipes.  With the
-// one-launch CG, V-cycles went from (streaming tiles filling the SMs) 1017 to 703 us (FP32, level 4 / 17
-// layers), 3097 to 2772 us (FP32, 6 / 65), 1404 to 1072 us (FP32, two radial points, 5 / 33) and 3999 to 2816 us
-// (FP64, 5 / 33).
+// Bound by latency (two dependent launches of a few microseconds), in FP64 by the FP64 pipes (a cell's chain of
+// about 265 instructions at 64 cycles each on an SM partition).  V-cycles went from (streaming tiles filling the SMs) 1017
+// to 366 us (FP32, level 4 / 17 layers), 1404 to 647 us (FP32, two radial points, 5 / 33) and 3999 to 1756 us (FP64,
+// 5 / 33); a thread per group that walks its copies, instead of one per copy, left them at 703, 1072 and 2816 us.
 // Sums run in a fixed order (copies in ascending layout order; corners 00, 10, 01, 11; bottom then top
 // contributions), so results do not depend on scheduling.
 
-// Index data of a small level: unique lateral points are the interface groups first, then the points inside
-// the diamonds.
 struct SmallDims {
   int N, n_r, P, ls, ds, nll;  // ls / ds: layer / diamond stride of the node layout, nll: lateral layout size
-  int n_groups, n_lat, ncell;  // interface groups, unique lateral points, cells
-  const int* gptr;
-  const int64_t* goff;
+  int ncell, npad, n_groups;   // cells, lateral points (every copy) rounded up to whole warps, interface groups
+  Points pts;
 };
 inline SmallDims small_dims(const Level& L) {
   SmallDims s;
   s.N = L.N, s.n_r = L.n_r, s.P = L.P, s.ls = (int)L.layer_stride, s.ds = (int)L.diamond_stride;
   s.nll = (int)L.n_lat_layout;
-  s.n_groups = L.n_groups, s.n_lat = 10 * L.N * L.N + 2, s.ncell = 10 * L.N * L.N * (L.n_r - 1);
-  s.gptr = L.grp_ptr, s.goff = L.grp_off;
+  s.ncell = 10 * L.N * L.N * (L.n_r - 1);
+  s.pts = points_of(L);
+  s.npad = (s.pts.n + 31) / 32 * 32, s.n_groups = L.n_groups;
   return s;
 }
 
 template <typename T>
 struct SmallTab {  // tables of the level in its precision
-  const T *geo, *lay, *svec;
+  const T *geo, *lay, *svec, *gs;
   EtaView<T> eta;
   int bc_in, bc_out;
 };
 template <typename T>
 inline SmallTab<T> small_tab(const Level& L, BC bc) {
-  return SmallTab<T>{Tab<T>::geo(L), Tab<T>::lay(L), Tab<T>::s(L), etav<T>(L), bc.in, bc.out};
+  return SmallTab<T>{Tab<T>::geo(L), Tab<T>::lay(L), Tab<T>::s(L), Tab<T>::gs(L), etav<T>(L), bc.in, bc.out};
 }
 
 // Contributions of cell c = ((d (n_r - 1) + k) N + i) N + j to its eight nodes: bottom corner q, component x
@@ -110,52 +108,31 @@ __device__ __forceinline__ void small_gather(const SmallDims& S, const T* __rest
     v[x] += ((a[0][x] + a[1][x]) + (a[2][x] + a[3][x])) + ((a[4][x] + a[5][x]) + (a[6][x] + a[7][x]));
 }
 
-// Copies of unique lateral point u: count and, for copy q, (d, i, j).
-__device__ __forceinline__ void small_copies(const SmallDims& S, int u, int& b, int& e) {
-  if (u < S.n_groups) b = S.gptr[u], e = S.gptr[u + 1];
-  else b = 0, e = 1;
-}
-__device__ __forceinline__ void small_copy(const SmallDims& S, int u, int q, int& d, int& i, int& j) {
-  if (u < S.n_groups) {
-    const int off = (int)S.goff[q];
-    d = off / S.ds;
-    const int r = off - d * S.ds;
-    i = r / S.P, j = r - i * S.P;
-  } else {
-    const int w = u - S.n_groups, n1 = S.N - 1, per = n1 * n1;
-    d = w / per;
-    const int r = w - d * per;
-    i = r / n1 + 1, j = r - (i - 1) * n1 + 1;
-  }
-}
-
-// y = (P A P + I - P) in at unique node (u, k) from the cells' contributions; o0: the layout offset of its
-// first copy (the canonical one).
+// y = (P A P + I - P) in at node layer k of point p from the cells' contributions, the same at every copy; o: the
+// copy's layout offset, u: its warp's first point.  All lanes of the warp call it.
 template <typename T, bool CG>
 __device__ __forceinline__ void small_node(const SmallDims& S, const SmallTab<T>& B, const T* const (&in)[3],
-                                           const T* __restrict__ sc, int u, int k, T (&v)[3], int& o0) {
-  int b, e;
-  small_copies(S, u, b, e);
+                                           const T* __restrict__ sc, const Point& p, int u, int k, int o, T (&v)[3]) {
   v[0] = v[1] = v[2] = (T)0;
-  int lat0 = 0;
-  for (int q = b; q < e; ++q) {
-    int d, i, j;
-    small_copy(S, u, q, d, i, j);
-    if (q == b) lat0 = d * S.ls + i * S.P + j, o0 = d * S.ds + k * S.ls + i * S.P + j;
-    small_gather(S, sc, d, i, j, k, v);
-  }
-  if (k == 0 || k == S.n_r - 1) {
-    const int bc = k == 0 ? B.bc_in : B.bc_out;
-    T w[3];
+  T w[3] = {0, 0, 0};
+  const bool surface = k == 0 || k == S.n_r - 1;
+  if (p.cnt) {
+    if (surface)
 #pragma unroll
-    for (int x = 0; x < 3; ++x) w[x] = CG ? __ldcg(in[x] + o0) : in[x][o0];
-    if (bc == TN_BC_NOSLIP) {
+      for (int x = 0; x < 3; ++x) w[x] = CG ? __ldcg(in[x] + o) : in[x][o];
+    small_gather(S, sc, p.d, p.i, p.j, k, v);
+  }
+  copies_sum<T, 3>(p, u, v);
+  if (surface && p.cnt) {
+    if ((k == 0 ? B.bc_in : B.bc_out) == TN_BC_NOSLIP) {
 #pragma unroll
       for (int x = 0; x < 3; ++x) v[x] = w[x];
     } else {
-      const T sx = B.svec[lat0], sy = B.svec[lat0 + S.nll], sz = B.svec[lat0 + 2 * S.nll];
-      const T dv = (w[0] - v[0]) * sx + (w[1] - v[1]) * sy + (w[2] - v[2]) * sz;
-      v[0] += dv * sx, v[1] += dv * sy, v[2] += dv * sz;
+      T s[3];
+      point_dir(p, B.gs, S.n_groups, B.svec, S.ls, S.P, S.nll, s);
+      const T dv = (w[0] - v[0]) * s[0] + (w[1] - v[1]) * s[1] + (w[2] - v[2]) * s[2];
+#pragma unroll
+      for (int x = 0; x < 3; ++x) v[x] += dv * s[x];
     }
   }
 }
@@ -178,31 +155,28 @@ __global__ void __launch_bounds__(128) k_small_node(SmallDims S, SmallTab<T> B, 
                                                     const T* __restrict__ in1, const T* __restrict__ in2,
                                                     const T* __restrict__ sc, T* __restrict__ out0, T* __restrict__ out1,
                                                     T* __restrict__ out2, EpiArgs<T> E) {
-  const int t = blockIdx.x * 128 + threadIdx.x;
-  if (t >= S.n_lat * S.n_r) return;
-  const int k = t / S.n_lat, u = t - k * S.n_lat;
+  const int u = blockIdx.x * 128 + threadIdx.x, k = blockIdx.y;  // grid: points x layers
+  const Point p = point_at(S.pts, u);
   const T* const in[3] = {in0, in1, in2};
+  const int o = p.d * S.ds + k * S.ls + p.i * S.P + p.j;
+  if (p.cnt) epi_prefetch<T, EPI>(E, o);
   T v[3];
-  int o0;
-  small_node<T, false>(S, B, in, sc, u, k, v, o0);
-  int b, e;
-  small_copies(S, u, b, e);
-  for (int q = b; q < e; ++q) {
-    const int o = u < S.n_groups ? (int)S.goff[q] + k * S.ls : o0;
-    if (EPI != EPI_NONE) {
-      epilogue<T, EPI>(E, in0, in1, in2, o, v);
-    } else {
-      out0[o] = v[0], out1[o] = v[1], out2[o] = v[2];
-    }
+  small_node<T, false>(S, B, in, sc, p, u & ~31, k, o, v);
+  if (!p.cnt) return;
+  if (EPI != EPI_NONE) {
+    epilogue<T, EPI>(E, in0, in1, in2, o, v);
+  } else {
+    out0[o] = v[0], out1[o] = v[1], out2[o] = v[2];
   }
 }
 
 // ---------------------------------------------------------------- coarsest-level conjugate gradients
 // The whole block-Jacobi-preconditioned CG of the coarsest level (Sec. 7) in one launch of one cluster of
 // eight CTAs: the kernel-per-step form took three launches per step, about 150 in a captured V-cycle, each
-// of them a few microseconds of latency for a level of some hundred nodes.  Unique node t = k n_lat + u
-// belongs to one thread throughout; its r, z, x live at its canonical layout entry, p at every copy.  Cells
-// and nodes go round the CTAs warp by warp; data of other SMs is read past L1 after a cluster
+// of them a few microseconds of latency for a level of some hundred nodes.  Every copy of a node has its thread,
+// which keeps the copy's r, z, x, p (the copies of a node compute the same bits; the first one counts in the inner
+// products): in registers when the level has at most one node per thread, else in memory.  Cells and nodes go
+// round the CTAs warp by warp; data of other SMs (p, the cells' contributions) is read past L1 after a cluster
 // barrier (release / acquire).  Sums: a thread's products in FP64, then warps, CTA and the eight CTAs in a
 // fixed order, every thread the same result, so the stopping test is uniform.
 constexpr int kCgCtas = 8, kCgThreads = 256;
@@ -219,7 +193,7 @@ struct CgArgs {
   int maxit, project;
 };
 
-template <typename T, typename Op>
+template <typename T, typename Op, bool ONE>
 __global__ void __launch_bounds__(kCgThreads) k_cg_cluster(SmallDims S, SmallTab<T> B, Op op, CgArgs<T> A) {
   namespace cgr = cooperative_groups;
   cgr::cluster_group cl = cgr::this_cluster();
@@ -227,7 +201,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_cluster(SmallDims S, SmallTab
   const int rank = (int)cl.block_rank();
   const int gt = (((int)threadIdx.x >> 5) * kCgCtas + rank) * 32 + ((int)threadIdx.x & 31);
   constexpr int GT = kCgCtas * kCgThreads;
-  const int nn = S.n_lat * S.n_r;
+  const int nn = S.npad * S.n_r;  // a multiple of 32: warps enter the loops over nodes whole
   int par = 0;
   // sum of up to three values over the cluster; ends with a cluster barrier, which also publishes global writes
   auto total = [&](double (&a)[3], int n) {
@@ -254,73 +228,96 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_cluster(SmallDims S, SmallTab
     }
     par ^= 1;  // the next sum's remote writes go to the other buffer: it is read two barriers later
   };
-  auto first = [&](int t, int& o, int& lat, int& k) {  // canonical entry of unique node t
-    k = t / S.n_lat;
-    const int u = t - k * S.n_lat;
-    int b, e, d, i, j;
-    small_copies(S, u, b, e);
-    small_copy(S, u, b, d, i, j);
-    lat = d * S.ls + i * S.P + j, o = lat + d * (S.ds - S.ls) + k * S.ls;
+  // a thread's node: copy, layer, offsets, and its vectors (registers when ONE)
+  struct Node {
+    Point p;
+    int u, k, o;
+    T x[3], r[3], z[3], q[3], b[6], d[3];  // q: search direction; b: D^-1; d: unit direction times the radius
   };
-  auto put = [&](int t, const T (&v)[3], T* const (&dst)[3]) {  // to every copy
-    const int k = t / S.n_lat, u = t - k * S.n_lat;
-    int b, e;
-    small_copies(S, u, b, e);
-    for (int q = b; q < e; ++q) {
-      int d, i, j;
-      small_copy(S, u, q, d, i, j);
-      const int o = d * S.ds + k * S.ls + i * S.P + j;
+  Node one;
+  auto locate = [&](int t, Node& n) {
+    n.k = t / S.npad, n.u = t - n.k * S.npad;
+    n.p = point_at(S.pts, n.u);
+    n.o = n.p.d * S.ds + n.k * S.ls + n.p.i * S.P + n.p.j;
+    if (!n.p.cnt) return;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) dst[c][o] = v[c];
+    for (int q = 0; q < 6; ++q) n.b[q] = A.binv[q][n.o];
+    if (A.project) {
+      T s[3];
+      point_dir(n.p, B.gs, S.n_groups, B.svec, S.ls, S.P, S.nll, s);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) n.d[c] = s[c];
     }
   };
-  auto bmul3 = [&](int o, const T (&r)[3], T (&z)[3]) {
-    const T a = A.binv[0][o], e = A.binv[1][o], f = A.binv[2][o], xy = A.binv[3][o], xz = A.binv[4][o], yz = A.binv[5][o];
-    z[0] = a * r[0] + xy * r[1] + xz * r[2];
-    z[1] = xy * r[0] + e * r[1] + yz * r[2];
-    z[2] = xz * r[0] + yz * r[1] + f * r[2];
+  auto load = [&](T* const (&a)[3], const Node& n, T (&v)[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) v[c] = a[c][n.o];
   };
-  // rotation component: w = Ginv (sum over unique nodes of x cross v), removed as v - w cross x
-  auto spin = [&](const T* const (&v)[3], double (&w)[3]) {
-    double a[3] = {0, 0, 0};
-    for (int t = gt; t < nn; t += GT) {
-      int o, lat, k;
-      first(t, o, lat, k);
-      const double r = A.rad[k];
-      const double x[3] = {r * B.svec[lat], r * B.svec[lat + S.nll], r * B.svec[lat + 2 * S.nll]};
-      const double y[3] = {v[0][o], v[1][o], v[2][o]};
-      a[0] += x[1] * y[2] - x[2] * y[1];
-      a[1] += x[2] * y[0] - x[0] * y[2];
-      a[2] += x[0] * y[1] - x[1] * y[0];
+  auto store = [&](T* const (&a)[3], const Node& n, const T (&v)[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a[c][n.o] = v[c];
+  };
+  // f over this thread's nodes (whole warps, unused lanes with cnt = 0)
+  auto each = [&](auto&& f) {
+    if constexpr (ONE) {
+      if (gt < nn) f(one);
+    } else {
+      for (int t = gt; t < nn; t += GT) {
+        Node n;
+        locate(t, n);
+        f(n);
+      }
     }
+  };
+  auto counts = [&](const Node& n) { return n.p.cnt > 0 && n.p.lane == 0; };
+  auto bmul3 = [&](const Node& n, const T (&r)[3], T (&z)[3]) {
+    z[0] = n.b[0] * r[0] + n.b[3] * r[1] + n.b[4] * r[2];
+    z[1] = n.b[3] * r[0] + n.b[1] * r[1] + n.b[5] * r[2];
+    z[2] = n.b[4] * r[0] + n.b[5] * r[1] + n.b[2] * r[2];
+  };
+  // rotation component w = Ginv (sum over nodes of x cross v), removed as v - w cross x
+  auto spin = [&](const Node& n, const T (&v)[3], double (&a)[3]) {
+    const double r = A.rad[n.k], x[3] = {r * n.d[0], r * n.d[1], r * n.d[2]}, y[3] = {v[0], v[1], v[2]};
+    a[0] += x[1] * y[2] - x[2] * y[1];
+    a[1] += x[2] * y[0] - x[0] * y[2];
+    a[2] += x[0] * y[1] - x[1] * y[0];
+  };
+  auto omega = [&](double (&a)[3], double (&w)[3]) {
     total(a, 3);
     for (int c = 0; c < 3; ++c) w[c] = A.ginv[3 * c] * a[0] + A.ginv[3 * c + 1] * a[1] + A.ginv[3 * c + 2] * a[2];
   };
-  auto despin = [&](int lat, int k, const double (&w)[3], T (&v)[3]) {
-    const double r = A.rad[k];
-    const double x[3] = {r * B.svec[lat], r * B.svec[lat + S.nll], r * B.svec[lat + 2 * S.nll]};
+  auto despin = [&](const Node& n, const double (&w)[3], T (&v)[3]) {
+    const double r = A.rad[n.k], x[3] = {r * n.d[0], r * n.d[1], r * n.d[2]};
     v[0] -= (T)(w[1] * x[2] - w[2] * x[1]);
     v[1] -= (T)(w[2] * x[0] - w[0] * x[2]);
     v[2] -= (T)(w[0] * x[1] - w[1] * x[0]);
   };
 
-  double w[3] = {0, 0, 0}, acc[3];
-  const T* const bb[3] = {A.b0, A.b1, A.b2};
-  if (A.project) spin(bb, w);
+  if constexpr (ONE)
+    if (gt < nn) locate(gt, one);
+  double w[3] = {0, 0, 0}, acc[3] = {0, 0, 0};
+  if (A.project) {
+    each([&](Node& n) {
+      if (!counts(n)) return;
+      const T b[3] = {A.b0[n.o], A.b1[n.o], A.b2[n.o]};
+      spin(n, b, acc);
+    });
+    omega(acc, w);
+  }
   // r = b (rotations removed), z = D^-1 r, p = z, x = 0
   acc[0] = 0.0;
-  for (int t = gt; t < nn; t += GT) {
-    int o, lat, k;
-    first(t, o, lat, k);
-    T r[3] = {A.b0[o], A.b1[o], A.b2[o]}, z[3];
-    if (A.project) despin(lat, k, w, r);
-    bmul3(o, r, z);
+  each([&](Node& n) {
+    if (!n.p.cnt) return;
+    n.r[0] = A.b0[n.o], n.r[1] = A.b1[n.o], n.r[2] = A.b2[n.o];
+    if (A.project) despin(n, w, n.r);
+    bmul3(n, n.r, n.z);
     T d = (T)0;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) A.r[c][o] = r[c], A.x[c][o] = (T)0, d += r[c] * z[c];
-    acc[0] += (double)d;
-    put(t, z, A.p);
-  }
+    for (int c = 0; c < 3; ++c) n.x[c] = (T)0, n.q[c] = n.z[c], d += n.r[c] * n.z[c];
+    if (counts(n)) acc[0] += (double)d;
+    store(A.p, n, n.q);
+    if (!ONE) store(A.r, n, n.r), store(A.x, n, n.x);
+  });
   total(acc, 1);
   const double rz0 = acc[0];
   double rz = rz0;
@@ -329,60 +326,61 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_cluster(SmallDims S, SmallTab
     for (int it = 0; it < A.maxit; ++it) {
       for (int c = gt; c < S.ncell; c += GT) small_cell<T, Op, true>(S, B, op, pp, c, A.sc);
       cl.sync();
-      // q = K p, kept in z until the update
       acc[0] = 0.0;
-      for (int t = gt; t < nn; t += GT) {
-        T q[3];
-        int o;
-        small_node<T, true>(S, B, pp, A.sc, t % S.n_lat, t / S.n_lat, q, o);
+      each([&](Node& n) {  // z holds q = K p until the update
+        small_node<T, true>(S, B, pp, A.sc, n.p, n.u & ~31, n.k, n.o, n.z);
+        if (!n.p.cnt) return;
+        if (!ONE) load(A.p, n, n.q), store(A.z, n, n.z);
         T d = (T)0;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) A.z[c][o] = q[c], d += A.p[c][o] * q[c];
-        acc[0] += (double)d;
-      }
+        for (int c = 0; c < 3; ++c) d += n.q[c] * n.z[c];
+        if (counts(n)) acc[0] += (double)d;
+      });
       total(acc, 1);
       const T al = (T)(rz / acc[0]);
       acc[0] = 0.0;
-      for (int t = gt; t < nn; t += GT) {
-        int o, lat, k;
-        first(t, o, lat, k);
-        T r[3], z[3], d = (T)0;
+      each([&](Node& n) {
+        if (!n.p.cnt) return;
+        if (!ONE) load(A.x, n, n.x), load(A.r, n, n.r), load(A.p, n, n.q), load(A.z, n, n.z);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          A.x[c][o] += al * A.p[c][o];
-          r[c] = A.r[c][o] - al * A.z[c][o];
-          A.r[c][o] = r[c];
-        }
-        bmul3(o, r, z);
+        for (int c = 0; c < 3; ++c) n.x[c] += al * n.q[c], n.r[c] -= al * n.z[c];
+        bmul3(n, n.r, n.z);
+        T d = (T)0;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) A.z[c][o] = z[c], d += r[c] * z[c];
-        acc[0] += (double)d;
-      }
+        for (int c = 0; c < 3; ++c) d += n.r[c] * n.z[c];
+        if (counts(n)) acc[0] += (double)d;
+        if (!ONE) store(A.x, n, n.x), store(A.r, n, n.r), store(A.z, n, n.z);
+      });
       total(acc, 1);
       const double rzn = acc[0];
       if (!(rzn > A.tol2 * rz0) || it == A.maxit - 1) break;
       const T be = (T)(rzn / rz);
       rz = rzn;
-      for (int t = gt; t < nn; t += GT) {
-        int o, lat, k;
-        first(t, o, lat, k);
-        T p[3];
+      each([&](Node& n) {
+        if (!n.p.cnt) return;
+        if (!ONE) load(A.p, n, n.q), load(A.z, n, n.z);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) p[c] = A.z[c][o] + be * A.p[c][o];
-        put(t, p, A.p);
-      }
+        for (int c = 0; c < 3; ++c) n.q[c] = n.z[c] + be * n.q[c];
+        store(A.p, n, n.q);
+      });
       cl.sync();
     }
   }
-  // x (rotations removed) to every copy
-  const T* const xx[3] = {A.x[0], A.x[1], A.x[2]};
-  if (A.project) spin(xx, w);
-  for (int t = gt; t < nn; t += GT) {
-    int o, lat, k;
-    first(t, o, lat, k);
-    T x[3] = {A.x[0][o], A.x[1][o], A.x[2][o]};
-    if (A.project) despin(lat, k, w, x);
-    put(t, x, A.x);
+  // x (rotations removed)
+  acc[0] = acc[1] = acc[2] = 0.0;
+  if (A.project) {
+    each([&](Node& n) {
+      if (!counts(n)) return;
+      if (!ONE) load(A.x, n, n.x);
+      spin(n, n.x, acc);
+    });
+    omega(acc, w);
   }
+  each([&](Node& n) {
+    if (!n.p.cnt) return;
+    if (!ONE) load(A.x, n, n.x);
+    if (A.project) despin(n, w, n.x);
+    store(A.x, n, n.x);
+  });
   cl.sync();  // no CTA leaves while another may still write its shared memory
 }

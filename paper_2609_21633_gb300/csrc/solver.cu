@@ -760,9 +760,7 @@ void vcycle_level(MGState* m, const tn_mesh* mesh, int h, cudaStream_t st) {
   }
   ck(launch_restrict<T>(F, Lc, bc, 3, 1, G.r.cc(), C.b.mm(), st));
   vcycle_level<T>(m, mesh, h + 1, st);
-  ck(launch_prolong<T>(F, Lc, bc, 3, 1, C.x().cc(), G.t.mm(), st));
-  k_axpby<T><<<nb(n), EB, 0, st>>>(n, 3, 1.0, P4<T>(G.t.cc(), 3), 1.0, M4<T>(G.x().mm(), 3));
-  ckl();
+  ck(launch_prolong<T>(F, Lc, bc, 3, 1, C.x().cc(), G.x().mm(), st, true));
   for (int s = 0; s < m->opts.post_smooth; ++s) cheb_step<T>(m, mesh, h, false, st);
 }
 
