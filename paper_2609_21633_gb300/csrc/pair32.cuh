@@ -386,6 +386,23 @@ __global__ void __launch_bounds__(kPThreads, 2)
       if (w == 7) ring_put(kn, 0, rrow0 + (N + 1) + 1, r2);
     }
   };
+  // L2 prefetch of the fused update's operands, one layer ahead of their use (L1 has no room beside the staging):
+  // lane a of a warp takes array a of the update's kNa for the warp's upper row, lane kNa + a for the lower one
+  constexpr int kNa = EPI == EPI_CHEB2 ? 12 : EPI == EPI_CHEB1 ? 9 : 3;
+  const float* pf = nullptr;
+  if (EPI != EPI_NONE && lane < 2 * kNa) {
+    const int a = lane % kNa;
+    if (EPI == EPI_CHEB2) pf = a < 3 ? E.r[a] : a < 6 ? E.xacc[a - 3] : E.binv[a - 6];
+    else pf = a < 3 ? E.b[a] : E.binv[a - 3];
+    pf += dbase + (i0 + 2 * w + lane / kNa) * P + j0;
+  }
+  auto prefetch_layer = [&](int kn) {
+    if (EPI != EPI_NONE && lane < 2 * kNa) {
+      const float* q = pf + (int64_t)kn * LS;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(q));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(q + 31));
+    }
+  };
   // one cell layer: cin holds the top contributions of cell layer k - 1 to node layer k, cout
   // receives those of cell layer k to node layer k + 1
   auto step = [&](int k, const float2 (&cin)[4][3], float2 (&cout)[4][3]) {
@@ -396,6 +413,7 @@ __global__ void __launch_bounds__(kPThreads, 2)
     // the buffer of layer k + kPAhead last held layer k - 1, read by every thread before the
     // previous barrier
     issue(k + kPAhead);
+    if (k + 1 < n_r) prefetch_layer(k + 1);
     float2 bq[4][3];
     pair_cell<HG>(tp, bt, gc, lct[k - kstart], e, op.div_term, op.hgk, bq, cout);
     cp_async_wait<kPAhead - 2>();  // layer k + 2 is in (made visible by the next barrier)
