@@ -199,12 +199,12 @@ struct EpiArgs {
 template <typename T>
 cudaError_t launch_apply_A_epi(const Level& L, BC bc, int div_term, int epi, const T* const* in, const EpiArgs<T>& E,
                                T* const* t, cudaStream_t st, const int* skip = nullptr);
-// A apply of a coarse multigrid level (N <= 16) through a scratch array of the cells' contributions
+// A apply of a coarse multigrid level (N <= 16) through a scratch array of the wedges' contributions
 // (small.cuh), with one of the fused updates or (EPI_NONE) to y; `scratch` holds small_scratch_entries(L)
 // values and belongs to the caller: calls that share it must not overlap.
 inline bool small_level(const Level& L) { return L.N <= 16 && L.n_layout < ((int64_t)1 << 26); }
 inline int64_t small_scratch_entries(const Level& L) {
-  return small_level(L) ? (int64_t)24 * 10 * L.N * L.N * (L.n_r - 1) : 0;
+  return small_level(L) ? (int64_t)36 * 10 * L.N * L.N * (L.n_r - 1) : 0;
 }
 template <typename T>
 cudaError_t launch_small_A(const Level& L, BC bc, int div_term, int epi, const T* const* in, const EpiArgs<T>& E,

@@ -3061,12 +3061,27 @@ TN_INST_SADDLE(double)
 TN_INST_SADDLE(float)
 #undef TN_INST_SADDLE
 
-template <typename T, typename Op>
-cudaError_t small_A(const Level& L, BC bc, const Op& op, int epi, const T* const* in, const EpiArgs<T>& E, T* const* y,
-                    T* sc, cudaStream_t st) {
-  const SmallDims S = small_dims(L);
+template <typename T>
+cudaError_t launch_small_A(const Level& L, BC bc, int div_term, int epi, const T* const* in, const EpiArgs<T>& E,
+                           T* const* y, T* sc, cudaStream_t st) {
+  if (!small_level(L)) return cudaErrorInvalidValue;
+  const SmallDims S = small_dims(L, div_term, hg_coef(L, div_term));
   const SmallTab<T> B = small_tab<T>(L, bc);
-  k_small_cell<T, Op><<<nblk(S.ncell, kSmallBlock), kSmallBlock, 0, st>>>(S, B, op, in[0], in[1], in[2], sc);
+  if constexpr (kSmallWedges<T>) {
+    const unsigned nw = nblk(nblk(2 * (int64_t)S.ncell, 10) * (int64_t)32, kSmallBlock);
+    if (L.quad == 2) k_small_wedge<T, false, true><<<nw, kSmallBlock, 0, st>>>(S, B, in[0], in[1], in[2], sc);
+    else if (L.hg_kappa > 0) k_small_wedge<T, true, false><<<nw, kSmallBlock, 0, st>>>(S, B, in[0], in[1], in[2], sc);
+    else k_small_wedge<T, false, false><<<nw, kSmallBlock, 0, st>>>(S, B, in[0], in[1], in[2], sc);
+  } else {
+    const unsigned nc = nblk(S.ncell, kSmallBlock);
+#define TN_SMALL_CELL(HG, Q2)                                                                                  \
+  k_small_cell<T, decltype(SmallOp<T, HG, Q2>::make(S))><<<nc, kSmallBlock, 0, st>>>(S, B, SmallOp<T, HG, Q2>::make(S), \
+                                                                                    in[0], in[1], in[2], sc)
+    if (L.quad == 2) TN_SMALL_CELL(false, true);
+    else if (L.hg_kappa > 0) TN_SMALL_CELL(true, false);
+    else TN_SMALL_CELL(false, false);
+#undef TN_SMALL_CELL
+  }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const dim3 nb(nblk(S.npad, 128), S.n_r);
@@ -3082,28 +3097,18 @@ cudaError_t small_A(const Level& L, BC bc, const Op& op, int epi, const T* const
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_small_A(const Level& L, BC bc, int div_term, int epi, const T* const* in, const EpiArgs<T>& E,
-                           T* const* y, T* sc, cudaStream_t st) {
-  if (!small_level(L)) return cudaErrorInvalidValue;
-  const T hgk = (T)hg_coef(L, div_term);
-  if (L.quad == 2) return small_A<T>(L, bc, OpA2<T>{div_term}, epi, in, E, y, sc, st);
-  if (L.hg_kappa > 0) return small_A<T>(L, bc, OpA<T, true>{div_term, hgk}, epi, in, E, y, sc, st);
-  return small_A<T>(L, bc, OpA<T, false>{div_term, hgk}, epi, in, E, y, sc, st);
-}
-
-template <typename T, typename Op>
-cudaError_t cg_cluster(const Level& L, BC bc, const Op& op, const CgArgs<T>& A, cudaStream_t st) {
+template <typename T, bool HG, bool Q2>
+cudaError_t cg_cluster(const Level& L, BC bc, int div_term, const CgArgs<T>& A, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(kCgCtas), cfg.blockDim = dim3(kCgThreads), cfg.stream = st;
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
   at.val.clusterDim.x = kCgCtas, at.val.clusterDim.y = 1, at.val.clusterDim.z = 1;
   cfg.attrs = &at, cfg.numAttrs = 1;
-  const SmallDims S = small_dims(L);
+  const SmallDims S = small_dims(L, div_term, hg_coef(L, div_term));
   if (S.npad * S.n_r <= kCgCtas * kCgThreads)
-    return cudaLaunchKernelEx(&cfg, k_cg_cluster<T, Op, true>, S, small_tab<T>(L, bc), op, A);
-  return cudaLaunchKernelEx(&cfg, k_cg_cluster<T, Op, false>, S, small_tab<T>(L, bc), op, A);
+    return cudaLaunchKernelEx(&cfg, k_cg_cluster<T, HG, Q2, true>, S, small_tab<T>(L, bc), A);
+  return cudaLaunchKernelEx(&cfg, k_cg_cluster<T, HG, Q2, false>, S, small_tab<T>(L, bc), A);
 }
 
 template <typename T>
@@ -3117,10 +3122,9 @@ cudaError_t launch_coarse_cg(const Level& L, BC bc, int div_term, const T* const
   A.rad = sizeof(T) == 8 ? (const T*)L.rad64 : (const T*)L.rad32;
   A.sc = C.scratch, A.tol2 = C.tol2, A.maxit = C.maxit, A.project = C.project;
   for (int q = 0; q < 9; ++q) A.ginv[q] = C.ginv[q];
-  const T hgk = (T)hg_coef(L, div_term);
-  if (L.quad == 2) return cg_cluster<T>(L, bc, OpA2<T>{div_term}, A, st);
-  if (L.hg_kappa > 0) return cg_cluster<T>(L, bc, OpA<T, true>{div_term, hgk}, A, st);
-  return cg_cluster<T>(L, bc, OpA<T, false>{div_term, hgk}, A, st);
+  if (L.quad == 2) return cg_cluster<T, false, true>(L, bc, div_term, A, st);
+  if (L.hg_kappa > 0) return cg_cluster<T, true, false>(L, bc, div_term, A, st);
+  return cg_cluster<T, false, false>(L, bc, div_term, A, st);
 }
 
 #define TN_INST_SMALL(T)                                                                                          \

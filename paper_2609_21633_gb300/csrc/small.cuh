@@ -1,31 +1,35 @@
-// A apply on the coarse multigrid levels (N <= 16), cell-parallel (included by kernels.cu inside its
+// A apply on the coarse multigrid levels (N <= 16), element-parallel (included by kernels.cu inside its
 // namespace, after the element ops, the epilogue and project_vec).
 //
 // A streaming tile kernel gives such a level 10 tile columns, each a serial radial sweep: on level 4 / 17
 // layers the FP64 apply ran 20 CTAs on 152 SMs (229 us; 25 us per layer of one SM's FP64 pipe).  Here every
-// cell is its own thread, computed once, and leaves its 24 corner contributions in a scratch array (about
-// 200 bytes per cell, in L2); a second kernel gathers every copy of a node from the cells of its diamond, sums the
-// copies by shuffles -- no interface pass -- and runs the fused vector update at every copy.
+// cell has a thread (every wedge three, FP64), is computed once and leaves its contributions in a scratch array (in
+// L2); a second kernel gathers every copy of a node from the elements of its diamond, sums the copies by shuffles
+// -- no interface pass -- and runs the fused vector update at every copy.
 // The same two device functions carry the coarsest-level conjugate gradients (k_cg_cluster below).
-// Bound by latency (two dependent launches of a few microseconds), in FP64 by the FP64 pipes (a cell's chain of
-// about 265 instructions at 64 cycles each on an SM partition).  V-cycles went from (streaming tiles filling the SMs) 1017
-// to 366 us (FP32, level 4 / 17 layers), 1404 to 647 us (FP32, two radial points, 5 / 33) and 3999 to 1756 us (FP64,
+// Bound by latency (two dependent launches of a few microseconds), in FP64 by the FP64 pipes (64 cycles
+// per instruction of a warp on an SM partition).  V-cycles went from (streaming tiles filling the SMs) 1017
+// to 366 us (FP32, level 4 / 17 layers), 1404 to 647 us (FP32, two radial points, 5 / 33) and 3999 to 1521 us (FP64,
 // 5 / 33); a thread per group that walks its copies, instead of one per copy, left them at 703, 1072 and 2816 us.
-// Sums run in a fixed order (copies in ascending layout order; corners 00, 10, 01, 11; bottom then top
+// Sums run in a fixed order (copies in ascending layout order; the six triangles; bottom then top
 // contributions), so results do not depend on scheduling.
 
 struct SmallDims {
   int N, n_r, P, ls, ds, nll;  // ls / ds: layer / diamond stride of the node layout, nll: lateral layout size
   int ncell, npad, n_groups;   // cells, lateral points (every copy) rounded up to whole warps, interface groups
+  int div_term;
+  double hgc;  // kappa (3 + c) / 18 of the hourglass control
   Points pts;
+  template <typename T>
+  __device__ __forceinline__ T hgk() const { return (T)hgc; }
 };
-inline SmallDims small_dims(const Level& L) {
+inline SmallDims small_dims(const Level& L, int div_term, double hgc) {
   SmallDims s;
   s.N = L.N, s.n_r = L.n_r, s.P = L.P, s.ls = (int)L.layer_stride, s.ds = (int)L.diamond_stride;
   s.nll = (int)L.n_lat_layout;
   s.ncell = 10 * L.N * L.N * (L.n_r - 1);
   s.pts = points_of(L);
-  s.npad = (s.pts.n + 31) / 32 * 32, s.n_groups = L.n_groups;
+  s.npad = (s.pts.n + 31) / 32 * 32, s.n_groups = L.n_groups, s.div_term = div_term, s.hgc = hgc;
   return s;
 }
 
@@ -40,7 +44,142 @@ inline SmallTab<T> small_tab(const Level& L, BC bc) {
   return SmallTab<T>{Tab<T>::geo(L), Tab<T>::lay(L), Tab<T>::s(L), Tab<T>::gs(L), etav<T>(L), bc.in, bc.out};
 }
 
-// Contributions of cell c = ((d (n_r - 1) + k) N + i) N + j to its eight nodes: bottom corner q, component x
+// How a level's elements are spread: three threads per wedge in FP64, where a cell's chain of instructions bounds the
+// small levels (level 3 / 9 layers: 8.5 against 13 us, FP64 V-cycle level 5 / 33 1521 against 1756 us), one thread per
+// cell in FP32, where the extra contributions cost more than the shorter chain saves (V-cycle level 4 / 17 layers
+// 381 to 388 against 366 us).
+template <typename T>
+constexpr bool kSmallWedges = sizeof(T) == 8;
+
+// FP64: contributions of the wedges to their six nodes, thread per wedge and component: three neighbouring lanes share a
+// wedge, ten wedges a warp (two lanes idle).  A lane forms its component's row of the strain, exchanges the transposed
+// entries and the trace by shuffles and contracts its row of the stress: about 45 dependent FP64 instructions
+// instead of the 265 of a thread per cell (13 us of latency on every small level).  The rows of M^-1 and of the strain
+// are held in the order c, c + 1, c + 2 (mod 3) of the lane's component c, so no register is indexed by c.
+// HG: hourglass control, Q2: the second radial point (see OpA, OpA2).  Wedge v of wb .. wb + 9 (wedge layout); its
+// local node a, component c gets sc[(3 a + c) nw + v] at the bottom and sc[(9 + 3 a + c) nw + v] at the top.  CG: loads
+// bypass L1 (the input was written by other SMs within the same kernel).  All lanes of the warp call it.
+template <typename T, bool HG, bool Q2, bool CG>
+__device__ __forceinline__ void small_wedges(const SmallDims& S, const SmallTab<T>& B, const T* const (&in)[3], int wb,
+                                             T* __restrict__ sc) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = (int)threadIdx.x & 31, g = lane / 3, c = lane - 3 * g, base = 3 * g, nw = 2 * S.ncell;
+  const int v = min(wb + min(g, 9), nw - 1);  // idle lanes repeat the last wedge
+  const bool live = g < 10 && wb + g < nw;
+  const int N = S.N, nc = S.n_r - 1;
+  const int w = v & 1, cell = v >> 1, j = cell % N, r0 = cell / N, i = r0 % N, r1 = r0 / N, k = r1 % nc, d = r1 / nc;
+  const int t = ((d * N + i) * N + j) * 2 + w, nt = 20 * N * N;
+  const int lat = d * S.ls + i * S.P + j, o = lat + d * (S.ds - S.ls) + k * S.ls;
+  // local nodes 0, 1, 2: W0 (i, j), (i + 1, j), (i, j + 1); W1 (i + 1, j + 1), (i, j + 1), (i + 1, j)
+  const int del[3] = {w ? S.P + 1 : 0, w ? 1 : S.P, w ? S.P : 1};
+  const T* const u = c == 0 ? in[0] : (c == 1 ? in[1] : in[2]);
+  T b[3], tp[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    b[a] = CG ? __ldcg(u + o + del[a]) : u[o + del[a]];
+    tp[a] = CG ? __ldcg(u + o + S.ls + del[a]) : u[o + S.ls + del[a]];
+  }
+  const int c1 = c == 2 ? 0 : c + 1, c2 = c == 0 ? 2 : c - 1;
+  T M[3][3];  // M[m][r] = M^-1[m, c + r]
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    M[m][0] = B.geo[(3 * m + c) * nt + t], M[m][1] = B.geo[(3 * m + c1) * nt + t], M[m][2] = B.geo[(3 * m + c2) * nt + t];
+  }
+  const T dM = B.geo[9 * nt + t], e = eta_at(B.eta, (int64_t)v, (int64_t)t);
+  const T* const lc = B.lay + kLayerStride * k;
+  const T r = lc[4], ve = lc[5] * dM * e;
+  // boundary projection: v_c -= (v . s) s_c, the dot product over the three lanes
+  auto project = [&](T (&x)[3], bool here, int bc) {
+    if (!__any_sync(kAll, here)) return;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const T s = B.svec[c * S.nll + lat + del[a]], q = x[a] * s;
+      const T dot = (__shfl_sync(kAll, q, base) + __shfl_sync(kAll, q, base + 1)) + __shfl_sync(kAll, q, base + 2);
+      if (here) x[a] = bc == TN_BC_NOSLIP ? (T)0 : x[a] - dot * s;
+    }
+  };
+  project(b, k == 0, B.bc_in);
+  project(tp, k == nc - 1, B.bc_out);
+  const T d0 = tp[0] - b[0], d1 = tp[1] - b[1], d2 = tp[2] - b[2];
+  const T ax = (tp[1] + b[1]) - (tp[0] + b[0]), ay = (tp[2] + b[2]) - (tp[0] + b[0]), az = (d0 + d1) + d2;
+  // stress row of a strain row G: f (G + G^T) - 2/3 f tr G on the diagonal
+  auto stress = [&](const T (&G)[3], T f, T (&R)[3]) {
+    const T g1 = __shfl_sync(kAll, G[2], base + c1), g2 = __shfl_sync(kAll, G[1], base + c2);  // G^T entries
+    R[0] = (f + f) * G[0];
+    if (S.div_term) {
+      const T tr = (__shfl_sync(kAll, G[0], base) + __shfl_sync(kAll, G[0], base + 1)) + __shfl_sync(kAll, G[0], base + 2);
+      R[0] += (f * (T)(-2.0 / 3.0)) * tr;
+    }
+    R[1] = f * (G[1] + g1), R[2] = f * (G[2] + g2);
+  };
+  auto dot = [&](const T (&R)[3], int m) { return R[0] * M[m][0] + R[1] * M[m][1] + R[2] * M[m][2]; };
+  T G[3], R[3];
+  const T azr = az * r;
+#pragma unroll
+  for (int x = 0; x < 3; ++x) G[x] = ax * M[0][x] + ay * M[1][x] + azr * M[2][x];
+  stress(G, ve, R);
+  T h0 = dot(R, 0), h1 = dot(R, 1);
+  const T h2 = r * dot(R, 2);
+  T y0 = h2, y1 = h2, y2 = h2;
+  if constexpr (HG) {
+    T l = 0, q = 0;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      const T s01 = M[0][x] + M[1][x];
+      l += s01 * s01 + M[0][x] * M[0][x] + M[1][x] * M[1][x];
+      q += M[2][x] * M[2][x];
+    }
+    const T k9 = lc[8], a3 = az * (T)(1.0 / 3.0);
+    const T al1 = (d1 - a3) - k9 * (ax + ax - ay), al2 = (d2 - a3) - k9 * (ay + ay - ax);
+    const T eps = (S.template hgk<T>() * e) * (lc[5] * ((T)2 * dM * l) + lc[9] * ((T)6 * dM * q));
+    const T ek = eps * k9, e3 = eps * (T)(1.0 / 3.0);
+    const T b1 = (al1 + al1) - al2, b2 = (al2 + al2) - al1;
+    h0 -= ek * b1, h1 -= ek * b2;
+    const T v1 = e3 * b1, v2 = e3 * b2;
+    y0 -= v1 + v2, y1 += v1, y2 += v2;
+  }
+  if constexpr (Q2) {
+    const T bx = d1 - d0, by = d2 - d0, a3 = az * (T)(1.0 / 3.0);
+    T G1[3], R1[3];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) G1[x] = bx * M[0][x] + by * M[1][x] + a3 * M[2][x];
+    stress(G1, ve * (T)(1.0 / 3.0), R1);
+    const T k0 = dot(R1, 0), k1 = dot(R1, 1), k2 = dot(R1, 2) * (T)(1.0 / 3.0);
+    y0 += k2 - (k0 + k1), y1 += k2 + k0, y2 += k2 + k1;
+  }
+  if (!live) return;
+  const T x0 = -(h0 + h1);
+  T* const q = sc + v;
+  q[c * nw] = x0 - y0, q[(3 + c) * nw] = h0 - y1, q[(6 + c) * nw] = h1 - y2;
+  q[(9 + c) * nw] = x0 + y0, q[(12 + c) * nw] = h0 + y1, q[(15 + c) * nw] = h1 + y2;
+}
+
+// Partial sum of the wedges of diamond d around node (i, j, k).
+template <typename T>
+__device__ __forceinline__ void small_gather(const SmallDims& S, const T* __restrict__ sc, int d, int i, int j, int k,
+                                             T (&v)[3]) {
+  const int N = S.N, nc = S.n_r - 1, nw = 2 * S.ncell;
+  // cell offset, wedge and local node of the six triangles around a node
+  constexpr int tri[6][4] = {{0, 0, 0, 0}, {-1, 0, 0, 1}, {-1, 0, 1, 2}, {0, -1, 0, 2}, {0, -1, 1, 1}, {-1, -1, 1, 0}};
+  T a[12][3];  // all loads issued before the sums; absent wedges count 0
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const int ci = i + tri[q][0], cj = j + tri[q][1];
+    const bool ok = ci >= 0 && cj >= 0 && ci < N && cj < N;
+    const int vb = (((d * nc + k) * N + ci) * N + cj) * 2 + tri[q][2], vt = vb - 2 * N * N;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      a[q][x] = ok && k < nc ? __ldcg(sc + (3 * tri[q][3] + x) * nw + vb) : (T)0;
+      a[6 + q][x] = ok && k > 0 ? __ldcg(sc + (9 + 3 * tri[q][3] + x) * nw + vt) : (T)0;
+    }
+  }
+#pragma unroll
+  for (int x = 0; x < 3; ++x)
+    v[x] += (((a[0][x] + a[1][x]) + (a[2][x] + a[3][x])) + (a[4][x] + a[5][x])) +
+            (((a[6][x] + a[7][x]) + (a[8][x] + a[9][x])) + (a[10][x] + a[11][x]));
+}
+
+// FP32, thread per cell: contributions of cell c = ((d (n_r - 1) + k) N + i) N + j to its eight nodes: bottom corner q, component x
 // at sc[(3 q + x) ncell + c], top at sc[(12 + 3 q + x) ncell + c].  CG loads bypass L1 when the input was
 // written by other SMs within the same kernel.
 template <typename T, typename Op, bool CG>
@@ -87,7 +226,7 @@ __device__ __forceinline__ void small_cell(const SmallDims& S, const SmallTab<T>
 
 // Partial sum of the cells of diamond d around node (i, j, k).
 template <typename T>
-__device__ __forceinline__ void small_gather(const SmallDims& S, const T* __restrict__ sc, int d, int i, int j, int k,
+__device__ __forceinline__ void small_gather_cells(const SmallDims& S, const T* __restrict__ sc, int d, int i, int j, int k,
                                              T (&v)[3]) {
   const int N = S.N, nc = S.n_r - 1;
   const int di[4] = {0, 1, 0, 1}, dj[4] = {0, 0, 1, 1};
@@ -120,7 +259,8 @@ __device__ __forceinline__ void small_node(const SmallDims& S, const SmallTab<T>
     if (surface)
 #pragma unroll
       for (int x = 0; x < 3; ++x) w[x] = CG ? __ldcg(in[x] + o) : in[x][o];
-    small_gather(S, sc, p.d, p.i, p.j, k, v);
+    if constexpr (kSmallWedges<T>) small_gather(S, sc, p.d, p.i, p.j, k, v);
+    else small_gather_cells(S, sc, p.d, p.i, p.j, k, v);
   }
   copies_sum<T, 3>(p, u, v);
   if (surface && p.cnt) {
@@ -137,8 +277,17 @@ __device__ __forceinline__ void small_node(const SmallDims& S, const SmallTab<T>
   }
 }
 
-constexpr int kSmallBlock = 64;  // threads per CTA: 32 FP64 lanes of a warp take 16 cycles per instruction on an
-                                 // SM's FP64 pipe, so short CTAs spread a level's cells evenly over the SMs
+constexpr int kSmallBlock = 64;  // 20 wedges or 64 cells: short CTAs spread a level evenly over the SMs
+
+template <typename T, bool HG, bool Q2>
+__global__ void __launch_bounds__(kSmallBlock) k_small_wedge(SmallDims S, SmallTab<T> B, const T* __restrict__ in0,
+                                                             const T* __restrict__ in1, const T* __restrict__ in2,
+                                                             T* __restrict__ sc) {
+  const int wb = ((int)(blockIdx.x * kSmallBlock + threadIdx.x) >> 5) * 10;
+  if (wb >= 2 * S.ncell) return;
+  const T* const in[3] = {in0, in1, in2};
+  small_wedges<T, HG, Q2, false>(S, B, in, wb, sc);
+}
 
 template <typename T, typename Op>
 __global__ void __launch_bounds__(kSmallBlock) k_small_cell(SmallDims S, SmallTab<T> B, Op op, const T* __restrict__ in0,
@@ -149,6 +298,16 @@ __global__ void __launch_bounds__(kSmallBlock) k_small_cell(SmallDims S, SmallTa
   const T* const in[3] = {in0, in1, in2};
   small_cell<T, Op, false>(S, B, op, in, c, sc);
 }
+
+// The element op of a level's variant (FP32).
+template <typename T, bool HG, bool Q2>
+struct SmallOp {
+  static __host__ __device__ __forceinline__ OpA<T, HG> make(const SmallDims& S) { return OpA<T, HG>{S.div_term, (T)S.hgc}; }
+};
+template <typename T, bool HG>
+struct SmallOp<T, HG, true> {
+  static __host__ __device__ __forceinline__ OpA2<T> make(const SmallDims& S) { return OpA2<T>{S.div_term}; }
+};
 
 template <typename T, int EPI>
 __global__ void __launch_bounds__(128) k_small_node(SmallDims S, SmallTab<T> B, const T* __restrict__ in0,
@@ -193,8 +352,8 @@ struct CgArgs {
   int maxit, project;
 };
 
-template <typename T, typename Op, bool ONE>
-__global__ void __launch_bounds__(kCgThreads) k_cg_cluster(SmallDims S, SmallTab<T> B, Op op, CgArgs<T> A) {
+template <typename T, bool HG, bool Q2, bool ONE>
+__global__ void __launch_bounds__(kCgThreads) k_cg_cluster(SmallDims S, SmallTab<T> B, CgArgs<T> A) {
   namespace cgr = cooperative_groups;
   cgr::cluster_group cl = cgr::this_cluster();
   __shared__ double wsum[kCgThreads / 32][3], csum[2][kCgCtas][3];
@@ -324,7 +483,12 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_cluster(SmallDims S, SmallTab
   const T* const pp[3] = {A.p[0], A.p[1], A.p[2]};
   if (rz0 > 0.0) {
     for (int it = 0; it < A.maxit; ++it) {
-      for (int c = gt; c < S.ncell; c += GT) small_cell<T, Op, true>(S, B, op, pp, c, A.sc);
+      if constexpr (kSmallWedges<T>) {
+        for (int wb = (gt >> 5) * 10; wb < 2 * S.ncell; wb += (GT / 32) * 10) small_wedges<T, HG, Q2, true>(S, B, pp, wb, A.sc);
+      } else {
+        const auto op = SmallOp<T, HG, Q2>::make(S);
+        for (int c = gt; c < S.ncell; c += GT) small_cell<T, decltype(op), true>(S, B, op, pp, c, A.sc);
+      }
       cl.sync();
       acc[0] = 0.0;
       each([&](Node& n) {  // z holds q = K p until the update
