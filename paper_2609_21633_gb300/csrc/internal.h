@@ -210,6 +210,10 @@ template <typename T>
 cudaError_t launch_small_A(const Level& L, BC bc, int div_term, int epi, const T* const* in, const EpiArgs<T>& E,
                            T* const* y, T* scratch, cudaStream_t st);
 
+// Power-iteration start vector of a level: seeded draws in [-1, 1) per node and component.
+template <typename T>
+cudaError_t launch_start_vector(const Level& L, uint64_t seed, T* const* x, cudaStream_t st);
+
 // Coarsest-level block-Jacobi CG from x = 0 in one launch (small.cuh): until (r, D^-1 r) <= tol2 (r0, D^-1 r0)
 // or maxit steps; project: rigid rotations out of b and x (ginv: inverse rotation Gram matrix).  r, z, p: work
 // vectors of the level's layout.  One cluster of eight SMs: levels whose cells those carry faster than the

