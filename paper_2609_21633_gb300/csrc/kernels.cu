@@ -2409,7 +2409,7 @@ cudaError_t launch_pair32(const Level& L, BC bc, const OpA<float, HG>& op, const
   const EtaView<float> ev = etav<float>(L);
   float4* const ring = reinterpret_cast<float4*>(L.ring64);  // 16 floats per 12 doubles of the FP64 layout
 #define TN_PAIR_LAUNCH(EKv)                                                                                    \
-  k_pair32<HG, F, EPI, EKv><<<grid, kPThreads, kPSmemBytes, st>>>(D, op, in[0], in[1], in[2], out[0], out[1],   \
+  k_pair32<HG, F, EPI, EKv><<<grid, kPThreads, PairPlan<HG>::smem, st>>>(D, op, in[0], in[1], in[2], out[0], out[1],   \
                                                                  out[2], L.geo32, L.lay32, ev, L.s32, bc.in,     \
                                                                  bc.out, kc, skip, E, ring)
   if (ev.kind == TN_ETA_BF16) TN_PAIR_LAUNCH(TN_ETA_BF16);
@@ -2922,7 +2922,7 @@ TN_INST_A(float)
 template <bool HG, int EPI, int EK>
 cudaError_t set_pair32_attr() {
   return cudaFuncSetAttribute(k_pair32<HG, PROJ_IN | PROJ_OUT | ADD_ID, EPI, EK>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPSmemBytes);
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairPlan<HG>::smem);
 }
 template <bool HG, int EPI>
 cudaError_t set_pair32_attrs() {

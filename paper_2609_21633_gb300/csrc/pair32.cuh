@@ -27,17 +27,24 @@ constexpr int kPNodes = 3 * kPRows * kPRow;           // node values per staged 
 constexpr int kPEta = kPTI * kPTJ * 2;                // viscosity values of the tile's wedges per cell layer
 constexpr int kPStage = kPNodes + kPEta;              // floats per stage
 constexpr int kPNodeChunks = kPNodes / 4;             // 16-byte copies of the node values of a layer
-constexpr int kPStages = 4;                           // staged layers
-constexpr int kPAhead = kPStages - 1;                 // layers requested ahead of the bottom one
 constexpr int kPExch = 8 * 33;                        // per component: one down-going value per lane + 1
 constexpr int kPGeo = 2 * 12;                         // float2 column values per thread: 2 wedges x 12
 constexpr int kPMaxKc = 128;                          // cell layers per radial chunk at most
-constexpr size_t kPSmemBytes = sizeof(float) * ((size_t)kPStages * kPStage + 2 * 3 * kPExch) +
-                               sizeof(float2) * (size_t)kPGeo * kPThreads + sizeof(float4) * (kPMaxKc + 1);
+// Staged layers, and the contributions carried from one cell layer to the next in shared memory (of 12 per thread).
+// With hourglass control a thread needs some 25 registers more than the 128 of two CTAs per SM; spilled, they went
+// through an L1 that the staging leaves too small (18 % hits) and their reloads were the kernel's largest stall.  So it
+// gives up a staged layer for most of the carry: k_pair32 at N = 64, n_r = 65 with bf16 viscosity 71 -> 62 us (issue 43 ->
+// 49 % of the slots; math_pipe_throttle is the largest stall now), 524 -> 457 us for the whole apply at N = 128, n_r = 129.
+template <bool HG>
+struct PairPlan {
+  static constexpr int stages = HG ? 3 : 4, ahead = stages - 1, carry = HG ? 11 : 0;
+  static constexpr size_t smem = sizeof(float) * ((size_t)stages * kPStage + 2 * 3 * kPExch) +
+                                 sizeof(float2) * (size_t)(kPGeo + carry) * kPThreads + sizeof(float4) * (kPMaxKc + 1);
+  static_assert(smem <= 113 * 1024, "two CTAs per SM");
+};
 static_assert(kPNodes % 4 == 0 && (kPRows * kPRow) % 4 == 0 && kPRow % 4 == 0 && kPStage % 4 == 0,
               "16-byte staging");
 static_assert(kPNodeChunks <= 2 * kPThreads && kPEta / 4 == kPThreads, "copies per thread per layer");
-static_assert(kPSmemBytes <= 113 * 1024, "two CTAs per SM");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -69,7 +76,11 @@ __device__ __forceinline__ void pair_cell(const float2 (&tp)[4][3], const float2
                                           float2 (&bq)[4][3], float2 (&tq)[4][3]) {
   const float2 r = p2(lc.x, lc.x), vw2 = p2(lc.y, lc.y);
   float2 A[2][3][3];                        // A[w][c] = (a_xi, a_eta, a_zeta) of wedge w, component c
-  float2 D1[HG ? 2 : 1][3], D2[HG ? 2 : 1][3];  // d at a wedge's local nodes 1 and 2 (hourglass control)
+  // Hourglass control: with alpha_a = (d_a - a_zeta / 3) - k9 (2 a_a - a_b), {a, b} = {xi, eta}, a wedge needs
+  // b_1 = 2 alpha_1 - alpha_2 = (2 d_1 - d_2) - 4 k9 (a_xi - a_eta) - a_zeta / 3 - k9 a_xi and b_2 with 1 and 2
+  // exchanged.  The first two terms, g1 and g2, are the same for both wedges: W1 has the two nodes and the sign of
+  // a_xi - a_eta exchanged.
+  float2 g1[HG ? 3 : 1], g2[HG ? 3 : 1];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     float2 sq[4], dq[4];
@@ -78,27 +89,30 @@ __device__ __forceinline__ void pair_cell(const float2 (&tp)[4][3], const float2
     const float2 d12 = add2(dq[1], dq[2]);
     A[0][c][0] = sub2(sq[1], sq[0]), A[0][c][1] = sub2(sq[2], sq[0]), A[0][c][2] = add2(dq[0], d12);
     A[1][c][0] = sub2(sq[2], sq[3]), A[1][c][1] = sub2(sq[1], sq[3]), A[1][c][2] = add2(dq[3], d12);
-    if constexpr (HG) D1[0][c] = dq[1], D2[0][c] = dq[2], D1[HG ? 1 : 0][c] = dq[2], D2[HG ? 1 : 0][c] = dq[1];
+    if constexpr (HG) {
+      const float2 sd = sub2(sq[1], sq[2]), dd = sub2(dq[1], dq[2]);
+      g1[HG ? c : 0] = fma2(p2(-4.f * lc.z, -4.f * lc.z), sd, add2(dq[1], dd));
+      g2[HG ? c : 0] = fma2(p2(4.f * lc.z, 4.f * lc.z), sd, sub2(dq[2], dd));
+    }
   }
-  float2 H0[2][3], H1[2][3], Y[2][HG ? 3 : 1][3];  // Y[w][a][c]: top-minus-bottom part at local node a
+  // X parts h0, h1 of each wedge; Y (top minus bottom) at corners 00 and 11 (Y0), 10 (y1) and 01 (y2 if not y1)
+  float2 H0[2][3], H1[2][3], Y0[2][3], y1[3], y2[HG ? 3 : 1];
 #pragma unroll
   for (int w = 0; w < 2; ++w) {
     float2 M[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) M[q] = gc[(12 * w + q) * kPThreads];
     const float2 mr[3] = {mul2(r, M[6]), mul2(r, M[7]), mul2(r, M[8])};  // r M^-1[2,:]
-    float2 G[3][3], al1[3], al2[3];
+    float2 G[3][3], b1[HG ? 3 : 1], b2[HG ? 3 : 1];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const float2 ax = A[w][c][0], ay = A[w][c][1], az = A[w][c][2];
 #pragma unroll
       for (int x = 0; x < 3; ++x) G[c][x] = fma2(ax, M[x], fma2(ay, M[3 + x], mul2(az, mr[x])));
       if constexpr (HG) {
-        // alpha_1 = (d_1 - a_zeta / 3) - k9 (2 a_xi - a_eta), alpha_2 = (d_2 - a_zeta / 3) - k9 (2 a_eta - a_xi)
-        const float2 nk9 = p2(-lc.z, -lc.z), a3 = mul2(az, p2(1.f / 3.f, 1.f / 3.f));
-        const float2 dl = sub2(ax, ay);
-        al1[c] = fma2(nk9, add2(ax, dl), sub2(D1[HG ? w : 0][c], a3));
-        al2[c] = fma2(nk9, sub2(ay, dl), sub2(D2[HG ? w : 0][c], a3));
+        const float2 nk9 = p2(-lc.z, -lc.z), n3 = p2(-1.f / 3.f, -1.f / 3.f);
+        b1[HG ? c : 0] = fma2(nk9, ax, fma2(n3, az, w ? g2[HG ? c : 0] : g1[HG ? c : 0]));
+        b2[HG ? c : 0] = fma2(nk9, ay, fma2(n3, az, w ? g1[HG ? c : 0] : g2[HG ? c : 0]));
       }
     }
     const float2 ve = mul2(mul2(vw2, gc[(12 * w + 9) * kPThreads]), eta[w]);
@@ -113,11 +127,11 @@ __device__ __forceinline__ void pair_cell(const float2 (&tp)[4][3], const float2
     S[0][1] = S[1][0] = mul2(ve, add2(G[0][1], G[1][0]));
     S[0][2] = S[2][0] = mul2(ve, add2(G[0][2], G[2][0]));
     S[1][2] = S[2][1] = mul2(ve, add2(G[1][2], G[2][1]));
-    float2 nek = p2(0.f, 0.f), e3 = p2(0.f, 0.f);  // -eps k9, eps / 3
+    float2 nek = p2(0.f, 0.f), e3 = nek, ne3 = nek;  // -eps k9, eps / 3, -eps / 3
     if constexpr (HG) {
       const float2 eps = mul2(mul2(p2(hgk, hgk), eta[w]),
                               fma2(vw2, gc[(12 * w + 10) * kPThreads], mul2(p2(lc.w, lc.w), gc[(12 * w + 11) * kPThreads])));
-      nek = mul2(eps, p2(-lc.z, -lc.z)), e3 = mul2(eps, p2(1.f / 3.f, 1.f / 3.f));
+      nek = mul2(eps, p2(-lc.z, -lc.z)), e3 = mul2(eps, p2(1.f / 3.f, 1.f / 3.f)), ne3 = mul2(eps, p2(-1.f / 3.f, -1.f / 3.f));
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -125,13 +139,15 @@ __device__ __forceinline__ void pair_cell(const float2 (&tp)[4][3], const float2
       float2 h1 = fma2(S[c][0], M[3], fma2(S[c][1], M[4], mul2(S[c][2], M[5])));
       const float2 h2 = fma2(S[c][0], mr[0], fma2(S[c][1], mr[1], mul2(S[c][2], mr[2])));
       if constexpr (HG) {
-        // b_1 = 2 alpha_1 - alpha_2, b_2 = 2 alpha_2 - alpha_1 (b_1 + b_2 = alpha_1 + alpha_2)
-        const float2 b1 = sub2(add2(al1[c], al1[c]), al2[c]), b2 = sub2(add2(al2[c], al2[c]), al1[c]);
-        h0 = fma2(nek, b1, h0), h1 = fma2(nek, b2, h1);
-        Y[w][0][c] = sub2(h2, mul2(e3, add2(al1[c], al2[c])));
-        Y[w][HG ? 1 : 0][c] = fma2(e3, b1, h2), Y[w][HG ? 2 : 0][c] = fma2(e3, b2, h2);
+        const float2 q1 = b1[HG ? c : 0], q2 = b2[HG ? c : 0];
+        h0 = fma2(nek, q1, h0), h1 = fma2(nek, q2, h1);
+        // local nodes 1 and 2 of W1 are the corners 01 and 10, those of W0 the other way round
+        Y0[w][c] = fma2(ne3, add2(q1, q2), h2);
+        y1[c] = w ? fma2(e3, q2, add2(y1[c], h2)) : fma2(e3, q1, h2);
+        y2[HG ? c : 0] = w ? fma2(e3, q1, add2(y2[HG ? c : 0], h2)) : fma2(e3, q2, h2);
       } else {
-        Y[w][0][c] = h2;
+        Y0[w][c] = h2;
+        y1[c] = w ? add2(y1[c], h2) : h2;
       }
       H0[w][c] = h0, H1[w][c] = h1;
     }
@@ -142,18 +158,11 @@ __device__ __forceinline__ void pair_cell(const float2 (&tp)[4][3], const float2
   for (int c = 0; c < 3; ++c) {
     const float2 u0 = add2(H0[0][c], H1[0][c]), u3 = add2(H0[1][c], H1[1][c]);  // -X at 00 and 11
     const float2 x1 = add2(H0[0][c], H1[1][c]), x2 = add2(H1[0][c], H0[1][c]);
-    float2 y0, y1, y2, y3;
-    if constexpr (HG) {
-      y0 = Y[0][0][c], y3 = Y[1][0][c];
-      y1 = add2(Y[0][HG ? 1 : 0][c], Y[1][HG ? 2 : 0][c]), y2 = add2(Y[0][HG ? 2 : 0][c], Y[1][HG ? 1 : 0][c]);
-    } else {
-      y0 = Y[0][0][c], y3 = Y[1][0][c];
-      y1 = y2 = add2(y0, y3);
-    }
-    bq[0][c] = add2(u0, y0), tq[0][c] = sub2(y0, u0);
-    bq[3][c] = add2(u3, y3), tq[3][c] = sub2(y3, u3);
-    bq[1][c] = sub2(x1, y1), tq[1][c] = add2(x1, y1);
-    bq[2][c] = sub2(x2, y2), tq[2][c] = add2(x2, y2);
+    const float2 v1 = y1[c], v2 = HG ? y2[HG ? c : 0] : v1;
+    bq[0][c] = add2(u0, Y0[0][c]), tq[0][c] = sub2(Y0[0][c], u0);
+    bq[3][c] = add2(u3, Y0[1][c]), tq[3][c] = sub2(Y0[1][c], u3);
+    bq[1][c] = sub2(x1, v1), tq[1][c] = add2(x1, v1);
+    bq[2][c] = sub2(x2, v2), tq[2][c] = add2(x2, v2);
   }
 }
 
@@ -175,10 +184,12 @@ __global__ void __launch_bounds__(kPThreads, 2)
              EtaView<float> eta, const float* __restrict__ svec, int bc_in, int bc_out, int kc,
              const int* __restrict__ skip, EpiArgs<float> E, float4* __restrict__ ring) {
   extern __shared__ __align__(16) float psm[];
+  constexpr int kPStages = PairPlan<HG>::stages, kPAhead = PairPlan<HG>::ahead, kCarry = PairPlan<HG>::carry;
   float* const stg = psm;                                                   // [kPStages][kPStage]
   float* const exb = psm + kPStages * kPStage;                              // [2][3][kPExch]
   float2* const gc0 = reinterpret_cast<float2*>(exb + 2 * 3 * kPExch);      // [kPGeo][kPThreads]
-  float4* const lct = reinterpret_cast<float4*>(gc0 + kPGeo * kPThreads);   // [kPMaxKc + 1]
+  float2* const cy = gc0 + kPGeo * kPThreads + threadIdx.x;                 // [kCarry][kPThreads], this thread's slot
+  float4* const lct = reinterpret_cast<float4*>(gc0 + (kPGeo + kCarry) * kPThreads);  // [kPMaxKc + 1]
   float2* const gc = gc0 + threadIdx.x;
   if (skip && *skip) return;
   const int N = D.N, n_r = D.n_r, P = D.P;
@@ -404,7 +415,7 @@ __global__ void __launch_bounds__(kPThreads, 2)
     }
   };
   // one cell layer: cin holds the top contributions of cell layer k - 1 to node layer k, cout
-  // receives those of cell layer k to node layer k + 1
+  // receives those of cell layer k to node layer k + 1 (values 3 q + c < kCarry of both in shared memory)
   auto step = [&](int k, const float2 (&cin)[4][3], float2 (&cout)[4][3]) {
     float2 tp[4][3], bt[4][3], e[2];
     read_pairs(k + 1, tp);
@@ -414,20 +425,22 @@ __global__ void __launch_bounds__(kPThreads, 2)
     // previous barrier
     issue(k + kPAhead);
     if (k + 1 < n_r) prefetch_layer(k + 1);
-    float2 bq[4][3];
-    pair_cell<HG>(tp, bt, gc, lct[k - kstart], e, op.div_term, op.hgk, bq, cout);
-    cp_async_wait<kPAhead - 2>();  // layer k + 2 is in (made visible by the next barrier)
-    if (k >= kc0) {
-      float2 tot[4][3];
+    float2 bq[4][3], tq[4][3];
+    pair_cell<HG>(tp, bt, gc, lct[k - kstart], e, op.div_term, op.hgk, bq, tq);
+    float2 tot[4][3];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        tot[0][c] = sub2(cin[0][c], bq[0][c]), tot[3][c] = sub2(cin[3][c], bq[3][c]);
-        tot[1][c] = add2(cin[1][c], bq[1][c]), tot[2][c] = add2(cin[2][c], bq[2][c]);
+        const bool sm = 3 * q + c < kCarry;
+        const float2 ci = sm ? cy[(sm ? 3 * q + c : 0) * kPThreads] : cin[q][c];
+        tot[q][c] = q == 0 || q == 3 ? sub2(ci, bq[q][c]) : add2(ci, bq[q][c]);
+        if (sm) cy[(sm ? 3 * q + c : 0) * kPThreads] = tq[q][c];
+        else cout[q][c] = tq[q][c];
       }
-      finish_layer(k, tot);
-    } else {
-      __syncthreads();
-    }
+    cp_async_wait<kPAhead - 2>();  // layer k + 2 is in (made visible by the next barrier)
+    if (k >= kc0) finish_layer(k, tot);
+    else __syncthreads();
   };
 
 #pragma unroll
@@ -438,7 +451,10 @@ __global__ void __launch_bounds__(kPThreads, 2)
 #pragma unroll
   for (int q = 0; q < 4; ++q)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) ca[q][c] = p2(0.f, 0.f);
+    for (int c = 0; c < 3; ++c) {
+      ca[q][c] = p2(0.f, 0.f);
+      if (3 * q + c < kCarry) cy[(3 * q + c < kCarry ? 3 * q + c : 0) * kPThreads] = ca[q][c];
+    }
   int k = kstart;
   for (; k + 1 < kc1; k += 2) {  // two layers per trip: the carried contributions swap arrays
     step(k, ca, cb);
@@ -446,8 +462,17 @@ __global__ void __launch_bounds__(kPThreads, 2)
   }
   if (k < kc1) {
     step(k, ca, cb);
-    if (kc1 == n_r - 1) finish_layer(n_r - 1, cb);
-  } else if (kc1 == n_r - 1) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) ca[q][c] = cb[q][c];
+  }
+  if (kc1 == n_r - 1) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        if (3 * q + c < kCarry) ca[q][c] = cy[(3 * q + c < kCarry ? 3 * q + c : 0) * kPThreads];
     finish_layer(n_r - 1, ca);
   }
   cp_async_wait<0>();
