@@ -2419,13 +2419,10 @@ cudaError_t launch_pair32(const Level& L, BC bc, const OpA<float, HG>& op, const
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const RingDims RD = ring_dims(L.N, kPTI, kPTJ);
-  k_ring4_fix<F, EPI><<<dim3(nblk(RD.RC, 256), L.n_r, 10), 256, 0, st>>>(D, RD, ring, in[0], in[1], in[2], out[0],
-                                                                        out[1], out[2], L.s32, bc.in, bc.out, skip, E);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_ring4_edges<EPI><<<dim3(nblk(L.n_edge, 128), L.n_r), 128, 0, st>>>(
-      D, RD, L.n_edge, L.edge, L.n_groups, L.grp_s32, ring, in[0], in[1], in[2], out[0], out[1], out[2],
-      bc.in, bc.out, skip, E);
+  const int ne = nblk(L.n_edge, 128), nrc = nblk(RD.RC, 128);
+  k_ring4<F, EPI><<<dim3(ne + 10 * nrc, L.n_r), 128, 0, st>>>(D, RD, ne, nrc, L.n_edge, L.edge, L.n_groups, L.grp_s32, ring,
+                                                             in[0], in[1], in[2], out[0], out[1], out[2], L.s32, bc.in,
+                                                             bc.out, skip, E);
   return cudaGetLastError();
 }
 

@@ -16,9 +16,9 @@
 // * Cell contributions are summed into node values in a fixed order: the two cells of a thread in
 //   registers, the left neighbour's by a warp shuffle, the upper warp's through shared memory.
 //   Nodes on the tile lines i = i0, i0 + 16 and j = j0, j0 + 32 leave one float4 partial per tile
-//   in the level's ring buffer (the tile-line index of the FP64 halo-free tiles).  k_ring4_fix
-//   sums and finishes those inside the diamond, k_ring4_edges those on the diamond edges with the
-//   sum over their copies; no atomics, so results do not depend on scheduling.
+//   in the level's ring buffer (the tile-line index of the FP64 halo-free tiles).  k_ring4 sums and
+//   finishes them, on the diamond edges with the sum over their copies; no atomics, so results do
+//   not depend on scheduling.
 
 constexpr int kPTI = 16, kPTJ = 32, kPThreads = 256;  // cells per tile, threads per CTA
 constexpr int kPRows = kPTI + 1;                      // node rows i0 .. i0 + 16 of a tile
@@ -496,58 +496,52 @@ __device__ __forceinline__ void ring4_sum(const RingDims& RD, int N, int n_r, co
   }
 }
 
-// Diamond-edge nodes of the paired-cell tiles, one thread per copy and node layer k: the ring partials of the copy's
-// diamond, summed over the copies by shuffles, the boundary rows projected and (I - P) u added once, then the
-// value -- or the fused vector update -- at the copy (what k_ring_fix and k_interface do in two passes for the
-// other tiles).
-template <int EPI>
-__global__ void __launch_bounds__(128)
-    k_ring4_edges(Dims D, RingDims RD, int n_edge, const int4* __restrict__ edge, int n_groups,
-                  const float* __restrict__ gs, const float4* __restrict__ ring, const float* __restrict__ in0,
-                  const float* __restrict__ in1, const float* __restrict__ in2, float* __restrict__ out0,
-                  float* __restrict__ out1, float* __restrict__ out2, int bc_in, int bc_out,
-                  const int* __restrict__ skip, EpiArgs<float> E) {
-  if (skip && *skip) return;
-  const int t = blockIdx.x * 128 + threadIdx.x, k = blockIdx.y;  // grid: edge entries x layers
-  const Point p = t < n_edge ? edge_point(edge[t]) : Point{0, 0, 0, 0, 0, 0};
-  const int N = D.N, n_r = D.n_r;
-  const int o = (int)(p.d * D.diamond_stride) + k * (int)D.layer_stride + p.i * D.P + p.j;
-  const bool surface = k == 0 || k == n_r - 1;
-  float v[3] = {0.f, 0.f, 0.f}, w[3] = {0.f, 0.f, 0.f};
-  if (p.cnt) {
-    epi_prefetch<float, EPI>(E, o);
-    ring4_sum(RD, N, n_r, ring, k, p.d, p.i, p.j, v);
-    if (surface) w[0] = in0[o], w[1] = in1[o], w[2] = in2[o];
-  }
-  copies_sum<float, 3>(p, t & ~31, v);
-  if (!p.cnt) return;
-  if (surface) {
-    const int bc = k == 0 ? bc_in : bc_out;
-    if (bc == TN_BC_NOSLIP) {
-      for (int c = 0; c < 3; ++c) v[c] = w[c];
-    } else {
-      const float s[3] = {gs[p.g], gs[n_groups + p.g], gs[2 * n_groups + p.g]};
-      const float dv = v[0] * s[0] + v[1] * s[1] + v[2] * s[2], dw = w[0] * s[0] + w[1] * s[1] + w[2] * s[2];
-      for (int c = 0; c < 3; ++c) v[c] += (dw - dv) * s[c];
-    }
-  }
-  if (EPI != EPI_NONE) {
-    epilogue<float, EPI>(E, in0, in1, in2, o, v);
-  } else {
-    out0[o] = v[0], out1[o] = v[1], out2[o] = v[2];
-  }
-}
-
-// Sums the ring partials of k_pair32 and finishes the tile-line nodes inside the diamond (as
-// k_ring_fix does for the FP64 halo-free tiles); the diamond-edge nodes are k_ring4_edges'.
+// The tile-line nodes of the paired-cell tiles, one launch: the first ne blocks of a layer take the diamond edges, one
+// thread per copy -- the ring partials of the copy's diamond, summed over the copies by shuffles, the boundary rows
+// projected and (I - P) u added once, then the value, or the fused vector update, at the copy (what k_ring_fix and
+// k_interface do in two passes for the other tiles) --, the others the tile lines inside the diamonds (as k_ring_fix),
+// nrc blocks per diamond.  Both are chains of dependent loads on few nodes, so they run side by side: as two launches
+// the FP32 V-cycle at N = 64, n_r = 65 took 1897 us instead of 1874, an apply at N = 128, n_r = 129 457 instead of 449.
 template <int FLAGS, int EPI>
-__global__ void k_ring4_fix(Dims D, RingDims RD, const float4* __restrict__ ring, const float* __restrict__ in0,
-                            const float* __restrict__ in1, const float* __restrict__ in2, float* __restrict__ out0,
-                            float* __restrict__ out1, float* __restrict__ out2, const float* __restrict__ svec,
-                            int bc_in, int bc_out, const int* __restrict__ skip, EpiArgs<float> E) {
+__global__ void __launch_bounds__(128)
+    k_ring4(Dims D, RingDims RD, int ne, int nrc, int n_edge, const int4* __restrict__ edge, int n_groups,
+            const float* __restrict__ gs, const float4* __restrict__ ring, const float* __restrict__ in0,
+            const float* __restrict__ in1, const float* __restrict__ in2, float* __restrict__ out0,
+            float* __restrict__ out1, float* __restrict__ out2, const float* __restrict__ svec, int bc_in, int bc_out,
+            const int* __restrict__ skip, EpiArgs<float> E) {
   if (skip && *skip) return;
-  const int N = D.N, n_r = D.n_r;
-  const int rid = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y, d = blockIdx.z;  // grid: RC x n_r x 10
+  const int N = D.N, n_r = D.n_r, k = blockIdx.y;
+  if ((int)blockIdx.x < ne) {
+    const int t = blockIdx.x * 128 + threadIdx.x;
+    const Point p = t < n_edge ? edge_point(edge[t]) : Point{0, 0, 0, 0, 0, 0};
+    const int o = (int)(p.d * D.diamond_stride) + k * (int)D.layer_stride + p.i * D.P + p.j;
+    const bool surface = k == 0 || k == n_r - 1;
+    float v[3] = {0.f, 0.f, 0.f}, w[3] = {0.f, 0.f, 0.f};
+    if (p.cnt) {
+      epi_prefetch<float, EPI>(E, o);
+      ring4_sum(RD, N, n_r, ring, k, p.d, p.i, p.j, v);
+      if (surface) w[0] = in0[o], w[1] = in1[o], w[2] = in2[o];
+    }
+    copies_sum<float, 3>(p, t & ~31, v);
+    if (!p.cnt) return;
+    if (surface) {
+      const int bc = k == 0 ? bc_in : bc_out;
+      if (bc == TN_BC_NOSLIP) {
+        for (int c = 0; c < 3; ++c) v[c] = w[c];
+      } else {
+        const float s[3] = {gs[p.g], gs[n_groups + p.g], gs[2 * n_groups + p.g]};
+        const float dv = v[0] * s[0] + v[1] * s[1] + v[2] * s[2], dw = w[0] * s[0] + w[1] * s[1] + w[2] * s[2];
+        for (int c = 0; c < 3; ++c) v[c] += (dw - dv) * s[c];
+      }
+    }
+    if (EPI != EPI_NONE) {
+      epilogue<float, EPI>(E, in0, in1, in2, o, v);
+    } else {
+      out0[o] = v[0], out1[o] = v[1], out2[o] = v[2];
+    }
+    return;
+  }
+  const int rb = (int)blockIdx.x - ne, d = rb / nrc, rid = rb % nrc * 128 + threadIdx.x;
   if (rid >= RD.RC) return;
   int i, j;
   if (rid < RD.H) {
