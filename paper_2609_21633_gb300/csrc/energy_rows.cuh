@@ -6,8 +6,8 @@
 // level 6 / 65 layers, the FP64 pipe); a stencil residual reads 160 bytes per node and does 40 FP64
 // instructions.  Constants are in the null space of all three terms, so the rows hold no diagonal and act on
 // differences to the node's own value: exactly zero for constants, and no cancellation of large T.
-// Measured, level 6 / 65 layers: ten Heun steps 39.9 -> 7.7 ms (wedge values 0.73 ms, rows 2.3 ms, 0.23 ms per stage,
-// all held by the FP64 pipe); one step 4.0 -> 3.6 ms.
+// Measured, level 6 / 65 layers: ten Heun steps 39.9 -> 7.1 ms (wedge values 0.73 ms, rows 1.7 ms, 0.23 ms per stage,
+// all held by the FP64 pipe); one step 4.0 -> 2.9 ms.
 // Nodes that several diamonds share keep one partial row per copy (the wedges of that diamond).
 
 struct RowDims {
@@ -90,55 +90,75 @@ __global__ void __launch_bounds__(128) k_energy_wedge(Dims D, const double* __re
 // Rows dt / m_j (K + C + S)_j of the interior node layers, thread per layout node.  Node j = (local a, side s) of
 // wedge (t, k) has, with A = V w0^2, beta_a,s = lam_a + s mu (w0 ubar . grad) and C = V / 6 + V tau beta_a,s, the entries
 //   (b, s'):  P_b + s' Q,  P_b = A (l_a . l_b + s r l_b . m2) + C lam_b,  Q = A (r l_a . m2 + s r^2 |m2|^2) + C mu.
-__global__ void __launch_bounds__(128) k_energy_rows(Dims D, const double* __restrict__ geo, const double* __restrict__ lay,
+// The sums over the wedges run over P_b and Q apart, per side (three and five fused operations per wedge, side and b; adding
+// P - Q and P + Q to the 21 entries took seven), and the dot products of a column's M^-1 rows serve kRowLayers node layers:
+// about 350 FP64 instructions a node instead of 770.  2.3 -> 1.7 ms at level 6 / 65 layers; ten Heun steps 7.73 -> 7.11 ms, at
+// level 4 / 17 layers 767 -> 760 us.
+constexpr int kRowLayers = 8;  // at most: fewer where the grid would not give every SM three CTAs
+__global__ void __launch_bounds__(128, 3) k_energy_rows(Dims D, int nk, const double* __restrict__ geo, const double* __restrict__ lay,
                                                      const WedgeFlow* __restrict__ wq, const double* __restrict__ mass,
                                                      double dt, int64_t n, double* __restrict__ rows) {
   const int N = D.N, M1 = N + 1;
-  const int p = blockIdx.x * 128 + threadIdx.x;  // grid: lattice points x (n_r - 2) x 10 diamonds
+  const int p = blockIdx.x * 128 + threadIdx.x;  // grid: lattice points x groups of interior node layers x 10 diamonds
   if (p >= M1 * M1) return;
-  const int i = p / M1, j = p - i * M1, k = blockIdx.y + 1, d = blockIdx.z;
-  double c[kRowCoef + 1];  // [7 (dk + 1) + lateral neighbour]; the diagonal is dropped at the end
-#pragma unroll
-  for (int q = 0; q <= kRowCoef; ++q) c[q] = 0.0;
+  const int i = p / M1, j = p - i * M1, d = blockIdx.z;
+  const int k0 = 1 + blockIdx.y * nk, k1 = min(D.n_r - 1, k0 + nk);
+  bool on[6];
+  double lr[6][2], nr[6][2], gg[6], dM[6];  // l_a . l_1, l_a . l_2 (l_0 = -(l_1 + l_2)), the same with m2, |m2|^2, |det M|
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
     const int ci = i + kRowTri[q][0], cj = j + kRowTri[q][1];
-    if (ci < 0 || cj < 0 || ci >= N || cj >= N) continue;
+    on[q] = ci >= 0 && cj >= 0 && ci < N && cj < N;
+    lr[q][0] = lr[q][1] = nr[q][0] = nr[q][1] = gg[q] = dM[q] = 0.0;
+    if (!on[q]) continue;
     const int a = kRowTri[q][3] == 0 ? 0 : (kRowTri[q][4] == 0 ? 1 : 2);
-    const int t = (ci * N + cj) * 2 + kRowTri[q][2];
-    const int64_t lt = (int64_t)d * 2 * N * N + t;
+    const int64_t lt = (int64_t)d * 2 * N * N + (ci * N + cj) * 2 + kRowTri[q][2];
     double m[9];
 #pragma unroll
     for (int x = 0; x < 9; ++x) m[x] = geo[(int64_t)x * D.n_tri + lt];
-    const double dM = geo[9 * D.n_tri + lt];
+    dM[q] = geo[9 * D.n_tri + lt];
     const double g00 = m[0] * m[0] + m[1] * m[1] + m[2] * m[2], g01 = m[0] * m[3] + m[1] * m[4] + m[2] * m[5],
-                 g11 = m[3] * m[3] + m[4] * m[4] + m[5] * m[5], g02 = m[0] * m[6] + m[1] * m[7] + m[2] * m[8],
-                 g12 = m[3] * m[6] + m[4] * m[7] + m[5] * m[8], g22 = m[6] * m[6] + m[7] * m[7] + m[8] * m[8];
-    const double nm[3] = {-(g02 + g12), g02, g12};                                    // l_b . m2
-    const double r0 = a == 0 ? -(g00 + g01) : (a == 1 ? g00 : g01), r1 = a == 0 ? -(g01 + g11) : (a == 1 ? g01 : g11);
-    const double ll[3] = {-(r0 + r1), r0, r1};                                        // l_a . l_b
+                 g11 = m[3] * m[3] + m[4] * m[4] + m[5] * m[5];
+    nr[q][0] = m[0] * m[6] + m[1] * m[7] + m[2] * m[8], nr[q][1] = m[3] * m[6] + m[4] * m[7] + m[5] * m[8];
+    gg[q] = m[6] * m[6] + m[7] * m[7] + m[8] * m[8];
+    lr[q][0] = a == 0 ? -(g00 + g01) : (a == 1 ? g00 : g01), lr[q][1] = a == 0 ? -(g01 + g11) : (a == 1 ? g01 : g11);
+  }
+  for (int k = k0; k < k1; ++k) {
+    double P[2][7], Q[2][7];  // [side][lateral neighbour], side 0: the node is on the wedge's bottom layer
 #pragma unroll
-    for (int side = 0; side < 2; ++side) {  // 0: the node is on the wedge's bottom layer
-      const int kk = k - side;
-      const double* l = lay + kLayerStride * kk;
-      const WedgeFlow v = wq[((int64_t)d * (D.n_r - 1) + kk) * 2 * N * N + t];
-      const double lam[3] = {-(v.l0 + v.l1), v.l0, v.l1}, r = l[4], A = l[5] * dM, V = l[2] * dM;
-      const double sr = side ? r : -r, beta = lam[a] + (side ? v.mu : -v.mu), C = V * (1.0 / 6.0) + v.vt * beta;
-      const double Q = A * (r * (nm[a] + sr * g22)) + C * v.mu;
+    for (int x = 0; x < 7; ++x) P[0][x] = P[1][x] = Q[0][x] = Q[1][x] = 0.0;
 #pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const double P = A * (ll[b] + sr * nm[b]) + C * lam[b];
-        const int nb = kRowTri[q][3 + b];
-        c[7 * (1 - side) + nb] += P - Q;  // bottom layer kk
-        c[7 * (2 - side) + nb] += P + Q;  // top layer kk + 1
+    for (int q = 0; q < 6; ++q) {
+      if (!on[q]) continue;
+      const int a = kRowTri[q][3] == 0 ? 0 : (kRowTri[q][4] == 0 ? 1 : 2);
+      const int t = ((i + kRowTri[q][0]) * N + j + kRowTri[q][1]) * 2 + kRowTri[q][2];
+      const double ll[3] = {-(lr[q][0] + lr[q][1]), lr[q][0], lr[q][1]}, nm[3] = {-(nr[q][0] + nr[q][1]), nr[q][0], nr[q][1]};
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        const int kk = k - side;
+        const double* l = lay + kLayerStride * kk;
+        const WedgeFlow v = wq[((int64_t)d * (D.n_r - 1) + kk) * 2 * N * N + t];
+        const double lam[3] = {-(v.l0 + v.l1), v.l0, v.l1}, r = l[4], A = l[5] * dM[q], V = l[2] * dM[q];
+        const double sr = side ? r : -r, beta = lam[a] + (side ? v.mu : -v.mu), C = V * (1.0 / 6.0) + v.vt * beta;
+        const double q0 = (A * r) * (nm[a] + sr * gg[q]) + C * v.mu;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          const int nb = kRowTri[q][3 + b];
+          P[side][nb] += A * (ll[b] + sr * nm[b]);
+          P[side][nb] += C * lam[b];
+          Q[side][nb] += q0;
+        }
       }
     }
-  }
-  const int64_t idx = (int64_t)d * D.diamond_stride + (int64_t)k * D.layer_stride + (int64_t)i * D.P + j;
-  const double f = dt / mass[idx];
+    const int64_t idx = (int64_t)d * D.diamond_stride + (int64_t)k * D.layer_stride + (int64_t)i * D.P + j;
+    const double f = dt / mass[idx];
 #pragma unroll
-  for (int q = 0; q <= kRowCoef; ++q)
-    if (q != 7) rows[(int64_t)(q < 7 ? q : q - 1) * n + idx] = f * c[q];
+    for (int x = 0; x < 7; ++x) {
+      rows[(int64_t)x * n + idx] = f * (P[1][x] - Q[1][x]);
+      if (x > 0) rows[(int64_t)(6 + x) * n + idx] = f * ((P[1][x] + Q[1][x]) + (P[0][x] - Q[0][x]));
+      rows[(int64_t)(13 + x) * n + idx] = f * (P[0][x] + Q[0][x]);
+    }
+  }
 }
 
 // One Heun stage over the unique lateral points: with d = dt M^-1 R(X), stage 1: out = X - d; stage 2: out = ((T + X) -
@@ -224,7 +244,9 @@ inline cudaError_t heun_rows(EnergyState& S, const Level& L, double* T, double* 
       D, L.geo64, L.lay64, u[0], u[1], u[2], supg, S.wq);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) {
-    k_energy_rows<<<dim3(np, L.n_r - 2, 10), 128, 0, st>>>(D, L.geo64, L.lay64, S.wq, S.mass, dt, L.n_layout, S.rows);
+    const int nk = std::max(1, std::min(kRowLayers, (int)(np * 10 * (L.n_r - 2) / (152 * 3))));
+    k_energy_rows<<<dim3(np, (L.n_r - 2 + nk - 1) / nk, 10), 128, 0, st>>>(D, nk, L.geo64, L.lay64, S.wq, S.mass, dt, L.n_layout,
+                                                                          S.rows);
     e = cudaGetLastError();
   }
   const RowDims R = row_dims(L);
