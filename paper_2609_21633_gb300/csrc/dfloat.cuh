@@ -249,27 +249,9 @@ __device__ __forceinline__ df2 mul2(const df2& x, const df2& y) {
   fast_two_sum2(ch, p2add(cl1, cl2), zh, zl);
   return df2{zh, zl};
 }
-// add_nc / fma_nc, lane-wise
-__device__ __forceinline__ df2 add_nc2(const df2& x, const df2& y) {
-  float2 sh, sl, zh, zl;
-  two_sum2(x.hi, y.hi, sh, sl);
-  fast_two_sum2(sh, p2add(sl, p2add(x.lo, y.lo)), zh, zl);
-  return df2{zh, zl};
-}
-__device__ __forceinline__ df2 fma_nc2(const df2& x, const df2& y, const df2& w) {
-  const float2 ph = p2mul(x.hi, y.hi);
-  float2 pl = p2fma(x.hi, y.hi, p2neg(ph));
-  pl = p2fma(x.hi, y.lo, pl);
-  pl = p2fma(x.lo, y.hi, pl);
-  float2 sh, sl, zh, zl;
-  two_sum2(ph, w.hi, sh, sl);
-  fast_two_sum2(sh, p2add(sl, p2add(pl, w.lo)), zh, zl);
-  return df2{zh, zl};
-}
-
 // Running sums of packed double-words, not renormalised between steps (acc2: value s + l, s the rounded sum
 // of the high parts, l everything below it).  A contraction of three products costs 24 packed
-// operations this way against 39 with a renormalised multiplication and two fma_nc2.  Errors: each
+// operations this way against 39 with a renormalised multiplication and two renormalised fused operations.  Errors: each
 // step rounds l, which stays a few u |terms|, so a step adds about u^2 |terms|; the products drop l l.  That
 // is the level at which the operands are rounded to double-words anyway (the accurate additions they
 // replace keep no more digits of such operands).

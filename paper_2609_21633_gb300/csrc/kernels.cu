@@ -76,10 +76,6 @@ inline unsigned nblk(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); 
 #ifndef TN_WIDE_MAXREG
 #define TN_WIDE_MAXREG 96
 #endif
-// 1: load node layer k+2 while cell layer k is computed
-#ifndef TN_PREFETCH
-#define TN_PREFETCH 0
-#endif
 // FP32 A apply on paired-cell tiles (pair32.cuh) where N >= 32 (0: the square tiles)
 #ifndef TN_PAIR32
 #define TN_PAIR32 1

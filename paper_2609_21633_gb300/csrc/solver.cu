@@ -296,30 +296,20 @@ __global__ void k_bmul(int64_t n, B6<T> binv, Ptr4<T> x, MPtr4<T> y) {
   for (int c = 0; c < 3; ++c) y.c[c][i] = z[c];
 }
 
+// First half of a Chebyshev step from x = 0 (Saad, Iterative Methods for Sparse Linear Systems, Alg. 12.1, with the
+// block-Jacobi preconditioner D^-1 = inverse 3x3 node blocks): r = b, d = D^-1 r / theta, x = d
 template <typename T>
-__global__ void k_recip(int64_t n, const T* __restrict__ d, T* __restrict__ inv) {
-  const int64_t i = blockIdx.x * (int64_t)EB + threadIdx.x;
-  if (i >= n) return;
-  const T v = d[i];
-  inv[i] = v != (T)0 ? (T)1 / v : (T)0;
-}
-
-// Chebyshev step, part 1 (Saad, Iterative Methods for Sparse Linear Systems, Alg. 12.1, with the
-// block-Jacobi preconditioner D^-1 = inverse 3x3 node blocks):
-// r = b - t (t = K x; zero_x: x = 0, t unused), d = D^-1 r / theta, x += d
-template <typename T>
-__global__ void k_cheb1(int64_t n, int zero_x, double inv_theta, Ptr4<T> b, Ptr4<T> t, B6<T> binv, MPtr4<T> r,
-                        MPtr4<T> d, MPtr4<T> x) {
+__global__ void k_cheb1(int64_t n, double inv_theta, Ptr4<T> b, B6<T> binv, MPtr4<T> r, MPtr4<T> d, MPtr4<T> x) {
   const int64_t i = blockIdx.x * (int64_t)EB + threadIdx.x;
   if (i >= n) return;
   T rr[3], z[3];
-  for (int c = 0; c < 3; ++c) rr[c] = zero_x ? b.c[c][i] : b.c[c][i] - t.c[c][i];
+  for (int c = 0; c < 3; ++c) rr[c] = b.c[c][i];
   bmul(binv, i, rr, z);
   for (int c = 0; c < 3; ++c) {
     const T dd = (T)inv_theta * z[c];
     r.c[c][i] = rr[c];
     d.c[c][i] = dd;
-    x.c[c][i] = zero_x ? dd : x.c[c][i] + dd;
+    x.c[c][i] = dd;
   }
 }
 // ---- coarse CG (device scalars in S, stop flag) ----------------------------------------------
@@ -744,8 +734,8 @@ void cheb_step(MGState* m, const tn_mesh* mesh, int h, bool zero_x, cudaStream_t
   const double theta = 0.5 * (b + a), delta = 0.5 * (b - a), sigma = theta / delta;
   const double rho0 = 1.0 / sigma, rho1 = 1.0 / (2.0 * sigma - rho0);
   if (zero_x) {
-    k_cheb1<T><<<nb(n), EB, 0, st>>>(n, 1, 1.0 / theta, P4<T>(G.b.cc(), 3), P4<T>(G.b.cc(), 3), G.bi(),
-                                     M4<T>(G.r.mm(), 3), M4<T>(G.d().mm(), 3), M4<T>(G.x().mm(), 3));
+    k_cheb1<T><<<nb(n), EB, 0, st>>>(n, 1.0 / theta, P4<T>(G.b.cc(), 3), G.bi(), M4<T>(G.r.mm(), 3), M4<T>(G.d().mm(), 3),
+                                     M4<T>(G.x().mm(), 3));
     ckl();
   } else {
     EpiArgs<T> E = epi_of(G);
