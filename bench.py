@@ -47,22 +47,20 @@ LAW = dict(E=math.log(1e3), jump_r=0.9, jump_factor=30.0)  # x30 below r = 0.9, 
 # the inverse Jacobian and the differences-only scatter of Eq. epsq / Eq. localapply, counted
 # from their structure at 240 flops per wedge.
 A_FLOPS_PER_CELL = 480.0
-# ncu figures of the A tile kernel with the packed double-float element op (level 6, 65 layers,
-# 2,621,440 cells, one launch): DRAM bytes (126.14 MB read + 49.46 MB written) and issued warp
-# instructions (262,034,000) per cell, scaled to the bench size by cells; None once the kernel
-# changes.
-A_TRAFFIC_BYTES_PER_CELL = (126.14e6 + 49.46e6) / 2621440
-A_WARP_INST_PER_CELL = 262034000 / 2621440
+# ncu figures of the double-float A kernel k_df_A (level 6, 65 layers, 2,621,440 cells, one
+# launch): DRAM bytes (134.97 MB read + 45.42 MB written) and issued warp instructions
+# (173,101,283) per cell, scaled to the bench size by cells; None once the kernel changes.
+A_TRAFFIC_BYTES_PER_CELL = (134.97e6 + 45.42e6) / 2621440
+A_WARP_INST_PER_CELL = 173101283 / 2621440
 # Issue rate derived from unit counts: 152 SMs x 4 schedulers x 1 warp instruction per clock.
 ISSUE_SLOTS_PER_CLOCK = 152 * 4
 # Hourglass-control coefficient of the solves and the serving stream that use it.
 HG_KAPPA = 0.3
-# Kernel launches of one A + B + B^T + diag step: A 2 (tile, interface), B 4 (tile, interface,
-# restriction, interface), B^T 3 (prolongation, tile, interface), diag 3 (tile, boundary-layer
-# gather, interface); FP64 levels with N >= 32 add one tile-line pass to each of the four tile
-# kernels.
+# Kernel launches of one A + B + B^T + diag step: A 2 (tile, interface), B 2 and B^T 2
+# (with the pressure transfer inside, and the interface), diag 3 (tile, boundary layers or tile
+# lines, interface); FP64 levels with N >= 32 add the tile-line pass of A.
 def launches_per_step(level):
-    return 12 + (4 if level >= 5 else 0)
+    return 9 + (1 if level >= 5 else 0)
 # FP64 peak derived from unit counts and clocks: 152 SMs x 2 DFMA / clk x 2 flops x 2.07 GHz;
 # the roofline uses the DFMA rate measured live by tn_probe_fma_peak, this figure is context.
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12

@@ -3,8 +3,8 @@
 // interpolation and B^T the interpolation followed by the element gradient; both run here in one kernel over
 // coarse cell layers (two fine cell layers at a time), with no fine-level intermediate in memory.
 //
-// Measured (B + B^T with their interface passes): level 7 / 129 layers FP64 3.76 -> 1.96 ms, 6 / 65 FP32 185 -> 103 us,
-// 5 / 101 FP64 278 -> 170 us.
+// Measured (B + B^T with their interface passes): level 7 / 129 layers FP64 3.76 -> 1.95 ms, 6 / 65 FP32 186 -> 93 us,
+// 5 / 101 FP64 278 -> 157 us.
 //
 // Compute type C: float, double, or double-float on FP64 levels with N >= 32 (unnormalised running sums, see
 // acc2 in dfloat.cuh).  All arithmetic is on pairs of C: Pr<C>.
