@@ -939,32 +939,27 @@ __device__ __forceinline__ void epilogue(const EpiArgs<T>& E, const T* in0, cons
     for (int c = 0; c < 3; ++c) E.r[c][idx] = E.b[c][idx] - y[c];
     return;
   }
-  T rr[3];
-  if (EPI == EPI_CHEB1) {
+  // every operand first: a store between the loads would hold back the ones after it (the arrays may be the same)
+  const T* const in[3] = {in0, in1, in2};
+  T rr[3], u[3], xa[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) rr[c] = E.b[c][idx] - y[c];
-  } else {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) rr[c] = E.r[c][idx] - y[c];
+  for (int c = 0; c < 3; ++c) {
+    rr[c] = EPI == EPI_CHEB1 ? E.b[c][idx] : E.r[c][idx];
+    u[c] = in[c][idx];
+    xa[c] = EPI == EPI_CHEB1 ? u[c] : E.xacc[c][idx];
   }
   const T a = E.binv[0][idx], e = E.binv[1][idx], f = E.binv[2][idx], xy = E.binv[3][idx], xz = E.binv[4][idx],
           yz = E.binv[5][idx];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) rr[c] -= y[c];
   const T z[3] = {a * rr[0] + xy * rr[1] + xz * rr[2], xy * rr[0] + e * rr[1] + yz * rr[2],
                   xz * rr[0] + yz * rr[1] + f * rr[2]};
-  const T* in[3] = {in0, in1, in2};
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    T dd, xn;
-    if (EPI == EPI_CHEB1) {
-      dd = (T)E.c0 * z[c];
-      xn = in[c][idx] + dd;
-    } else {
-      dd = (T)E.c1 * in[c][idx] + (T)E.c2 * z[c];
-      xn = E.xacc[c][idx] + dd;
-    }
+    const T dd = EPI == EPI_CHEB1 ? (T)E.c0 * z[c] : (T)E.c1 * u[c] + (T)E.c2 * z[c];
     E.r[c][idx] = rr[c];
     E.dout[c][idx] = dd;
-    E.xout[c][idx] = xn;
+    E.xout[c][idx] = xa[c] + dd;
   }
 }
 
