@@ -517,8 +517,9 @@ __global__ void __launch_bounds__(128)
     const int o = (int)(p.d * D.diamond_stride) + k * (int)D.layer_stride + p.i * D.P + p.j;
     const bool surface = k == 0 || k == n_r - 1;
     float v[3] = {0.f, 0.f, 0.f}, w[3] = {0.f, 0.f, 0.f};
+    EpiOps<float, EPI> ops;
     if (p.cnt) {
-      epi_prefetch<float, EPI>(E, o);
+      ops.load(E, in0, in1, in2, o);
       ring4_sum(RD, N, n_r, ring, k, p.d, p.i, p.j, v);
       if (surface) w[0] = in0[o], w[1] = in1[o], w[2] = in2[o];
     }
@@ -535,7 +536,7 @@ __global__ void __launch_bounds__(128)
       }
     }
     if (EPI != EPI_NONE) {
-      epilogue<float, EPI>(E, in0, in1, in2, o, v);
+      ops.apply(E, o, v);
     } else {
       out0[o] = v[0], out1[o] = v[1], out2[o] = v[2];
     }
@@ -555,7 +556,8 @@ __global__ void __launch_bounds__(128)
   if (i == 0 || i == N || j == 0 || j == N) return;  // diamond edge
   float v[3] = {0.f, 0.f, 0.f};
   const int idx = (int)(d * D.diamond_stride) + k * (int)D.layer_stride + i * D.P + j;
-  epi_prefetch<float, EPI>(E, idx);
+  EpiOps<float, EPI> ops;
+  ops.load(E, in0, in1, in2, idx);
   ring4_sum(RD, N, n_r, ring, k, d, i, j, v);
   const int M = N + 1;
   const int64_t so = ((int64_t)d * M + i) * D.P + j;
@@ -570,7 +572,7 @@ __global__ void __launch_bounds__(128)
     }
   }
   if (EPI != EPI_NONE) {
-    epilogue<float, EPI>(E, in0, in1, in2, idx, v);
+    ops.apply(E, idx, v);
     return;
   }
   out0[idx] = v[0], out1[idx] = v[1], out2[idx] = v[2];

@@ -318,12 +318,13 @@ __global__ void __launch_bounds__(128) k_small_node(SmallDims S, SmallTab<T> B, 
   const Point p = point_at(S.pts, u);
   const T* const in[3] = {in0, in1, in2};
   const int o = p.d * S.ds + k * S.ls + p.i * S.P + p.j;
-  if (p.cnt) epi_prefetch<T, EPI>(E, o);
+  EpiOps<T, EPI> ops;
+  if (p.cnt) ops.load(E, in0, in1, in2, o);
   T v[3];
   small_node<T, false>(S, B, in, sc, p, u & ~31, k, o, v);
   if (!p.cnt) return;
   if (EPI != EPI_NONE) {
-    epilogue<T, EPI>(E, in0, in1, in2, o, v);
+    ops.apply(E, o, v);
   } else {
     out0[o] = v[0], out1[o] = v[1], out2[o] = v[2];
   }
