@@ -916,20 +916,6 @@ __device__ __forceinline__ void prefetch_l1(const T* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
-// L1 prefetch of the operands that the fused update of node idx will read.
-template <typename T, int EPI>
-__device__ __forceinline__ void epi_prefetch(const EpiArgs<T>& E, int idx) {
-  if (EPI == EPI_NONE) return;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    if (EPI == EPI_CHEB2) prefetch_l1(E.r[c] + idx), prefetch_l1(E.xacc[c] + idx);
-    else prefetch_l1(E.b[c] + idx);
-  }
-  if (EPI != EPI_RESID)
-#pragma unroll
-    for (int q = 0; q < 6; ++q) prefetch_l1(E.binv[q] + idx);
-}
-
 // Fused vector update at node idx from y = (K x)(idx) (see EpiArgs); `in` is the apply input.  Every operand is loaded
 // before the first store, which would hold back the loads after it (the arrays may be the same), and the gather kernels
 // load them before they sum the node: one memory latency instead of two or three.  FP32 V-cycle at level 6 / 65 layers

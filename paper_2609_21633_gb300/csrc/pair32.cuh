@@ -484,16 +484,16 @@ __device__ __forceinline__ void ring4_sum(const RingDims& RD, int N, int n_r, co
                                           int d, int i, int j, float (&v)[3]) {
   const int rid = ring_index(RD, N, i, j);
   const bool on_h = i % RD.TI == 0, on_v = j % RD.TJ == 0;
-  for (int bi = 0; bi < 2; ++bi) {
-    if (bi == 1 && !on_h) break;
-    if (on_h && ((bi == 0 && i == 0) || (bi == 1 && i == N))) continue;
-    for (int bj = 0; bj < 2; ++bj) {
-      if (bj == 1 && !on_v) break;
-      if (on_v && ((bj == 0 && j == 0) || (bj == 1 && j == N))) continue;
-      const float4 x = ring[ring4_at(RD, n_r, 2 * bi + bj, k, d, rid)];
-      v[0] += x.x, v[1] += x.y, v[2] += x.z;
-    }
+  float4 x[4];
+#pragma unroll
+  for (int slot = 0; slot < 4; ++slot) {
+    const int bi = slot >> 1, bj = slot & 1;
+    const bool has = (on_h ? !((bi == 0 && i == 0) || (bi == 1 && i == N)) : bi == 0) &&
+                     (on_v ? !((bj == 0 && j == 0) || (bj == 1 && j == N)) : bj == 0);
+    x[slot] = has ? ring[ring4_at(RD, n_r, slot, k, d, rid)] : make_float4(0.f, 0.f, 0.f, 0.f);
   }
+#pragma unroll
+  for (int slot = 0; slot < 4; ++slot) v[0] += x[slot].x, v[1] += x[slot].y, v[2] += x[slot].z;
 }
 
 // The tile-line nodes of the paired-cell tiles, one launch: the first ne blocks of a layer take the diamond edges, one
@@ -501,7 +501,8 @@ __device__ __forceinline__ void ring4_sum(const RingDims& RD, int N, int n_r, co
 // projected and (I - P) u added once, then the value, or the fused vector update, at the copy (what k_ring_fix and
 // k_interface do in two passes for the other tiles) --, the others the tile lines inside the diamonds (as k_ring_fix),
 // nrc blocks per diamond.  Both are chains of dependent loads on few nodes, so they run side by side: as two launches
-// the FP32 V-cycle at N = 64, n_r = 65 took 1897 us instead of 1874, an apply at N = 128, n_r = 129 457 instead of 449.
+// the FP32 V-cycle at N = 64, n_r = 65 took 1897 us instead of 1874, an apply at N = 128, n_r = 129 457 instead of 449.  Every
+// load a node needs is requested before the first sum (V-cycle 1788 -> 1646 us).
 template <int FLAGS, int EPI>
 __global__ void __launch_bounds__(128)
     k_ring4(Dims D, RingDims RD, int ne, int nrc, int n_edge, const int4* __restrict__ edge, int n_groups,
