@@ -9,7 +9,7 @@
 // The same two device functions carry the coarsest-level conjugate gradients (k_cg_cluster below).
 // Bound by latency (two dependent launches of a few microseconds), in FP64 by the FP64 pipes (64 cycles
 // per instruction of a warp on an SM partition).  V-cycles went from (streaming tiles filling the SMs) 1017
-// to 366 us (FP32, level 4 / 17 layers), 1404 to 647 us (FP32, two radial points, 5 / 33) and 3999 to 1521 us (FP64,
+// to 334 us (FP32, level 4 / 17 layers), 1404 to 594 us (FP32, two radial points, 5 / 33) and 3999 to 1521 us (FP64,
 // 5 / 33); a thread per group that walks its copies, instead of one per copy, left them at 703, 1072 and 2816 us.
 // Sums run in a fixed order (copies in ascending layout order; the six triangles; bottom then top
 // contributions), so results do not depend on scheduling.
