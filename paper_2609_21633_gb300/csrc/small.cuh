@@ -455,6 +455,9 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_cluster(SmallDims S, SmallTab
 
   if constexpr (ONE)
     if (gt < nn) locate(gt, one);
+  // A CTA's shared memory may be written by the others only once it runs: total() stores to all eight before its own
+  // barrier, so the cluster meets here first (one barrier per launch, behind the loads above).
+  cl.sync();
   double w[3] = {0, 0, 0}, acc[3] = {0, 0, 0};
   if (A.project) {
     each([&](Node& n) {
