@@ -3,8 +3,8 @@
 // interpolation and B^T the interpolation followed by the element gradient; both run here in one kernel over
 // coarse cell layers (two fine cell layers at a time), with no fine-level intermediate in memory.
 //
-// Measured (B + B^T with their interface passes): level 7 / 129 layers FP64 3.76 -> 1.95 ms, 6 / 65 FP32 186 -> 93 us,
-// 5 / 101 FP64 278 -> 157 us.
+// Measured (B + B^T with their interface passes): level 7 / 129 layers FP64 3.76 -> 1.93 ms, 6 / 65 FP32 186 -> 98 us,
+// 5 / 101 FP64 278 -> 162 us.
 //
 // Compute type C: float, double, or double-float on FP64 levels with N >= 32 (unnormalised running sums, see
 // acc2 in dfloat.cuh).  All arithmetic is on pairs of C: Pr<C>.
@@ -24,6 +24,16 @@ struct Pr<float> {
   static __device__ __forceinline__ V norm(V a) { return a; }
   static __device__ __forceinline__ V add_half(V s, V a) { return fma2(a, make_float2(0.5f, 0.5f), s); }
   static __device__ __forceinline__ V add_3half(V s, V a) { return fma2(a, make_float2(1.5f, 1.5f), s); }
+  // node sums of the divergence, compensated (TwoSum: s + e is the sum up to the rounding of e)
+  static __device__ __forceinline__ void acc(V& s, V& e, V x) {
+    const V t = add2(s, x), b = sub2(t, s);
+    e = add2(e, add2(sub2(s, sub2(t, b)), sub2(x, b)));
+    s = t;
+  }
+  static __device__ __forceinline__ V close(V s, V e) {  // (an infinite sum has no rounding error: e is not a number then)
+    const V t = add2(s, e);
+    return make_float2(t.x == t.x ? t.x : s.x, t.y == t.y ? t.y : s.y);
+  }
   static __device__ __forceinline__ float in(float v) { return v; }
   template <typename T>
   static __device__ __forceinline__ T out(float v) { return v; }
@@ -44,6 +54,8 @@ struct Pr<double> {
   static __device__ __forceinline__ V norm(V a) { return a; }
   static __device__ __forceinline__ V add_half(V s, V a) { return fma(a, make_double2(0.5, 0.5), s); }
   static __device__ __forceinline__ V add_3half(V s, V a) { return fma(a, make_double2(1.5, 1.5), s); }
+  static __device__ __forceinline__ void acc(V& s, V&, V x) { s = add(s, x); }
+  static __device__ __forceinline__ V close(V s, V) { return s; }
   static __device__ __forceinline__ double in(double v) { return v; }
   template <typename T>
   static __device__ __forceinline__ T out(double v) { return v; }
@@ -69,6 +81,8 @@ struct Pr<dfl> {
   static __device__ __forceinline__ V norm(const V& a) { return norm2(a); }
   static __device__ __forceinline__ V add_half(const V& s, const V& a) { return add(s, half(a)); }
   static __device__ __forceinline__ V add_3half(const V& s, const V& a) { return add(s, add(a, half(a))); }
+  static __device__ __forceinline__ void acc(V& s, V&, const V& x) { s = add(s, x); }
+  static __device__ __forceinline__ const V& close(const V& s, const V&) { return s; }
   static __device__ __forceinline__ dfl in(double v) { return split(v); }
   template <typename T>
   static __device__ __forceinline__ T out(const dfl& v) { return join(v); }
@@ -279,21 +293,28 @@ __global__ void __launch_bounds__(kGrThreads, 2)
 }
 
 // ------------------------------------------------------------------------------------ divergence
-// With Lam_t,k = sum over a of u_a,k . l_a and Mu_t,k = (sum over a of u_a,k) . m2 on node layer k, wedge (t, k) has
-//   v_t,k = -vol w0 |det M| / 6 (Lam_k + Lam_k+1 + r_k (Mu_k+1 - Mu_k)),
-// and the coarse pressure node (I, J, K) sums 6 psi(q_c) v: laterally 2, 1/2, 1/2 (the coarse triangle's corner
+// With Lam_t,k = sum over a of u_a,k . l_a on node layer k and Mu_t,k = (sum over a of u_a,k+1 - u_a,k) . m2, wedge (t, k)
+// has
+//   v_t,k = -vol w0 |det M| / 6 (Lam_k + Lam_k+1 + r_k Mu_k),
+// differences of nodal values before any product: r grows with the number of layers, and a rounded
+// (sum over a of u_a,k) . m2 per node layer, differenced afterwards, loses as many digits on smooth velocities
+// (error in norm over the interior nodes, sines and polynomials at level 5 / 101 layers: FP32 1.9e-7 that way,
+// 6.0e-8 this way; double-float 4.0e-14 and 9.6e-15; FP32 saddle 6 / 65 93 -> 98 us, FP64 5 / 101 158 -> 162 us).
+// The coarse pressure node (I, J, K) sums 6 psi(q_c) v: laterally 2, 1/2, 1/2 (the coarse triangle's corner
 // child at the node, the other two) and 1 (the middle child), radially 1/2, 3/2, 3/2, 1/2 over the fine cell
 // layers 2K - 2 .. 2K + 1.  A CTA owns ntile / 2 x ntile / 2 coarse nodes, one thread per fine cell of the tile
-// and of a rim of two cells at its low edges; Lam and Mu are formed once per node layer, and the lateral
+// and of a rim of two cells at its low edges; Lam is formed once per node layer and Mu once per cell layer, from a ring
+// of three node layers in shared memory (of which a coarse layer replaces two), and the lateral
 // sums run once per coarse layer: within a coarse cell first (four threads, one corner each), then over the
 // coarse cells around a node.  Bound by the FP32 pipe (double-float) or by memory.
 constexpr int kDvTile = 16, kDvThreads = 352, kDvCells = (kDvTile + 2) * (kDvTile + 2),
               kDvNodes = (kDvTile + 3) * (kDvTile + 3), kDvMaxKc = 32;
 template <typename T, typename C>
 constexpr size_t div_smem_bytes() {
-  return sizeof(typename Pr<C>::V) * (size_t)(10 * kDvThreads + 4 * kDvCells + 2 * (kDvMaxKc + 1)) +
-         (sizeof(C) + sizeof(T)) * (size_t)(2 * 3 * kDvNodes);
+  return sizeof(typename Pr<C>::V) * (size_t)(13 * kDvCells + 2 * (kDvMaxKc + 1)) +
+         (3 * sizeof(C) + 2 * sizeof(T)) * (size_t)(3 * kDvNodes);
 }
+static_assert(div_smem_bytes<double, dfl>() <= 113 * 1024, "two CTAs per SM");
 __device__ __forceinline__ void cp_async_elem(uint32_t dst, const float* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -309,12 +330,12 @@ __global__ void __launch_bounds__(kDvThreads, 2)
   using R = Pr<C>;
   using V = typename R::V;
   extern __shared__ __align__(16) unsigned char tile_smem[];
-  V* const gc = reinterpret_cast<V*>(tile_smem) + threadIdx.x;      // [10][kDvThreads] M^-1, |det M|
-  V* const tb = reinterpret_cast<V*>(tile_smem) + 10 * kDvThreads;  // [2][kDvCells] (bottom, top) of W0, W1
-  V* const cb = tb + 2 * kDvCells;                                  // [2][kDvCells] of coarse-cell corners
-  V* const lct = cb + 2 * kDvCells;                                 // [kDvMaxKc + 1][2]
-  C* const us = reinterpret_cast<C*>(lct + 2 * (kDvMaxKc + 1));     // [2][3][kDvNodes]: two node layers
-  T* const rw = reinterpret_cast<T*>(us + 2 * 3 * kDvNodes);        // [2][3][kDvNodes]: the next two, as stored
+  V* const gc = reinterpret_cast<V*>(tile_smem) + threadIdx.x;    // [10][kDvCells] M^-1, |det M|
+  V* const tb = reinterpret_cast<V*>(tile_smem) + 10 * kDvCells;  // [2][kDvCells] (bottom, top) of W0, W1
+  V* const cb = tb + 2 * kDvCells;                                // [kDvCells] of coarse-cell corners
+  V* const lct = cb + kDvCells;                                   // [kDvMaxKc + 1][2]
+  C* const us = reinterpret_cast<C*>(lct + 2 * (kDvMaxKc + 1));   // [3][3][kDvNodes]: ring of three node layers
+  T* const rw = reinterpret_cast<T*>(us + 3 * 3 * kDvNodes);      // [2][3][kDvNodes]: the next two, as stored
   const int N = F.N, n_r = F.n_r, P = F.P, LS = (int)F.layer_stride;
   const int d = blockIdx.z, nK = (n_r - 1) / 2;
   const int nt_ = N / ntile, W = ntile + 2, WN = ntile + 3;
@@ -354,20 +375,20 @@ __global__ void __launch_bounds__(kDvThreads, 2)
   auto put = [&](int k, int h, T (&v)[3], int s, int64_t so) {  // projected on the boundary layers
     if (k == 0 || k == n_r - 1) project_vec(v, svec, so, F.n_lat_layout, k == 0 ? bc_in : bc_out);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) us[(h * 3 + c) * kDvNodes + s] = R::in(v[c]);
+    for (int c = 0; c < 3; ++c) us[h + c * kDvNodes + s] = R::in(v[c]);
   };
-  auto put2 = [&](int k) {  // the requested layers k, k + 1
+  auto put2 = [&](int k, int h1, int h2) {  // the requested layers k, k + 1
     cp_async_wait<0>();
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const T* const r = rw + h * 3 * kDvNodes;
       if (cell) {
         T v[3] = {r[slot], r[kDvNodes + slot], r[2 * kDvNodes + slot]};
-        put(k + h, h, v, slot, (int64_t)lbase + ci * P + cj);
+        put(k + h, h == 0 ? h1 : h2, v, slot, (int64_t)lbase + ci * P + cj);
       }
       if (xs >= 0) {
         T v[3] = {r[xs], r[kDvNodes + xs], r[2 * kDvNodes + xs]};
-        put(k + h, h, v, xs, (int64_t)lbase + xi * P + xj);
+        put(k + h, h == 0 ? h1 : h2, v, xs, (int64_t)lbase + xi * P + xj);
       }
     }
   };
@@ -388,7 +409,7 @@ __global__ void __launch_bounds__(kDvThreads, 2)
   if (cell) {
     const int t0 = ((d * N + ci) * N + cj) * 2, nt = (int)F.n_tri;
 #pragma unroll
-    for (int g = 0; g < 10; ++g) gc[g * kDvThreads] = R::mk(R::in(geo[g * nt + t0]), R::in(geo[g * nt + t0 + 1]));
+    for (int g = 0; g < 10; ++g) gc[g * kDvCells] = R::mk(R::in(geo[g * nt + t0]), R::in(geo[g * nt + t0 + 1]));
   }
   for (int K = Kb + t; K < K1; K += kDvThreads) {  // (-vol w0 / 6, r) of the fine cell layers 2K, 2K + 1
     const C *l0 = lay + kLayerStride * (2 * K), *l1 = l0 + kLayerStride;
@@ -396,65 +417,84 @@ __global__ void __launch_bounds__(kDvThreads, 2)
   }
   const V zero = R::mk(C(0.0f), C(0.0f));
   if (in_tile && !cell) tb[t] = tb[kDvCells + t] = zero;  // cells outside the diamond
-  // Lam, Mu of this cell's wedges on the node layer in half h of us
-  auto layer = [&](int h, V& lam, V& mu) {
-    const C* const u = us + h * 3 * kDvNodes + slot;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const C u00 = u[c * kDvNodes], u10 = u[c * kDvNodes + WN], u01 = u[c * kDvNodes + 1], u11 = u[c * kDvNodes + WN + 1];
-      const V a = R::mk(u00, u11), b = R::mk(u10, u01), e = R::mk(u01, u10);
-      const V ax = R::sub(b, a), ay = R::sub(e, a), sm = R::add(R::add(b, e), a);
-      const V m0 = gc[c * kDvThreads], m1 = gc[(3 + c) * kDvThreads], m2 = gc[(6 + c) * kDvThreads];
-      lam = c == 0 ? R::mul(ax, m0) : R::fma(ax, m0, lam);
-      lam = R::fma(ay, m1, lam);
-      mu = c == 0 ? R::mul(sm, m2) : R::fma(sm, m2, mu);
-    }
+  auto corners = [&](int h, V& a, V& b) {  // u at the corners (00, 11) and (10, 01), from offset h of us
+    const C* const u = us + h;
+    a = R::mk(u[0], u[WN + 1]), b = R::mk(u[WN], u[1]);
   };
-  auto wedge = [&](const V& fr, const V& lam0, const V& mu0, const V& lam1, const V& mu1) {
-    const V f = R::mul(R::mk(R::x(fr), R::x(fr)), gc[9 * kDvThreads]);
-    return R::mul(f, R::fma(R::mk(R::y(fr), R::y(fr)), R::sub(mu1, mu0), R::add(lam0, lam1)));
+  auto lateral = [&](int c, const V& a, const V& b, V& lam) {  // + component c of Lam, a and b its corners
+    // (differences normalised: after a cancellation their low part is large, and the products drop low x low)
+    const V ax = R::norm(R::sub(b, a)), ay = R::norm(R::sub(R::mk(R::y(b), R::x(b)), a));
+    lam = c == 0 ? R::mul(ax, gc[0]) : R::fma(ax, gc[c * kDvCells], lam);
+    lam = R::fma(ay, gc[(3 + c) * kDvCells], lam);
+  };
+  auto radial = [&](int c, const V& a0, const V& b0, const V& a1, const V& b1, V& mu) {  // + component c of Mu
+    const V da = R::sub(a1, a0), db = R::sub(b1, b0);
+    const V dz = R::norm(R::add(R::add(db, R::mk(R::y(db), R::x(db))), da));
+    mu = c == 0 ? R::mul(dz, gc[6 * kDvCells]) : R::fma(dz, gc[(6 + c) * kDvCells], mu);
+  };
+  auto wedge = [&](const V& fr, const V& lam0, const V& lam1, const V& mu) {
+    const V f = R::mul(R::mk(R::x(fr), R::x(fr)), gc[9 * kDvCells]);
+    return R::mul(f, R::fma(R::mk(R::y(fr), R::y(fr)), mu, R::add(lam0, lam1)));
   };
   // coarse corner of this thread's coarse cell (four threads per coarse cell): q = 2 * (tj & 1) + (ti & 1)
   const int bt = (ti & ~1) * W + (tj & ~1);  // fine cell (2I, 2J) of the coarse cell
   const int corner = (ti & 1) + 2 * (tj & 1);
-  // coarse nodes of the tile: thread t < own count; the last tiles also own I = N / 2, J = N / 2
+  // coarse nodes of the tile, one thread each; the last tiles also own I = N / 2, J = N / 2.  FP32: by the last warps, which
+  // hold the fewest cells (repeated saddle passes at 6 / 65 94.5 -> 92.8 us); the others by the first (double-float 5 / 101 156.6 against 158 us)
   const int ho = ntile / 2, ni = ho + (i0 + 2 + ntile == N), nj = ho + (j0 + 2 + ntile == N);
-  const bool owner = t < ni * nj;
-  const int oi = t / nj, oj = t - oi * nj;  // coarse cell row / column oi + 1 of the tile has the node as corner 00
+  const int ot = t - (sizeof(C) == 4 ? kDvThreads - 96 : 0);
+  const bool owner = ot >= 0 && ot < ni * nj;
+  const int oi = ot / nj, oj = ot - oi * nj;  // coarse cell row / column oi + 1 of the tile has the node as corner 00
   const int qo = (int)(d * Cc.diamond_stride) + ((i0 + 2) / 2 + oi) * Cc.P + (j0 + 2) / 2 + oj;
-  C carry = C(0.0f);
+  // FP32 sums compensated: the values around a node cancel (wedges that share a node layer enter with opposite signs)
+  C carry = C(0.0f), ecarry = C(0.0f);
   auto finish = [&](int K) {  // coarse node layer K from the corners of coarse cell layer K (and the carried ones)
-    const V* const c = cb + (K & 1) * kDvCells;
+    const V* const c = cb;
     // coarse cells (oi + 1, oj + 1) corner 00, (oi, oj + 1) corner 10, (oi + 1, oj) corner 01, (oi, oj) corner 11 of
     // the tile, those inside it (the far edge's nodes have no cell beyond)
-    V s = zero;
+    V s = zero, e = zero;
     const int r1 = 2 * (oi + 1) * W, r0 = 2 * oi * W, c1 = 2 * (oj + 1), c0 = 2 * oj;
     if (oi < ho && oj < ho) s = c[r1 + c1];
-    if (oj < ho) s = R::add(s, c[r0 + W + c1]);
-    if (oi < ho) s = R::add(s, c[r1 + c0 + 1]);
-    s = R::add(s, c[r0 + W + c0 + 1]);
+    if (oj < ho) R::acc(s, e, c[r0 + W + c1]);
+    if (oi < ho) R::acc(s, e, c[r1 + c0 + 1]);
+    R::acc(s, e, c[r0 + W + c0 + 1]);
     if (K >= K0) {
-      const V z = R::add(R::mk(R::x(s), R::x(s)), R::mk(carry, carry));
-      q[qo + K * (int)Cc.layer_stride] = R::template out<T>(R::x(z));
+      V z = R::mk(R::x(s), R::x(s)), ez = R::mk(R::x(e), R::x(e));
+      R::acc(z, ez, R::mk(carry, carry));
+      ez = R::add(ez, R::mk(ecarry, ecarry));
+      q[qo + K * (int)Cc.layer_stride] = R::template out<T>(R::x(R::close(z, ez)));
     }
-    carry = R::y(s);
+    carry = R::y(s), ecarry = R::y(e);
   };
-  V lam = zero, mu = zero;
+  V lam = zero;
+  int h0 = 0, h1 = 3 * kDvNodes, h2 = 2 * 3 * kDvNodes;  // node layers 2K, 2K + 1, 2K + 2 in us
   __syncthreads();
-  if (cell) layer(0, lam, mu);
-  __syncthreads();  // us is rewritten next
+  if (cell)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      V a, b;
+      corners(h0 + c * kDvNodes + slot, a, b);
+      lateral(c, a, b, lam);
+    }
   for (int K = Kb; K < K1; ++K) {
-    put2(2 * K + 1);
+    // (h1, h2 held the layers 2K - 2 and 2K - 1, last read before the previous barrier)
+    put2(2 * K + 1, h1, h2);
     if (K + 1 < K1) request(2 * K + 3);
     __syncthreads();
     if (K > Kb && owner) finish(K - 1);
     if (cell) {
-      V l1, m1, l2, m2;
-      layer(0, l1, m1);
-      const V v0 = wedge(lct[2 * (K - Kb)], lam, mu, l1, m1);
-      layer(1, l2, m2);
-      const V v1 = wedge(lct[2 * (K - Kb) + 1], l1, m1, l2, m2);
-      lam = l2, mu = m2;
+      V l1, l2, m1, m2;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        V a0, b0, a1, b1;
+        corners(h0 + c * kDvNodes + slot, a0, b0), corners(h1 + c * kDvNodes + slot, a1, b1);
+        radial(c, a0, b0, a1, b1, m1);
+        corners(h2 + c * kDvNodes + slot, a0, b0);
+        radial(c, a1, b1, a0, b0, m2);
+        lateral(c, a1, b1, l1), lateral(c, a0, b0, l2);
+      }
+      const V v0 = wedge(lct[2 * (K - Kb)], lam, l1, m1), v1 = wedge(lct[2 * (K - Kb) + 1], l1, l2, m2);
+      lam = l2;
       const V b = R::add_3half(R::half(v1), v0), tp = R::add_3half(R::half(v0), v1);
       tb[t] = R::mk(R::x(b), R::x(tp)), tb[kDvCells + t] = R::mk(R::y(b), R::y(tp));
     }
@@ -470,13 +510,15 @@ __global__ void __launch_bounds__(kDvThreads, 2)
         const V s = R::add_3half(R::add_half(bm, R::add(R::add(b0, b1), b2)), corner == 3 ? b0 : corner == 1 ? b2 : b1);
         r = corner == 3 ? s : R::add(r, s);
       }
-      cb[(K & 1) * kDvCells + t] = r;
+      cb[t] = r;
     }
-    // cb is read past the next barrier; its other half and tb are rewritten after that barrier, us after this one's
+    // cb is read between the next two barriers and rewritten after them, tb after the next one
+    const int h = h0;
+    h0 = h2, h2 = h1, h1 = h;
   }
   __syncthreads();
   if (owner) {
     finish(K1 - 1);
-    if (K1 == nK) q[qo + nK * (int)Cc.layer_stride] = R::template out<T>(carry);
+    if (K1 == nK) q[qo + nK * (int)Cc.layer_stride] = R::template out<T>(R::x(R::close(R::mk(carry, carry), R::mk(ecarry, ecarry))));
   }
 }
