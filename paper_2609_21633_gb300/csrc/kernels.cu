@@ -2460,7 +2460,7 @@ cudaError_t df_diag(const Level& L, BC bc, int div_term, double* const* d, cudaS
       D, dfl(hg_coef(L, div_term)), B, d[0], d[1], d[2], L.dcoefdf2, (int)(L.n_tri / 2),
       reinterpret_cast<const dfl*>(L.laydf), L.eta64, kc, L.ring64);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || layers == 0) return e;  // two node layers: both are boundary layers, no tile lines between them
   const RingDims RD = ring_dims(L.N, kDfTI, kDfTJ);
   k_ring_fix<double, 3, 0, EPI_NONE><<<dim3(nblk(RD.RC, 256), layers, 10), 256, 0, st>>>(
       D, RD, L.ring64, d[0], d[0], d[0], d[0], d[1], d[2], L.s64, bc.in, bc.out, nullptr, EpiArgs<double>{}, 1);
