@@ -405,10 +405,11 @@ tn_status tn_stokes_solve_batch(tn_mesh* const* meshes, int n, const tn_solve_op
  * surface layers keep their values (prescribed temperatures).  The paper's own schemes (SUPG,
  * entropy viscosity, MMOC, Sec. 6) are named there without their discrete forms; this is the
  * library's explicit SUPG reading.  The first energy call on a mesh allocates its workspace
- * (five layout vectors), kept until tn_mesh_destroy; the first tn_energy_steps with a velocity another 20 layout
- * vectors and four values per wedge for the assembled rows of its residual, if they take at most a quarter of
- * the free device memory (element-by-element residuals otherwise, and while the stream is being captured
- * before they exist).
+ * (five layout vectors), kept until tn_mesh_destroy; the first tn_energy_steps with a velocity that finds room for
+ * them another 20 layout vectors and four values per wedge, also kept, for the assembled rows of its residual:
+ * room means at most a quarter of the device memory free at that call.  A call that finds none, or whose stream
+ * is being captured before they exist, takes the residuals element by element: the same steps up to rounding
+ * (identical calls give identical bits only on the same one of the two paths), several times slower.
  * ---------------------------------------------------------------------------------------- */
 /* R = (K + C(u) + S(u)) T (u_dev NULL: the diffusion K T only; supg 0 drops S).  T_dev, R_dev: node
  * layout of level 0, equal values on node copies; R must not alias T.  Stream-ordered. */

@@ -204,7 +204,8 @@ cudaError_t heun_steps(tn_mesh* mesh, double* T, const double* const* u, double 
   const Dims D = dims(L);
   EnergyState& S = mesh->en;
   double *R = S.w[0], *T1 = S.w[1], *R1 = S.w[2];
-  if (n > 0 && u && rows_ready(S, L, st)) return heun_rows(S, L, T, T1, u, dt, n, supg, st);
+  if (n > 0 && u && rows_ready(S.ws, sizeof(double) * kRowCoef * (size_t)L.n_layout, sizeof(WedgeFlow) * (size_t)L.n_wedges, st))
+    return heun_rows(S, L, T, T1, u, dt, n, supg, st);
   cudaError_t e = cudaSuccess;
   for (int s = 0; s < n && e == cudaSuccess; ++s) {
     e = launch_energy_residual(L, u, T, R, supg, st);
@@ -276,7 +277,7 @@ double min_spacing(const tn_mesh* mesh) {
 void energy_free(tn_mesh* mesh) {
   EnergyState& S = mesh->en;
   for (void* p : {(void*)S.mass, (void*)S.w[0], (void*)S.w[1], (void*)S.w[2], (void*)S.w[3], (void*)S.part,
-                  (void*)S.rows, (void*)S.wq})
+                  (void*)S.ws.rows, (void*)S.ws.wq})
     if (p) cudaFree(p);
   S = EnergyState();
 }

@@ -211,49 +211,25 @@ __global__ void __launch_bounds__(256) k_energy_stage(RowDims S, const double* _
   for (int c = b; c < e; ++c) out[S.goff[c] + lo] = v;
 }
 
-// The workspace of the stencil form (rows and per-wedge values), allocated with the first call that needs it and
-// kept with the mesh; not taken (element residuals then) when it exceeds a quarter of the free memory, or
-// while the stream is being captured.
-inline bool rows_ready(EnergyState& S, const Level& L, cudaStream_t st) {
-  if (S.rows) return true;
-  if (S.rows_refused) return false;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;
-  }
-  const size_t nr = sizeof(double) * kRowCoef * (size_t)L.n_layout, nw = sizeof(WedgeFlow) * (size_t)L.n_wedges;
-  size_t fr = 0, tot = 0;
-  bool ok = cudaMemGetInfo(&fr, &tot) == cudaSuccess && nr + nw <= fr / 4;
-  ok = ok && cudaMalloc((void**)&S.rows, nr) == cudaSuccess;
-  if (ok && cudaMalloc((void**)&S.wq, nw) != cudaSuccess) {
-    cudaFree(S.rows);
-    S.rows = nullptr, ok = false;
-  }
-  cudaGetLastError();
-  S.rows_refused = !ok;
-  return ok;
-}
-
 // n Heun steps of T (in place) through the rows; T1: scratch of the node layout.
 inline cudaError_t heun_rows(EnergyState& S, const Level& L, double* T, double* T1, const double* const* u, double dt,
                              int n, int supg, cudaStream_t st) {
   const Dims D = dims(L);
   const unsigned nt = (unsigned)((2 * L.N * L.N + 127) / 128), np = (unsigned)(((L.N + 1) * (L.N + 1) + 127) / 128);
   k_energy_wedge<<<dim3(nt, (L.n_r - 1 + kWedgeLayers - 1) / kWedgeLayers, 10), 128, 0, st>>>(
-      D, L.geo64, L.lay64, u[0], u[1], u[2], supg, S.wq);
+      D, L.geo64, L.lay64, u[0], u[1], u[2], supg, S.ws.wq);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) {
     const int nk = std::max(1, std::min(kRowLayers, (int)(np * 10 * (L.n_r - 2) / (152 * 3))));
-    k_energy_rows<<<dim3(np, (L.n_r - 2 + nk - 1) / nk, 10), 128, 0, st>>>(D, nk, L.geo64, L.lay64, S.wq, S.mass, dt, L.n_layout,
-                                                                          S.rows);
+    k_energy_rows<<<dim3(np, (L.n_r - 2 + nk - 1) / nk, 10), 128, 0, st>>>(D, nk, L.geo64, L.lay64, S.ws.wq, S.mass, dt, L.n_layout,
+                                                                          S.ws.rows);
     e = cudaGetLastError();
   }
   const RowDims R = row_dims(L);
   const dim3 grid((unsigned)((R.n_lat + 255) / 256), L.n_r);
   for (int s = 0; s < n && e == cudaSuccess; ++s) {
-    k_energy_stage<1><<<grid, 256, 0, st>>>(R, T, T, S.rows, T1);
-    k_energy_stage<2><<<grid, 256, 0, st>>>(R, T1, T, S.rows, T);
+    k_energy_stage<1><<<grid, 256, 0, st>>>(R, T, T, S.ws.rows, T1);
+    k_energy_stage<2><<<grid, 256, 0, st>>>(R, T1, T, S.ws.rows, T);
     e = cudaGetLastError();
   }
   return e;

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/terra_wedge.h"
+#include "energy_workspace.h"
 
 namespace tn {
 
@@ -116,20 +117,15 @@ void mg_free(MGState*);
 }
 
 namespace tn {
-struct alignas(32) WedgeFlow {  // per-wedge velocity terms of the energy rows (energy_rows.cuh)
-  double vt, l0, l1, mu;
-};
 // Energy-equation workspace of a mesh (level 0): lumped mass, four work vectors, a reduction
 // buffer, the cached largest eigenvalue of M^-1 K (0: not computed) and the assembled rows of the Heun steps
-// with their per-wedge values (energy_rows.cuh; rows_refused: no room for them); freed by energy_free.
+// with their per-wedge values; freed by energy_free.
 struct EnergyState {
   double* mass = nullptr;
   double* w[4] = {};
   double* part = nullptr;
   double lambda = 0;
-  double* rows = nullptr;
-  WedgeFlow* wq = nullptr;
-  bool rows_refused = false;
+  RowsWorkspace ws;
 };
 }  // namespace tn
 
