@@ -35,6 +35,7 @@
 
 #include "dfloat.cuh"
 #include "internal.h"
+#include "radial_chunk.h"
 
 // The file is compiled six times: TN_PART 1 holds everything but the A-apply launchers, TN_PART 2
 // the FP64 and TN_PART 3 the FP32 A-apply launchers, TN_PART 4 and 5 those of the A apply with
@@ -81,25 +82,6 @@ inline unsigned nblk(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); 
 #define TN_PAIR32 1
 #endif
 
-// Cell layers per radial chunk of a streaming tile kernel with `columns` tile columns and `resident`
-// CTAs per SM.  A CTA sweeps its chunk plus the cell layer below it (recomputed for the carried
-// contributions) and a prologue worth about half a layer, and the GPU runs the CTAs in
-// ceil(CTAs / (152 resident)) waves, so a launch takes waves * (kc + 1.5) layer times; the chunk
-// count that minimises it is taken.  Small grids get short chunks that fill the SMs (level 4 / 17
-// layers FP64: 80 CTAs of 2 layers instead of 20 of 8), large ones a last wave that is nearly full
-// (level 7 / 129 layers: 16 layers, the best of a sweep as well).
-inline int radial_chunk(int64_t columns, int ncells, int resident, int kmax) {
-  int best = 1;
-  double cost = 1e30;
-  for (int c = 1; c <= ncells; ++c) {
-    const int kc = (ncells + c - 1) / c;
-    if (kc > kmax) continue;
-    const int64_t ctas = columns * ((ncells + kc - 1) / kc), slots = (int64_t)152 * resident;
-    const double t = (double)((ctas + slots - 1) / slots) * (kc + 1.5);
-    if (t < cost) cost = t, best = kc;
-  }
-  return best;
-}
 template <typename T>
 struct MinBlocks {
   static constexpr int value = sizeof(T) == 8 ? TN_MINB_F64 : TN_MINB_F32;
