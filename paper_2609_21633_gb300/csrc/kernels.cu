@@ -2105,8 +2105,8 @@ __global__ void k_block_inv(int64_t n, T* b0, T* b1, T* b2, T* b3, T* b4, T* b5)
 // (i/2, (j+1)/2); odd/odd -> midpoint of the coarse anti-diagonal ((i+1)/2, (j-1)/2), ((i-1)/2, (j+1)/2).
 // Semi-coarsened level pairs (lateral factor lf or radial factor rf equal to 1) keep the
 // index in that direction (weight 1).
-// Every value is the mean of two lateral parents (one twice where the position is a coarse one), then of two radial
-// ones.  ADD: f += P c (the coarse-grid correction).
+// Every value is the mean of two lateral parents (the value itself where the position is a coarse one, so that no sum
+// of equal values can overflow), then of two radial ones.  ADD: f += P c (the coarse-grid correction).
 template <typename T, int NC, bool ADD>
 __global__ void k_prolong(Dims F, Dims C, int lf, int rf, int apply_bc, const T* __restrict__ c0,
                           const T* __restrict__ c1, const T* __restrict__ c2, T* f0, T* f1, T* f2,
@@ -2124,6 +2124,7 @@ __global__ void k_prolong(Dims F, Dims C, int lf, int rf, int apply_bc, const T*
   const int64_t b0 = (int64_t)d * C.diamond_stride + (int64_t)K0 * C.layer_stride,
                 b1 = (int64_t)d * C.diamond_stride + (int64_t)K1 * C.layer_stride;
   const int o0 = I0 * C.P + J0, o1 = I1 * C.P + J1;
+  const bool mid = o0 != o1;
   const int64_t idx = (int64_t)d * F.diamond_stride + (int64_t)k * F.layer_stride + (int64_t)i * F.P + j;
   const T* cs[3] = {c0, c1, c2};
   T* fs[3] = {f0, f1, f2};
@@ -2132,7 +2133,8 @@ __global__ void k_prolong(Dims F, Dims C, int lf, int rf, int apply_bc, const T*
   for (int c = 0; c < NC; ++c) {
     const T p0 = cs[c][b0 + o0], p1 = cs[c][b0 + o1], q0 = cs[c][b1 + o0], q1 = cs[c][b1 + o1];
     if (ADD) x[c] = fs[c][idx];
-    v[c] = (T)0.5 * ((T)0.5 * (p0 + p1) + (T)0.5 * (q0 + q1));
+    const T lo = mid ? (T)0.5 * (p0 + p1) : p0, hi = mid ? (T)0.5 * (q0 + q1) : q0;
+    v[c] = K0 != K1 ? (T)0.5 * (lo + hi) : lo;
   }
   if constexpr (NC == 3) {
     if (apply_bc && (k == 0 || k == F.n_r - 1))
