@@ -196,11 +196,15 @@ template <typename T>
 cudaError_t launch_apply_A_epi(const Level& L, BC bc, int div_term, int epi, const T* const* in, const EpiArgs<T>& E,
                                T* const* t, cudaStream_t st, const int* skip = nullptr);
 // A apply of a coarse multigrid level (N <= 16) through a scratch array of the wedges' contributions
-// (small.cuh), with one of the fused updates or (EPI_NONE) to y; `scratch` holds small_scratch_entries(L)
+// (small.cuh), with one of the fused updates or (EPI_NONE) to y; `scratch` holds small_scratch_entries<T>(L)
 // values and belongs to the caller: calls that share it must not overlap.
 inline bool small_level(const Level& L) { return L.N <= 16 && L.n_layout < ((int64_t)1 << 26); }
+// Values per cell: FP64 six nodes of both wedges, FP32 the cell's eight nodes, three components each.
+template <typename T>
+constexpr int small_values() { return sizeof(T) == 8 ? 36 : 24; }
+template <typename T>
 inline int64_t small_scratch_entries(const Level& L) {
-  return small_level(L) ? (int64_t)36 * 10 * L.N * L.N * (L.n_r - 1) : 0;
+  return small_level(L) ? (int64_t)small_values<T>() * 10 * L.N * L.N * (L.n_r - 1) : 0;
 }
 template <typename T>
 cudaError_t launch_small_A(const Level& L, BC bc, int div_term, int epi, const T* const* in, const EpiArgs<T>& E,
@@ -213,7 +217,9 @@ cudaError_t launch_start_vector(const Level& L, uint64_t seed, T* const* x, cuda
 // Coarsest-level block-Jacobi CG from x = 0 in one launch (small.cuh): until (r, D^-1 r) <= tol2 (r0, D^-1 r0)
 // or maxit steps; project: rigid rotations out of b and x (ginv: inverse rotation Gram matrix).  r, z, p: work
 // vectors of the level's layout.  One cluster of eight SMs: levels whose cells those carry faster than the
-// launches of a step cost (FP64: eight FP64 pipes, 4096 cells take about 35 us).
+// launches of a step cost (FP64: eight FP64 pipes, 4096 cells take about 35 us).  FP64 levels past the line take the
+// general form, ten launches a step (V-cycle at level 3 / 27 layers, whose coarsest level has 8320 cells, 2.7 ms; at
+// 3 / 9 0.52 ms): a form between the two is open.
 template <typename T>
 struct CoarseCg {
   T *x[3], *r[3], *z[3], *p[3];

@@ -94,14 +94,14 @@ struct Shape {
 // workspaces), estimated from the finest node layout.  Per layout entry and component: FP64
 // solves hold 63 Krylov and about 30 multigrid / work vectors in FP64; mixed solves hold them in
 // FP32 plus 4 FP64 work vectors.  The coarser levels add about 1/7; geometry, viscosity and
-// masks about 40 bytes.  The coarse levels' apply (N <= 16) adds 36 values per cell of its largest level.
+// masks about 40 bytes.  The coarse levels' apply (N <= 16) adds small_values per cell of its largest level.
 size_t footprint(const Shape& s, int mode) {
   const int N = 1 << s.l;
   const size_t P = (size_t)(N + 4) / 4 * 4;
   const size_t n0 = (size_t)10 * s.nr * (N + 1) * P;
   const double per = mode == TN_SOLVE_MIXED ? 3.0 * (93.0 * 4.0 + 4.0 * 8.0) : 3.0 * 93.0 * 8.0;
   const double cells = 10.0 * std::min(N, 16) * std::min(N, 16) * (s.nr - 1);
-  const double sc = 36.0 * cells * (mode == TN_SOLVE_MIXED ? 4.0 : 8.0);
+  const double sc = cells * (mode == TN_SOLVE_MIXED ? 4.0 * small_values<float>() : 8.0 * small_values<double>());
   return (size_t)((double)n0 * (per * 8.0 / 7.0 + 40.0) + sc) + ((size_t)64 << 20);
 }
 

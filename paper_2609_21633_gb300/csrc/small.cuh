@@ -50,6 +50,8 @@ inline SmallTab<T> small_tab(const Level& L, BC bc) {
 // 381 to 388 against 366 us).
 template <typename T>
 constexpr bool kSmallWedges = sizeof(T) == 8;
+static_assert(small_values<double>() == (kSmallWedges<double> ? 36 : 24), "scratch of a cell");
+static_assert(small_values<float>() == (kSmallWedges<float> ? 36 : 24), "scratch of a cell");
 
 // FP64: contributions of the wedges to their six nodes, thread per wedge and component: three neighbouring lanes share a
 // wedge, ten wedges a warp (two lanes idle).  A lane forms its component's row of the strain, exchanges the transposed

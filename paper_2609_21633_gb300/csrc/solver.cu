@@ -798,8 +798,8 @@ void run_vcycle(MGState* m, const tn_mesh* mesh, cudaStream_t st) {
   else vcycle_level<T>(m, mesh, 0, st);
 }
 
-// Capture the V-cycle into a graph (kernel parameters such as the Chebyshev coefficients are
-// fixed at capture, so this runs at the end of every set-up).
+// Capture the V-cycle into a graph.  Kernel parameters such as the Chebyshev coefficients are fixed at capture, so
+// every set-up captures anew: after the eigenvalue estimates, and before the deflation, whose V-cycles replay the graph.
 template <typename T>
 void capture_vcycle(MGState* m, const tn_mesh* mesh) {
   PrecState<T>& P = ps<T>(m);
@@ -842,7 +842,7 @@ tn_status mg_setup_t(tn_mesh* mesh, const void* const* v0, cudaStream_t st) {
       if (h == m->nlev - 1) G.p = alloc3<T>(m, n);
     }
     int64_t cells = 0;
-    for (int h = 0; h < m->nlev; ++h) cells = std::max(cells, small_scratch_entries(*m->geo[h]));
+    for (int h = 0; h < m->nlev; ++h) cells = std::max(cells, small_scratch_entries<T>(*m->geo[h]));
     if (cells > 0) P.cells = alloc_zero<T>(m, cells);
     P.mdiag = alloc_zero<T>(m, mesh->lv[1].n_layout);
     P.ones_p = alloc_zero<T>(m, mesh->lv[1].n_layout);
