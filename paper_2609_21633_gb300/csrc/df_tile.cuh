@@ -18,10 +18,10 @@
 //     neighbour's contributions arrive by warp shuffle, the column's geometry stays in shared memory, so
 //     that nothing spills (registers are the limit of the packed arithmetic: each value takes four).
 
-// Measured (A apply, tile-line pass and interface included): level 7 / 129 layers 4.00 -> 2.13 ms, 6 / 65 0.51 ->
+// Measured (A apply, tile-line pass and interface included): level 7 / 129 layers 4.00 -> 2.17 ms, 6 / 65 0.51 ->
 // 0.33 ms, with hourglass control 6 / 65 1.25 -> 0.46 ms; FMA pipes 55 % busy (43 % before, on 1.7 times the
-// operations), the rest math-pipe throttle, dependent-issue waits and the barrier.  Error against binary64: 8e-15 in
-// norm (3.5e-14 before), most of it from the 48-bit rounding of inputs and tables.
+// operations), the rest math-pipe throttle, dependent-issue waits and the barrier.  Error against binary64: 5.5e-15 in
+// norm on random fields (3.5e-14 before), most of it from the 48-bit rounding of inputs and tables.
 
 constexpr int kDfTI = 16, kDfTJ = 16, kDfThreads = kDfTI * kDfTJ;
 constexpr int kDfNodes = (kDfTI + 1) * (kDfTJ + 1);
